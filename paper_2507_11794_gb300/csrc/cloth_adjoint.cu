@@ -260,9 +260,11 @@ __global__ void copy_planes_kernel(const float4 *__restrict__ src, float4 *__res
 __global__ void segment_begin_kernel(DevCtrl *ctrl, unsigned long long k, uint32_t *bits, long long nwords)
 {
     const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i0 == 0) ctrl->k = k;
+    if (i0 == 0) ctrl_set_k(ctrl, k);
     for (long long i = i0; i < nwords; i += (long long)gridDim.x * blockDim.x) bits[i] = 0u;
 }
+
+__global__ void set_k_kernel(DevCtrl *ctrl, unsigned long long k) { ctrl_set_k(ctrl, k); }
 
 // Canonical spring order <-> [direction][r*pitch + c] slots.
 __global__ void scatter_kernel(const float *__restrict__ canon, const int *__restrict__ map, int S,
@@ -310,7 +312,7 @@ struct ClothRollout {
     ClothHandle *h = nullptr;
     int nsteps = 0, every = 0, nseg = 0, S = 0;
     unsigned long long k0 = 0, k_final = 0;
-    std::vector<unsigned long long> kseg;  // substep counter at each checkpoint (host copies for async uploads)
+    std::vector<unsigned long long> kseg;  // substep counter at each checkpoint
     float *x0 = nullptr, *v0 = nullptr;    // initial state, AoS [N][3]
     float *ckpt = nullptr;                 // nseg x 6 planes
     float *seg = nullptr;                  // 2 sets x (every*substeps+1) slots x 19 planes (x, v, v*, response data)
@@ -685,9 +687,8 @@ int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd
     if (d_ks && ro->S > 0) scatter_kernel<<<nblk(ro->S, 256), 256, 0, s>>>(d_ks, ro->map, ro->S, h->ks_slot);
     if (d_kd && ro->S > 0) scatter_kernel<<<nblk(ro->S, 256), 256, 0, s>>>(d_kd, ro->map, ro->S, h->kd_slot);
     RTRY(h, cudaGetLastError(), "constants scatter");
-    ro->kseg[0] = ro->k0;
-    RTRY(h, cudaMemcpyAsync(&h->ctrl->k, &ro->kseg[0], sizeof(unsigned long long), cudaMemcpyHostToDevice, s),
-         "set substep counter");
+    set_k_kernel<<<1, 1, 0, s>>>(h->ctrl, ro->k0);
+    RTRY(h, cudaGetLastError(), "set substep counter");
     RTRY(h, launch_aos_to_soa(ro->x0, d_v0 ? d_v0 : ro->v0, h->state, h->state + 6 * st, st, h->n, h->desc.nx,
                               h->pitch, h->ctrl, s),
          "initial state");
@@ -724,8 +725,8 @@ int cloth_rollout_backward(ClothRollout *ro, const float *d_gpos, const float *d
         gather_kernel<<<nblk(ro->S, 256), 256, 0, s>>>(ro->gslot + 6 * st, ro->map, ro->S, d_gkd);
     RTRY(h, cudaGetLastError(), "gradient outputs");
     // leave the cloth in its final forward state
-    RTRY(h, cudaMemcpyAsync(&h->ctrl->k, &ro->k_final, sizeof(unsigned long long), cudaMemcpyHostToDevice, s),
-         "set substep counter");
+    set_k_kernel<<<1, 1, 0, s>>>(h->ctrl, ro->k_final);
+    RTRY(h, cudaGetLastError(), "set substep counter");
     RTRY(h, copy_planes(ro->final_state, cur_state(h, ro->k_final), 6 * st, s), "restore final state");
     return CLOTH_OK;
 }

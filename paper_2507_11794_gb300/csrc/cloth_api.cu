@@ -169,6 +169,8 @@ void cloth_fill_params(ClothHandle *h)
     p.cell_start = h->grid.cell_start;
     p.tri_ids = h->grid.tri_ids;
     p.etri = h->grid.etri;
+    p.efil = h->grid.efil;
+    p.qs = h->grid.qs;
     for (int a = 0; a < 3; a++) {
         p.go[a] = h->grid.origin[a];
         p.gd[a] = h->grid.dims[a];
@@ -196,8 +198,9 @@ void cloth_fill_params(ClothHandle *h)
     p.edge_stamp = h->edge_stamp;
     p.edge_more = h->edge_more;
     p.coll_list = h->coll_list;
-    p.coll_count = h->ctrl ? &h->ctrl->coll_count : nullptr;
-    p.coll_blocks = h->sm_count * CLOTH_COLL_CTAS_PER_SM;
+    p.coll_count = h->ctrl ? h->ctrl->coll_count : nullptr;
+    p.coll_blocks = coll_ctas(h->n, h->sm_count);
+    p.coll_short = coll_short(h->n, h->sm_count);
 }
 
 namespace {
@@ -492,6 +495,9 @@ int cloth_set_mesh(ClothHandle *h, const float *verts, int32_t nverts, const int
         }
         if (e != cudaSuccess) return cuda_fail(h, e, "grid build");
     }
+    // substeps without a mesh advance k and leave the listing counts: both start
+    // again at zero
+    CTRY(h, cudaMemsetAsync(h->ctrl->coll_count, 0, sizeof(h->ctrl->coll_count), h->stream), "clear listing counts");
     grid_free(&h->grid);
     h->grid = g;
     h->has_mesh = ntris > 0;

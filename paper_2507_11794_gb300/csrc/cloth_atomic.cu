@@ -160,14 +160,17 @@ __global__ void __launch_bounds__(NODE_THREADS) node_integrate_kernel(const __gr
             const unsigned m = __ballot_sync(FULL, need);
             if (m) {
                 unsigned w0 = 0;
-                if (lane == 0) w0 = atomicAdd(p.coll_count, (unsigned)__popc(m));
+                if (lane == 0) w0 = atomicAdd(p.coll_count + (k & 1ull), (unsigned)__popc(m));
                 w0 = __shfl_sync(FULL, w0, 0);
                 if (need) p.coll_list[w0 + __popc(m & ((1u << lane) - 1u))] = (int)o;
             }
         }
     }
     if (__any_sync(FULL, !isfinite(fsum)) && lane == 0) atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
-    if (MESH) return;  // the collision kernel finishes the substep
+    if (MESH) {  // the collision kernel finishes the substep
+        if (blockIdx.x == 0 && threadIdx.x == 0) p.ctrl->kc = k;
+        return;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned prev = atomicAdd(&p.ctrl->blocks_done, 1u);

@@ -86,7 +86,7 @@ cudaError_t rebuild(ClothBatch *b)
         p.ctrl = b->ctrl;
         p.coll_list = b->coll_list;
         p.coll_cloth = b->coll_cloth;
-        p.coll_count = &b->ctrl->coll_count;
+        p.coll_count = b->ctrl->coll_count;
         prm[i] = p;
         for (int sy = 0; sy < p.strips_y; sy++)
             for (int sx = 0; sx < p.strips_x; sx++) {
@@ -116,7 +116,7 @@ cudaError_t rebuild(ClothBatch *b)
     b->args.ctrl = b->ctrl;
     b->args.coll_list = b->coll_list;
     b->args.coll_cloth = b->coll_cloth;
-    b->args.coll_count = &b->ctrl->coll_count;
+    b->args.coll_count = b->ctrl->coll_count;
     b->args.walk_blocks = b->sm_count * b->ctas_per_sm;
     b->args.coll_blocks = b->sm_count * CLOTH_COLL_CTAS_PER_SM;
     // one walk variant for the whole batch when every cloth has the same one

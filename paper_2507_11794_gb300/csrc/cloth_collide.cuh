@@ -39,11 +39,11 @@ __device__ __forceinline__ CollBox coll_box(const StepParams &p, float sx, float
 
 // One candidate: grid entry e met in cell (cx, cy, cz) of a box whose low
 // corner is (lox, loy, loz).  Returns true on a hit, with th the distance
-// along r and f = 1/a (a = e1 . (r x e2)); A, B, C receive the triangle
-// record (v0, e1, e2).
+// along r, over = th - delta (of the rounded th, whichever lane adds it up) and
+// f = 1/a (a = e1 . (r x e2)); A, B, C receive the triangle record (v0, e1, e2).
 __device__ __forceinline__ bool coll_candidate(const StepParams &p, const CollPath &q, long long e, int cx, int cy,
-                                               int cz, int lox, int loy, int loz, float &th, float &f, float4 &A,
-                                               float4 &B, float4 &C)
+                                               int cz, int lox, int loy, int loz, float &th, float &over, float &f,
+                                               float4 &A, float4 &B, float4 &C)
 {
     A = __ldg(p.etri + 3 * e);
     B = __ldg(p.etri + 3 * e + 1);
@@ -66,7 +66,9 @@ __device__ __forceinline__ bool coll_candidate(const StepParams &p, const CollPa
     const float qy = qz0 * B.x - qx0 * B.z;
     const float qz = qx0 * B.y - qy0 * B.x;
     const float v = f * (q.rx * qx + q.ry * qy + q.rz * qz);
-    th = f * (C.x * qx + C.y * qy + C.z * qz);
+    const float e2q = C.x * qx + C.y * qy + C.z * qz;
+    th = __fmul_rn(f, e2q);
+    over = __fsub_rn(th, p.delta);
     if (v < 0.0f || u + v > 1.0f) return false;
     return th > p.tmin && th < q.L;
 }
@@ -90,93 +92,79 @@ __device__ __forceinline__ bool coll_path(const StepParams &p, float sx, float s
     return true;
 }
 
-// Broad + narrow phase and response of one node, one thread walking all
-// candidates in (z, y, x) cell order and entry order.  On K > 0 hits returns
-// true and the response position.  GRAD also returns, for the adjoint's
-// recompute of an over-long path, mK = (m, K, r) with
-// m = mean max(t_k - delta, 0), and over the active hits (t_k > delta) the
-// sums g1 = sum n/a and g2 = sum t n/a (n = e1 x e2), the derivatives of t_k
-// w.r.t. S and r.  The cooperative kernel below sums the same hits in the
-// same order, so both see the same response.
-template <bool GRAD>
-__device__ __forceinline__ bool collide_t(const StepParams &p, float sx, float sy, float sz, float ex, float ey,
-                                          float ez, float &ox, float &oy, float &oz, float *g1 = nullptr,
-                                          float *g2 = nullptr, float *mK = nullptr)
+// Candidate filter: every grid entry carries its triangle's box in 16-bit
+// units of 1 / grid_filter_sub of a cell (grown by p.qpad units), laid out so
+// that three subtractions compare it with a path's box on all six sides: word
+// lanes of 15 bits under a guard bit, T = (hx, hy) (hz, M - lx) (M - ly,
+// M - lz) for the triangle and N = (lo x, lo y) (lo z, M - hi x) (...) for the
+// path, M = 32767; the boxes overlap iff every lane of T is >= that of N, i.e.
+// iff no guard bit is borrowed from.  A path can only hit a triangle whose
+// box it overlaps, so the test below it runs on the entries that pass.
+struct CollWords {
+    unsigned a, b, c;
+};
+
+__device__ __forceinline__ CollWords coll_words(const StepParams &p, float sx, float sy, float sz, float ex, float ey,
+                                                float ez, const CollPath &q)
 {
-    CollPath q;
-    if (!coll_path(p, sx, sy, sz, ex, ey, ez, q)) return false;
-    const CollBox bx = coll_box(p, sx, sy, sz, ex, ey, ez);
-    int K = 0;
-    float acc = 0.0f;
-    for (int cz = bx.loz; cz <= bx.hiz; cz++)
-        for (int cy = bx.loy; cy <= bx.hiy; cy++)
-            for (int cx = bx.lox; cx <= bx.hix; cx++) {
-                const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
-                const int e0 = __ldg(p.cell_start + cell), e1 = __ldg(p.cell_start + cell + 1);
-#pragma unroll 2
-                for (int e = e0; e < e1; e++) {
-                    float th, f;
-                    float4 A, B, C;
-                    if (!coll_candidate(p, q, e, cx, cy, cz, bx.lox, bx.loy, bx.loz, th, f, A, B, C)) continue;
-                    K++;
-                    acc += fmaxf(th - p.delta, 0.0f);
-                    if (GRAD && th - p.delta > 0.0f) {
-                        const float nx = B.y * C.z - B.z * C.y, ny = B.z * C.x - B.x * C.z, nz = B.x * C.y - B.y * C.x;
-                        g1[0] += nx * f; g1[1] += ny * f; g1[2] += nz * f;
-                        g2[0] += th * nx * f; g2[1] += th * ny * f; g2[2] += th * nz * f;
-                    }
-                }
-            }
-    if (K == 0) return false;
-    const float m = acc / (float)K;
-    if (GRAD) {
-        mK[0] = m;
-        mK[1] = (float)K;
-        mK[2] = q.rx; mK[3] = q.ry; mK[4] = q.rz;
+    if (p.tmin < 0.0f) {  // hits behind the start count: the box reaches back to S + tmin r
+        sx = fmaf(p.tmin, q.rx, sx);
+        sy = fmaf(p.tmin, q.ry, sy);
+        sz = fmaf(p.tmin, q.rz, sz);
     }
-    ox = sx + m * q.rx;
-    oy = sy + m * q.ry;
-    oz = sz + m * q.rz;
-    return true;
+    const unsigned lx = grid_filter_coord(fminf(sx, ex), p.go[0], p.qs), hx = grid_filter_coord(fmaxf(sx, ex), p.go[0], p.qs);
+    const unsigned ly = grid_filter_coord(fminf(sy, ey), p.go[1], p.qs), hy = grid_filter_coord(fmaxf(sy, ey), p.go[1], p.qs);
+    const unsigned lz = grid_filter_coord(fminf(sz, ez), p.go[2], p.qs), hz = grid_filter_coord(fmaxf(sz, ez), p.go[2], p.qs);
+    return {lx | ly << 16, lz | (GRID_FILTER_MAX - hx) << 16, (GRID_FILTER_MAX - hy) | (GRID_FILTER_MAX - hz) << 16};
+}
+__device__ __forceinline__ bool coll_overlap(const uint4 &t, const CollWords &n)
+{
+    return (((t.x - n.a) & (t.y - n.b) & (t.z - n.c)) & GRID_FILTER_GUARD) == GRID_FILTER_GUARD;
 }
 
-// ------------------------------------------------- cooperative list pass
-// The walk appends the nodes whose path box meets the box of the mesh's vertices.
-// Most of them find empty cells; the few next to the surface find about a
-// dozen candidates each, and those sit next to one another in the list.  One
-// thread per node would leave those few threads testing their candidates one
-// after another while the rest of the GPU idles, so each warp instead:
-//  1. takes 32 list entries dealt round robin over all warps (entry i to warp
-//     i mod #warps, spreading a run of neighbouring nodes over many warps),
-//     boxes each path and counts its candidates over the box's cells;
-//  2. spreads the warp's candidates over its 32 lanes, one test per lane and
-//     round; each owner lane then adds its hits in candidate order (the
-//     order collide_t uses, so the sum is the same float sum);
-//  3. owner lanes apply the response.
-// A path whose box spans more than COLL_MAXC cells (a node moving further
-// than a cell in one substep) is handled by its own lane with collide_t.
+// Running sums of one node's hits: K and sum max(t - delta, 0) and, for the
+// adjoint's recompute (REC), over the active hits (t > delta) g1 = sum n/a
+// and g2 = sum t n/a (n = e1 x e2), the derivatives of t w.r.t. S and r.
+template <bool REC>
+struct CollAcc {
+    int K;
+    float acc, g1[REC ? 3 : 1], g2[REC ? 3 : 1];
+};
+template <bool REC>
+__device__ __forceinline__ void coll_add(CollAcc<REC> &s, float val, float th, float f, const float4 &B,
+                                         const float4 &C)
+{
+    s.K++;
+    s.acc += val;
+    if constexpr (REC) {
+        if (val > 0.0f) {
+            const float nx = B.y * C.z - B.z * C.y, ny = B.z * C.x - B.x * C.z, nz = B.x * C.y - B.y * C.x;
+            // products rounded before they are added, in either walk below
+            s.g1[0] = __fadd_rn(s.g1[0], __fmul_rn(nx, f));
+            s.g1[1] = __fadd_rn(s.g1[1], __fmul_rn(ny, f));
+            s.g1[2] = __fadd_rn(s.g1[2], __fmul_rn(nz, f));
+            s.g2[0] = __fadd_rn(s.g2[0], __fmul_rn(__fmul_rn(th, nx), f));
+            s.g2[1] = __fadd_rn(s.g2[1], __fmul_rn(__fmul_rn(th, ny), f));
+            s.g2[2] = __fadd_rn(s.g2[2], __fmul_rn(__fmul_rn(th, nz), f));
+        }
+    }
+}
+
+// ------------------------------------------------------------ list pass
+// The walk appends the nodes whose path box meets the box of the mesh's
+// vertices.  A lane (or a group of lanes, see collide_list) per listed node: it
+// boxes the path and goes through its cells (mostly one) in x, y, z order.
+// Per cell it first runs the filter over up to 32 entries and keeps the
+// survivors as a bit mask (16 B and a handful of instructions per entry,
+// neighbouring lanes reading the same lines), then tests the survivors (a few
+// per node near the surface, 48 B and the full test each), all lanes of the
+// warp together.  Hits are added in candidate order,
+// so the sum does not depend on how the work is spread.  What is long is
+// walked by the whole warp: a path of more than COLL_MAXC cells, and a cell
+// of more than COLL_MAXE entries, 32 candidates at a time.
 constexpr int COLL_WARPS = 8;  // warps per CTA of the collision kernels
-constexpr int COLL_MAXC = 8;   // cells of a box spread over the warp
-
-struct CollLane {
-    float4 s;                   // S, L
-    float4 r;                   // r, owning cloth (int bits)
-    int4 box;                   // low cell, x extent | y extent << 16
-    int2 cell[COLL_MAXC];       // per cell of the box: first entry, end of the lane's running count
-};
-
-// Per-warp scratch of the cooperative pass, for a CTA of W warps.
-template <int W>
-struct CollSharedT {
-    CollLane lane[W][32];
-    int base[W][32];    // first candidate index of each lane (warp exclusive scan)
-    float val[W][32];   // one round's results: max(t - delta, 0) on a hit, else -1
-};
-using CollShared = CollSharedT<COLL_WARPS>;
-// The recording variant adds each candidate's terms of g1 and g2.
-struct CollSharedRec : CollShared {
-    float g[COLL_WARPS][6][32];
-};
+constexpr int COLL_MAXC = 8;   // cells of a box one lane goes through
+constexpr int COLL_MAXE = 96;  // entries of a cell one lane goes through
 
 // Records the response data of a hit node at plane offset o for the reverse
 // pass: m, r, g1 / K, g2 / K (the factors it multiplies by the adjoints) and
@@ -200,58 +188,57 @@ __device__ __forceinline__ void coll_record(const StepParams &p, long long o, fl
     atomicOr(p.cbits + (o >> 5), 1u << (o & 31));
 }
 
-// Src supplies per list entry i: entry(i, cloth, offset) and params(cloth).
-// REC (with CollSharedRec): also sums, over the active hits in the same
-// order, g1 and g2 as collide_t<true> does and records them (coll_record).
-// One round of the cooperative pass: every lane of the warp brings one entry
-// (valid: whether it has one; i: its index for src.entry).  ntest (lane 0)
-// accumulates the candidate triangles the warp tested, nhit (every lane) the
-// nodes that hit.
-// With has_pre the entry's offset is pre_o, loaded by the caller (cloth 0).
-template <bool REC, class Src, class Sh>
-__device__ __forceinline__ void collide_batch(const Src &src, Sh &sh, unsigned long long k, bool valid,
-                                              unsigned long long i, float &fsum, unsigned &ntest, unsigned &nhit,
-                                              bool has_pre = false, long long pre_o = 0)
+__device__ __forceinline__ float coll_shfl(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+// 32 candidates of one path tested by the warp, one per lane (have: whether
+// the lane has one, entry e of cell (cx, cy, cz)); the hits are added to s in
+// lane order.  Every lane passes the same path and ends with the same sums.
+template <bool REC>
+__device__ __forceinline__ void coll_warp_round(const StepParams &p, const CollPath &q, const CollWords &w,
+                                                const CollBox &bx, bool have, long long e, int cx, int cy, int cz,
+                                                CollAcc<REC> &s)
 {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    CollLane &me = sh.lane[wib][lane];
-    {
-        int cnt = 0, cloth = 0;
-        bool serial = false;
-        long long o = 0;
-        float sx = 0.0f, sy = 0.0f, sz = 0.0f, ex = 0.0f, ey = 0.0f, ez = 0.0f;
-        CollPath q;
-        float *out = nullptr;
-        long long st = 0;
-        if (valid) {
-            if (has_pre) o = pre_o;
-            else src.entry(i, cloth, o);
-            const StepParams &p = src.params(cloth);
-            st = p.stride;
-            const float *in = (k & 1ull) ? p.state1 : p.state0;
-            out = (k & 1ull) ? p.state0 : p.state1;
-            sx = __ldg(in + o); sy = __ldg(in + st + o); sz = __ldg(in + 2 * st + o);
-            ex = out[o]; ey = out[st + o]; ez = out[2 * st + o];
-            if (coll_path(p, sx, sy, sz, ex, ey, ez, q)) {
-                const CollBox bx = coll_box(p, sx, sy, sz, ex, ey, ez);
-                const int nxc = bx.hix - bx.lox + 1, nyc = bx.hiy - bx.loy + 1, nzc = bx.hiz - bx.loz + 1;
-                if ((long long)nxc * nyc * nzc > COLL_MAXC) {
-                    serial = true;
-                } else {
-                    int c = 0;
-                    for (int cz = bx.loz; cz <= bx.hiz; cz++)
-                        for (int cy = bx.loy; cy <= bx.hiy; cy++)
-                            for (int cx = bx.lox; cx <= bx.hix; cx++, c++) {
-                                const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
-                                const int e0 = __ldg(p.cell_start + cell), e1 = __ldg(p.cell_start + cell + 1);
-                                cnt += e1 - e0;
-                                me.cell[c] = make_int2(e0, cnt);
-                            }
-                    me.s = make_float4(q.sx, q.sy, q.sz, q.L);
-                    me.r = make_float4(q.rx, q.ry, q.rz, __int_as_float(cloth));
-                    me.box = make_int4(bx.lox, bx.loy, bx.loz, nxc | (nyc << 16));
-                }
-            }
+    float th = 0.0f, over = 0.0f, f = 0.0f;
+    float4 A, B = make_float4(0.0f, 0.0f, 0.0f, 0.0f), C = B;
+    const bool hit = have && coll_overlap(__ldg(p.efil + e), w) &&
+                     coll_candidate(p, q, e, cx, cy, cz, bx.lox, bx.loy, bx.loz, th, over, f, A, B, C);
+    const float val = fmaxf(over, 0.0f);
+    for (unsigned hm = __ballot_sync(0xffffffffu, hit); hm; hm &= hm - 1u) {
+        const int src = __ffs((int)hm) - 1;
+        const float hv = coll_shfl(val, src);
+        float ht = 0.0f, hf = 0.0f;
+        float4 hB = B, hC = C;
+        if constexpr (REC) {
+            ht = coll_shfl(th, src);
+            hf = coll_shfl(f, src);
+            hB.x = coll_shfl(B.x, src); hB.y = coll_shfl(B.y, src); hB.z = coll_shfl(B.z, src);
+            hC.x = coll_shfl(C.x, src); hC.y = coll_shfl(C.y, src); hC.z = coll_shfl(C.z, src);
+        }
+        coll_add<REC>(s, hv, ht, hf, hB, hC);
+    }
+}
+
+// All cells of a long path walked by the whole warp (every lane passes the
+// same arguments): 32 cells at a time, x fastest, then their candidates 32 at
+// a time in cell order, so the hits come in the order of a walk by one thread.
+template <bool REC>
+__device__ __noinline__ void coll_wide(const StepParams &p, const CollPath q, const CollWords w, const CollBox bx,
+                                       CollAcc<REC> &s)
+{
+    const int lane = threadIdx.x & 31;
+    const int nxc = bx.hix - bx.lox + 1, nyc = bx.hiy - bx.loy + 1, nzc = bx.hiz - bx.loz + 1;
+    const long long nxy = (long long)nxc * nyc, ncell = nxy * nzc;
+    for (long long c0 = 0; c0 < ncell; c0 += 32) {
+        const long long cc = c0 + lane;
+        int e0 = 0, cnt = 0, cx = 0, cy = 0, cz = 0;
+        if (cc < ncell) {
+            cz = bx.loz + (int)(cc / nxy);
+            const int rem = (int)(cc - (long long)(cz - bx.loz) * nxy);
+            cy = bx.loy + rem / nxc;
+            cx = bx.lox + rem % nxc;
+            const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
+            e0 = __ldg(p.cell_start + cell);
+            cnt = __ldg(p.cell_start + cell + 1) - e0;
         }
         int incl = cnt;
 #pragma unroll
@@ -260,133 +247,232 @@ __device__ __forceinline__ void collide_batch(const Src &src, Sh &sh, unsigned l
             if (lane >= d) incl += t;
         }
         const int total = __shfl_sync(0xffffffffu, incl, 31);
-        if (lane == 0) ntest += (unsigned)total;
         const int excl = incl - cnt;
-        sh.base[wib][lane] = excl;
-        __syncwarp();
-        float acc = 0.0f;
-        int K = 0;
-        float g1[3] = {0.0f, 0.0f, 0.0f}, g2[3] = {0.0f, 0.0f, 0.0f};
         for (int r0 = 0; r0 < total; r0 += 32) {
             const int j = r0 + lane;
-            float val = -1.0f;
-            float gn[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-            if (j < total) {
-                // owner: the last lane whose first candidate is <= j (it has cnt > 0)
-                int ow = 0;
+            // the lane whose cell holds candidate j: the last with excl <= j
+            int ow = 0;
 #pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (sh.base[wib][ow + step] <= j) ow += step;
-                const CollLane &L = sh.lane[wib][ow];
-                const int loc = j - sh.base[wib][ow];
-                int c = 0;
-                while (L.cell[c].y <= loc) c++;
-                const long long e = L.cell[c].x + (loc - (c ? L.cell[c - 1].y : 0));
-                const int nxc = L.box.w & 0xffff, nyc = L.box.w >> 16;
-                const int cx = L.box.x + c % nxc, cy = L.box.y + (c / nxc) % nyc, cz = L.box.z + c / (nxc * nyc);
-                const CollPath lq = {L.s.x, L.s.y, L.s.z, L.r.x, L.r.y, L.r.z, L.s.w};
-                const StepParams &lp = src.params(__float_as_int(L.r.w));
-                float th, f;
-                float4 A, B, C;
-                if (coll_candidate(lp, lq, e, cx, cy, cz, L.box.x, L.box.y, L.box.z, th, f, A, B, C)) {
-                    val = fmaxf(th - lp.delta, 0.0f);
-                    if (REC) {
-                        // the terms collide_t<true> adds for an active hit (t - delta > 0)
-                        const float nx = B.y * C.z - B.z * C.y, ny = B.z * C.x - B.x * C.z,
-                                    nz = B.x * C.y - B.y * C.x;
-                        gn[0] = nx * f; gn[1] = ny * f; gn[2] = nz * f;
-                        gn[3] = th * nx * f; gn[4] = th * ny * f; gn[5] = th * nz * f;
-                    }
-                }
-            }
-            sh.val[wib][lane] = val;
-            if constexpr (REC) {
-                if (val > 0.0f) {
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(0xffffffffu, excl, ow + step) <= j) ow += step;
+            const int oe0 = __shfl_sync(0xffffffffu, e0, ow), oex = __shfl_sync(0xffffffffu, excl, ow);
+            const int ocx = __shfl_sync(0xffffffffu, cx, ow), ocy = __shfl_sync(0xffffffffu, cy, ow),
+                      ocz = __shfl_sync(0xffffffffu, cz, ow);
+            coll_warp_round<REC>(p, q, w, bx, j < total, (long long)oe0 + (j - oex), ocx, ocy, ocz, s);
+        }
+    }
+}
+
+// One round of the list pass, G lanes per node (the lanes of a node are
+// neighbours in the warp and end with the same sums): every group brings one
+// entry (valid: whether it has one; i: its index for src.entry).  Src supplies
+// entry(i, cloth, offset) and params(cloth).  has_pre: the entry's offset is
+// pre_o, loaded by the caller (cloth 0).  ntest and nhit accumulate, in the
+// group's first lane, the candidate triangles and whether the node hit.  REC:
+// also records the hits' response data (coll_record).
+template <bool REC, int G, class Src>
+__device__ __forceinline__ void collide_round(const Src &src, unsigned long long k, bool valid, unsigned long long i,
+                                              float &fsum, unsigned &ntest, unsigned &nhit, bool has_pre, int pre_o)
+{
+    constexpr unsigned FULLW = 0xffffffffu;
+    const int lane = threadIdx.x & 31, sub = lane % G, gbase = lane - sub;
+    int cloth = 0;
+    long long o = 0;
+    if (valid) {
+        if (has_pre) o = pre_o;
+        else src.entry(i, cloth, o);
+    }
+    const StepParams &p = src.params(cloth);
+    const long long st = p.stride;
+    const float *in = (k & 1ull) ? p.state1 : p.state0;
+    float *out = (k & 1ull) ? p.state0 : p.state1;
+    CollPath q = {};
+    CollBox bx = {0, 0, 0, 0, 0, 0};
+    CollWords w = {0u, 0u, 0u};
+    int ncell = 0;
+    bool wide = false;
+    if (valid) {
+        const float sx = __ldg(in + o), sy = __ldg(in + st + o), sz = __ldg(in + 2 * st + o);
+        const float ex = out[o], ey = out[st + o], ez = out[2 * st + o];
+        if (coll_path(p, sx, sy, sz, ex, ey, ez, q)) {
+            bx = coll_box(p, sx, sy, sz, ex, ey, ez);
+            w = coll_words(p, sx, sy, sz, ex, ey, ez, q);
+            const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
+            wide = nc > COLL_MAXC;
+            ncell = wide ? 0 : (int)nc;
+        }
+    }
+    CollAcc<REC> s = {};
+    const int ncw = __reduce_max_sync(FULLW, ncell);
+    int cx = bx.lox, cy = bx.loy, cz = bx.loz;
+    for (int c = 0; c < ncw; c++) {
+        int e0 = 0, cnt = 0;
+        if (c < ncell) {
+            const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
+            e0 = __ldg(p.cell_start + cell);
+            cnt = __ldg(p.cell_start + cell + 1) - e0;
+            if (sub == 0) ntest += (unsigned)cnt;
+        }
+        const bool big = cnt > COLL_MAXE;
+        const int own = big ? 0 : cnt;
+        for (int b = 0; __any_sync(FULLW, b < own); b += 32) {
+            const int n = min(own - b, 32);
+            unsigned m = 0u;  // the entries of this run that pass the filter
+            const uint4 *fil = p.efil + e0 + b;
+#pragma unroll 4
+            for (int t = sub; t < n; t += G) m |= (unsigned)coll_overlap(__ldg(fil + t), w) << t;
 #pragma unroll
-                    for (int t = 0; t < 6; t++) sh.g[wib][t][lane] = gn[t];
+            for (int d = 1; d < G; d <<= 1) m |= __shfl_xor_sync(FULLW, m, d);
+            while (__any_sync(FULLW, m != 0u)) {
+                // the group's next G survivors, one per lane in entry order
+                unsigned mine = m;
+#pragma unroll
+                for (int t = 0; t < G; t++) {
+                    if (t < sub) mine &= mine - 1u;
+                    m &= m - 1u;
                 }
-            }
-            __syncwarp();
-            if (cnt > 0) {
-                const int q0 = max(excl, r0), q1 = min(excl + cnt, r0 + 32);
-                for (int t = q0; t < q1; t++) {
-                    const float v = sh.val[wib][t - r0];
-                    if (v >= 0.0f) {
-                        acc += v;
-                        K++;
+                const int t = __ffs((int)mine) - 1;
+                float th = 0.0f, over = 0.0f, f = 0.0f;
+                float4 A, B = make_float4(0.0f, 0.0f, 0.0f, 0.0f), C = B;
+                const bool hit = t >= 0 && coll_candidate(p, q, (long long)e0 + b + t, cx, cy, cz, bx.lox, bx.loy,
+                                                          bx.loz, th, over, f, A, B, C);
+                const float val = fmaxf(over, 0.0f);
+                if (G == 1) {
+                    if (hit) coll_add<REC>(s, val, th, f, B, C);
+                } else {
+                    unsigned hm = (__ballot_sync(FULLW, hit) >> gbase) & ((1u << G) - 1u);
+                    while (__any_sync(FULLW, hm != 0u)) {
+                        const int from = hm ? gbase + __ffs((int)hm) - 1 : lane;
+                        const float hv = coll_shfl(val, from);
+                        float ht = 0.0f, hf = 0.0f;
+                        float4 hB = B, hC = C;
                         if constexpr (REC) {
-                            if (v > 0.0f) {
-                                g1[0] += sh.g[wib][0][t - r0]; g1[1] += sh.g[wib][1][t - r0];
-                                g1[2] += sh.g[wib][2][t - r0];
-                                g2[0] += sh.g[wib][3][t - r0]; g2[1] += sh.g[wib][4][t - r0];
-                                g2[2] += sh.g[wib][5][t - r0];
-                            }
+                            ht = coll_shfl(th, from);
+                            hf = coll_shfl(f, from);
+                            hB.x = coll_shfl(B.x, from); hB.y = coll_shfl(B.y, from); hB.z = coll_shfl(B.z, from);
+                            hC.x = coll_shfl(C.x, from); hC.y = coll_shfl(C.y, from); hC.z = coll_shfl(C.z, from);
                         }
+                        if (hm) coll_add<REC>(s, hv, ht, hf, hB, hC);
+                        hm &= hm - 1u;
                     }
                 }
             }
-            __syncwarp();
         }
-        if (!valid) return;
-        const StepParams &p = src.params(cloth);
-        float ox, oy, oz;
-        bool hit;
-        if (serial) {
-            if (REC) {
-                float sg1[3] = {0.0f, 0.0f, 0.0f}, sg2[3] = {0.0f, 0.0f, 0.0f}, mK[5];
-                hit = collide_t<true>(p, sx, sy, sz, ex, ey, ez, ox, oy, oz, sg1, sg2, mK);
-                if (hit) coll_record(p, o, mK[0], mK[1], mK[2], mK[3], mK[4], sg1, sg2);
-            } else {
-                hit = collide_t<false>(p, sx, sy, sz, ex, ey, ez, ox, oy, oz);
+        // crowded cells, one node's at a time over the whole warp
+        for (unsigned bm = __ballot_sync(FULLW, big && sub == 0); bm; bm &= bm - 1u) {
+            const int l = __ffs((int)bm) - 1;
+            const StepParams &lp = src.params(__shfl_sync(FULLW, cloth, l));
+            const CollPath lq = {coll_shfl(q.sx, l), coll_shfl(q.sy, l), coll_shfl(q.sz, l), coll_shfl(q.rx, l),
+                                 coll_shfl(q.ry, l), coll_shfl(q.rz, l), coll_shfl(q.L, l)};
+            const CollWords lw = {__shfl_sync(FULLW, w.a, l), __shfl_sync(FULLW, w.b, l), __shfl_sync(FULLW, w.c, l)};
+            CollBox lb = bx;
+            lb.lox = __shfl_sync(FULLW, bx.lox, l);
+            lb.loy = __shfl_sync(FULLW, bx.loy, l);
+            lb.loz = __shfl_sync(FULLW, bx.loz, l);
+            const int le0 = __shfl_sync(FULLW, e0, l), lcnt = __shfl_sync(FULLW, cnt, l);
+            const int lcx = __shfl_sync(FULLW, cx, l), lcy = __shfl_sync(FULLW, cy, l), lcz = __shfl_sync(FULLW, cz, l);
+            CollAcc<REC> t;
+            t.K = __shfl_sync(FULLW, s.K, l);
+            t.acc = coll_shfl(s.acc, l);
+            if constexpr (REC) {
+#pragma unroll
+                for (int a = 0; a < 3; a++) {
+                    t.g1[a] = coll_shfl(s.g1[a], l);
+                    t.g2[a] = coll_shfl(s.g2[a], l);
+                }
             }
-        } else {
-            hit = K > 0;
-            if (hit) {
-                const float m = acc / (float)K;
-                ox = sx + m * q.rx;
-                oy = sy + m * q.ry;
-                oz = sz + m * q.rz;
-                if (REC) coll_record(p, o, m, (float)K, q.rx, q.ry, q.rz, g1, g2);
+            for (int r0 = 0; r0 < lcnt; r0 += 32)
+                coll_warp_round<REC>(lp, lq, lw, lb, r0 + lane < lcnt, (long long)le0 + r0 + lane, lcx, lcy, lcz, t);
+            if (gbase == l) s = t;
+        }
+        if (++cx > bx.hix) {
+            cx = bx.lox;
+            if (++cy > bx.hiy) {
+                cy = bx.loy;
+                cz++;
             }
         }
-        if (hit) {
-            out[o] = ox;
-            out[st + o] = oy;
-            out[2 * st + o] = oz;
-            out[3 * st + o] *= p.restitution;
-            out[4 * st + o] *= p.restitution;
-            out[5 * st + o] *= p.restitution;
-            fsum += ox + oy + oz;
-            nhit++;
-        }
+    }
+    // long paths, one at a time over the whole warp (their candidates are not counted)
+    for (unsigned wm = __ballot_sync(FULLW, wide && sub == 0); wm; wm &= wm - 1u) {
+        const int l = __ffs((int)wm) - 1;
+        const CollPath lq = {coll_shfl(q.sx, l), coll_shfl(q.sy, l), coll_shfl(q.sz, l), coll_shfl(q.rx, l),
+                             coll_shfl(q.ry, l), coll_shfl(q.rz, l), coll_shfl(q.L, l)};
+        const CollWords lw = {__shfl_sync(FULLW, w.a, l), __shfl_sync(FULLW, w.b, l), __shfl_sync(FULLW, w.c, l)};
+        const CollBox lb = {__shfl_sync(FULLW, bx.lox, l), __shfl_sync(FULLW, bx.loy, l), __shfl_sync(FULLW, bx.loz, l),
+                            __shfl_sync(FULLW, bx.hix, l), __shfl_sync(FULLW, bx.hiy, l), __shfl_sync(FULLW, bx.hiz, l)};
+        CollAcc<REC> t = {};
+        coll_wide<REC>(src.params(__shfl_sync(FULLW, cloth, l)), lq, lw, lb, t);
+        if (gbase == l) s = t;
+    }
+    if (s.K > 0 && sub == 0) {
+        const float m = s.acc / (float)s.K;
+        // product and sum rounded separately, the same bits in every kernel
+        const float ox = __fadd_rn(q.sx, __fmul_rn(m, q.rx)), oy = __fadd_rn(q.sy, __fmul_rn(m, q.ry)),
+                    oz = __fadd_rn(q.sz, __fmul_rn(m, q.rz));
+        if constexpr (REC) coll_record(p, o, m, (float)s.K, q.rx, q.ry, q.rz, s.g1, s.g2);
+        out[o] = ox;
+        out[st + o] = oy;
+        out[2 * st + o] = oz;
+        out[3 * st + o] *= p.restitution;
+        out[4 * st + o] *= p.restitution;
+        out[5 * st + o] *= p.restitution;
+        fsum += ox + oy + oz;
+        nhit++;
     }
 }
 
-// The cooperative pass over a list of n entries: entry i goes to warp
-// i mod #warps (see above), 32 entries per warp and round.  has_pre: the
-// lane's entry of the first round (index coll_first_index()) is pre_o, which
-// the caller loaded before it knew n.
-template <bool REC = false, class Src, class Sh>
-__device__ __forceinline__ void collide_list(const Src &src, Sh &sh, unsigned long long k, unsigned n, float &fsum,
-                                             unsigned &ntest, unsigned &nhit, bool has_pre = false,
-                                             long long pre_o = 0)
+// The pass over a list of n entries in chunks of 32 / G neighbours, one per
+// warp and round.  A list of fewer chunks than warps is dealt over the CTAs
+// first (every SM gets some); a longer one in runs of COLL_WARPS chunks per
+// CTA, so that a CTA's warps share the lines of the cells they read.
+// has_pre: the lane's entry of the first round with G = COLL_GMAX and fewer
+// chunks than warps (index coll_first_index()) is pre_o.
+constexpr int COLL_GMAX = 8;
+__device__ __forceinline__ unsigned coll_first_index()
 {
+    const unsigned c = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    return c * (32 / COLL_GMAX) + (threadIdx.x & 31) / COLL_GMAX;
+}
+template <bool REC, int G, class Src>
+__device__ __forceinline__ void collide_chunks(const Src &src, unsigned long long k, unsigned n, float &fsum,
+                                               unsigned &ntest, unsigned &nhit, bool has_pre, int pre_o)
+{
+    constexpr unsigned PER = 32 / G;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const unsigned long long nw = (unsigned long long)gridDim.x * COLL_WARPS;
-    const unsigned long long w = (unsigned long long)blockIdx.x * COLL_WARPS + wib;
-    for (unsigned long long b0 = 0; b0 < n; b0 += 32ull * nw) {
-        const unsigned long long i = b0 + (unsigned long long)lane * nw + w;
-        collide_batch<REC>(src, sh, k, i < n, i, fsum, ntest, nhit, has_pre && b0 == 0, pre_o);
+    const unsigned chunks = (n + PER - 1u) / PER, nw = gridDim.x * COLL_WARPS;
+    const bool deal = chunks < nw;
+    const unsigned first = deal ? (unsigned)wib * gridDim.x + blockIdx.x : blockIdx.x * COLL_WARPS + wib;
+    for (unsigned c = first; c < chunks; c += nw) {
+        const unsigned long long i = (unsigned long long)PER * c + (unsigned)(lane / G);
+        collide_round<REC, G>(src, k, i < n, i, fsum, ntest, nhit, has_pre && deal && c == first, pre_o);
     }
 }
-
-// The calling lane's list index in the first round of collide_list.
-__device__ __forceinline__ unsigned long long coll_first_index()
+// Lanes per node: a short list leaves most of the grid's lanes idle and is
+// bound by its chain of dependent loads, so COLL_GMAX lanes share a node's
+// candidates; two where that still takes one round; else one, which does
+// the least work per node.  SHORT: the cloth is small (coll_short), so only
+// the first form is compiled in.
+template <bool REC, bool SHORT, class Src>
+__device__ __forceinline__ void collide_list(const Src &src, unsigned long long k, unsigned n, float &fsum,
+                                             unsigned &ntest, unsigned &nhit, bool has_pre = false, int pre_o = 0)
 {
-    const unsigned long long nw = (unsigned long long)gridDim.x * COLL_WARPS;
-    return (unsigned long long)(threadIdx.x & 31) * nw + (unsigned long long)blockIdx.x * COLL_WARPS +
-           (threadIdx.x >> 5);
+    const unsigned lanes = gridDim.x * 32u * COLL_WARPS;
+    if (SHORT || n <= lanes / COLL_GMAX)
+        collide_chunks<REC, COLL_GMAX>(src, k, n, fsum, ntest, nhit, has_pre, pre_o);
+    else if (n <= lanes / 2u)
+        collide_chunks<REC, 2>(src, k, n, fsum, ntest, nhit, false, 0);
+    else
+        collide_chunks<REC, 1>(src, k, n, fsum, ntest, nhit, false, 0);
 }
+
+// Per-lane scratch of the edge pass's cooperative rounds.
+struct CollLane {
+    float4 s;                   // S, L
+    float4 r;                   // r, owning cloth (int bits)
+    int4 box;                   // low cell, x extent | y extent << 16
+    int2 cell[COLL_MAXC];       // per cell of the box: first entry, end of the lane's running count
+};
 
 // Adds a collision pass's counts to the cloth's running statistics: every
 // warp's tested candidates and hit nodes are summed per CTA in shared memory
@@ -395,9 +481,9 @@ __device__ __forceinline__ unsigned long long coll_first_index()
 // so no thread waits on them.
 __device__ __forceinline__ void coll_stats_add(DevCtrl *ctrl, unsigned *s2, unsigned n, unsigned ntest, unsigned nhit)
 {
-    const unsigned h = __reduce_add_sync(0xffffffffu, nhit);
+    const unsigned h = __reduce_add_sync(0xffffffffu, nhit), q = __reduce_add_sync(0xffffffffu, ntest);
     if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&s2[0], ntest);
+        atomicAdd(&s2[0], q);
         atomicAdd(&s2[1], h);
     }
     __syncthreads();
@@ -504,10 +590,10 @@ __device__ __forceinline__ float4 edge_hits_warp(const StepParams &p, const Coll
             bool hit = false;
             float th = 0.0f;
             if (j < total) {
-                float f;
+                float f, over;
                 float4 A, B, C;
                 hit = coll_candidate(p, path, (long long)oe0 + (j - oex), ocx, ocy, ocz, bx.lox, bx.loy, bx.loz, th,
-                                     f, A, B, C);
+                                     over, f, A, B, C);
             }
             const unsigned hm = __ballot_sync(FULLW, hit);
             if (hm) {
@@ -617,9 +703,9 @@ __device__ __forceinline__ void edge_test_list(const StepParams &p, EdgeShared &
                 const int nxc = L.box.w & 0xffff, nyc = L.box.w >> 16;
                 const int cx = L.box.x + cc % nxc, cy = L.box.y + (cc / nxc) % nyc, cz = L.box.z + cc / (nxc * nyc);
                 const CollPath lq = {L.s.x, L.s.y, L.s.z, L.r.x, L.r.y, L.r.z, L.s.w};
-                float th, f;
+                float th, over, f;
                 float4 A, B, C;
-                if (coll_candidate(p, lq, e, cx, cy, cz, L.box.x, L.box.y, L.box.z, th, f, A, B, C)) {
+                if (coll_candidate(p, lq, e, cx, cy, cz, L.box.x, L.box.y, L.box.z, th, over, f, A, B, C)) {
                     const float3 hp = coll_hit_point(lq, th);
                     hv = make_float4(hp.x, hp.y, hp.z, 1.0f);
                 }
@@ -699,9 +785,9 @@ static __device__ __noinline__ EdgeAcc edge_rewalk(const StepParams &p, const fl
                 const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
                 const int e0 = __ldg(p.cell_start + cell), e1 = __ldg(p.cell_start + cell + 1);
                 for (int ee = e0; ee < e1; ee++) {
-                    float th, f;
+                    float th, over, f;
                     float4 A, B, C;
-                    if (!coll_candidate(p, path, ee, cx, cy, cz, bx.lox, bx.loy, bx.loz, th, f, A, B, C)) continue;
+                    if (!coll_candidate(p, path, ee, cx, cy, cz, bx.lox, bx.loy, bx.loz, th, over, f, A, B, C)) continue;
                     if (first) {
                         first = false;
                         continue;

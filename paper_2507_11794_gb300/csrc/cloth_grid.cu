@@ -186,17 +186,36 @@ __global__ void cell_sort_kernel(const int *__restrict__ cell_start, long long n
     }
 }
 
+// One axis of a triangle's filter box (see cloth_collide.cuh), grown by pad
+// units.  Infinite bounds saturate; vertices are finite.
+__device__ __forceinline__ uint2 filter_side(float a, float e1, float e2, float o, float qs, float pad)
+{
+    const float b = a + e1, c = a + e2;
+    const float lo = floorf(__fmul_rn(__fsub_rn(fminf(fminf(a, b), c), o), qs)) - pad;
+    const float hi = floorf(__fmul_rn(__fsub_rn(fmaxf(fmaxf(a, b), c), o), qs)) + pad;
+    const float top = (float)GRID_FILTER_MAX;
+    return make_uint2((unsigned)fminf(fmaxf(lo, 0.0f), top), (unsigned)fminf(fmaxf(hi, 0.0f), top));
+}
+
 // Expand the sorted (cell, triangle) pairs into per-entry records read by the
-// narrow phase without an indirection: the triangle's plane and first cell.
+// narrow phase without an indirection: the triangle's plane and first cell,
+// and its box as filter words.
 __global__ void expand_kernel(const float4 *__restrict__ rec, const int *__restrict__ tri_ids, long long n,
-                              float4 *__restrict__ etri)
+                              float ox, float oy, float oz, float qs, float pad, float4 *__restrict__ etri,
+                              uint4 *__restrict__ efil)
 {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
     const int t = tri_ids[e];
-    etri[3 * e] = rec[3 * t];
-    etri[3 * e + 1] = rec[3 * t + 1];
-    etri[3 * e + 2] = rec[3 * t + 2];
+    const float4 A = rec[3 * t], B = rec[3 * t + 1], C = rec[3 * t + 2];
+    etri[3 * e] = A;
+    etri[3 * e + 1] = B;
+    etri[3 * e + 2] = C;
+    const uint2 x = filter_side(A.x, B.x, C.x, ox, qs, pad);
+    const uint2 y = filter_side(A.y, B.y, C.y, oy, qs, pad);
+    const uint2 z = filter_side(A.z, B.z, C.z, oz, qs, pad);
+    efil[e] = make_uint4(GRID_FILTER_GUARD | x.y | y.y << 16, GRID_FILTER_GUARD | z.y | (GRID_FILTER_MAX - x.x) << 16,
+                         GRID_FILTER_GUARD | (GRID_FILTER_MAX - y.x) | (GRID_FILTER_MAX - z.x) << 16, 0u);
 }
 
 __global__ void query_kernel(const float4 *__restrict__ rec, const int *__restrict__ cell_start,
@@ -300,6 +319,8 @@ cudaError_t grid_build(const float *d_verts, const int *d_tris, int nt, DevGrid 
     g->cell_start = nullptr;
     g->tri_ids = nullptr;
     g->etri = nullptr;
+    g->efil = nullptr;
+    g->qs = grid_filter_scale(g->dims, g->inv);
     GTRY(cudaMalloc(&g->tri, sizeof(float4) * 3 * (size_t)nt));
     GTRY(cudaMalloc(&g->cell_start, sizeof(int) * (size_t)(nc + 1)));
     GTRY(cudaMalloc(&box_hi, sizeof(int4) * (size_t)nt));
@@ -335,9 +356,18 @@ cudaError_t grid_build(const float *d_verts, const int *d_tris, int nt, DevGrid 
     GTRY(cudaGetLastError());
     cell_sort_kernel<<<blocks_for(nc, 256), 256, 0, s>>>(g->cell_start, nc, g->tri_ids);
     GTRY(cudaGetLastError());
-    GTRY(cudaMalloc(&g->etri, sizeof(float4) * 3 * (size_t)(htotal > 0 ? htotal : 1)));
+    // records and filter words in one allocation
+    GTRY(cudaMalloc(&g->etri, (sizeof(float4) * 3 + sizeof(uint4)) * (size_t)(htotal > 0 ? htotal : 1)));
+    g->efil = (uint4 *)(g->etri + 3 * htotal);
     if (htotal > 0) {
-        expand_kernel<<<blocks_for((long long)htotal, 256), 256, 0, s>>>(g->tri, g->tri_ids, (long long)htotal, g->etri);
+        // float32 coordinates up to `top` can be off by a few 2^-24 top
+        double top = 0.0;
+        for (int a = 0; a < 3; a++)
+            top = fmax(top, fmax(fabs((double)g->origin[a]), fabs((double)g->origin[a] + (double)g->dims[a] * g->h)));
+        const float pad = (float)fmin(1.0 + ceil(4e-7 * top * g->qs), 40000.0);
+        expand_kernel<<<blocks_for((long long)htotal, 256), 256, 0, s>>>(g->tri, g->tri_ids, (long long)htotal,
+                                                                         g->origin[0], g->origin[1], g->origin[2],
+                                                                         g->qs, pad, g->etri, g->efil);
         GTRY(cudaGetLastError());
     }
     GTRY(cudaStreamSynchronize(s));
@@ -358,6 +388,7 @@ void grid_free(DevGrid *g)
     cudaFree(g->tri_ids);
     cudaFree(g->etri);
     g->etri = nullptr;
+    g->efil = nullptr;
     g->tri = nullptr;
     g->cell_start = nullptr;
     g->tri_ids = nullptr;

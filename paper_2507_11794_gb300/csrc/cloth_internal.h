@@ -9,10 +9,15 @@
 // Device-side control block of one cloth (one per handle, in device memory).
 struct DevCtrl {
     unsigned long long k;     // global substep counter: selects time and ping-pong buffer
-    unsigned int blocks_done; // completion counter of the running substep launch
+    unsigned int blocks_done; // completion counter of the running substep launch (substeps without a mesh)
     unsigned int flags;       // CTRL_FLAG_* (sticky until set_state)
-    unsigned int coll_count;  // marked nodes of the running substep
-    unsigned int pad;
+    // With a surface model a substep needs no completion count: the walk
+    // copies k to kc, which the collision kernels read, so their first CTA can
+    // advance k at once; they list into coll_count[k & 1] and zero the other
+    // one, which the next substep uses.  Whoever sets k from outside zeroes
+    // both (ctrl_set_k).
+    unsigned long long kc;
+    unsigned int coll_count[2];
     // running collision statistics since create: listed nodes, candidate
     // triangles tested, nodes that hit (summed over substeps)
     unsigned long long stat_listed, stat_tested, stat_hits;
@@ -61,6 +66,8 @@ struct StepParams {
     const int *cell_start;
     const int *tri_ids;
     const float4 *etri;        // per grid entry: its triangle's 3 records (no dependent load)
+    const uint4 *efil;         // per grid entry: its triangle's box as filter words (cloth_collide.cuh)
+    float qs;                  // filter units per length (0: every entry passes)
     float go[3];
     float ginv;
     int gd[3];
@@ -75,8 +82,9 @@ struct StepParams {
     float4 *edge_hit;          // edge narrow phase: per edge (kind * stride + owner) first hit point, hit count
     float4 *edge_more;         // edge narrow phase: CLOTH_EDGE_MORE planes of 3 x stride later hit points
     unsigned long long *edge_stamp; // edge narrow phase: per node, 1 + the substep it was last listed in
-    unsigned *coll_count;      // entries in coll_list (reset by the collision kernel)
+    unsigned *coll_count;      // entries in coll_list, by substep parity (DevCtrl.coll_count)
     int coll_blocks;           // CTAs of the collision kernel
+    int coll_short;            // its form (see coll_short())
     float delta, eps, tmin, restitution;
     DevCtrl *ctrl;
 };
@@ -85,10 +93,24 @@ struct StepParams {
 // with more hits is walked again by the gather pass).
 #define CLOTH_EDGE_MORE 3
 
-// CTAs per SM of the collision kernels (grid = SMs x this).
+// The collision kernels come in two forms (see collide_list): for cloths
+// of up to COLL_SHORT_NODES per SM, whose lists leave lanes idle, and for more.
+// Grids are at most what is resident at once, and no more than give every node
+// its eight lanes.
 #ifndef CLOTH_COLL_CTAS_PER_SM
-#define CLOTH_COLL_CTAS_PER_SM 2
+#define CLOTH_COLL_CTAS_PER_SM 4
 #endif
+#ifndef CLOTH_COLL_SHORT_CTAS_PER_SM
+#define CLOTH_COLL_SHORT_CTAS_PER_SM 3
+#endif
+#define COLL_SHORT_NODES 128
+inline bool coll_short(long long n, int sms) { return n <= (long long)COLL_SHORT_NODES * sms; }
+inline int coll_ctas(long long n, int sms)
+{
+    const long long want = (8 * n + 255) / 256;
+    const long long most = (long long)sms * (coll_short(n, sms) ? CLOTH_COLL_SHORT_CTAS_PER_SM : CLOTH_COLL_CTAS_PER_SM);
+    return (int)(want < 1 ? 1 : (want > most ? most : want));
+}
 
 // Launch one substep (reads state k&1, writes the other, advances ctrl->k).
 cudaError_t launch_substep(const StepParams &p, cudaStream_t s);
@@ -138,6 +160,8 @@ struct DevGrid {
     int *cell_start;   // ncells + 1
     int *tri_ids;      // nentries
     float4 *etri;      // 3 per entry: copy of the entry's triangle record
+    uint4 *efil;       // 1 per entry: the triangle's box as filter words (in etri's allocation)
+    float qs;          // filter units per length
     int ntris;
     float lo[3], hi[3];  // box of the triangles' vertices
 };
@@ -162,7 +186,35 @@ cudaError_t launch_aos_to_soa(const float *aos_pos, const float *aos_vel, float 
 cudaError_t launch_soa_to_aos(const float *state0, const float *state1, long long stride, int n, int nx, int pitch,
                               const DevCtrl *ctrl, float *aos_pos, float *aos_vel, cudaStream_t s);
 
+// Narrow-phase filter (see cloth_collide.cuh): boxes in units of 1 / sub of a
+// cell, 15 bits a side; sub is 64 where the grid's longest side leaves room for
+// it.  The scale is 0 where it does not fit at all (then every box is the
+// same and passes).  The triangles' boxes grow by grid_filter_pad units: one
+// for the narrow phase's own rounding, far below 1 / 64 of a cell, and what
+// float32 coordinates of the mesh's magnitude can be off.
+#define GRID_FILTER_MAX 32767u
+#define GRID_FILTER_GUARD 0x80008000u
+inline float grid_filter_scale(const int dims[3], float inv)
+{
+    int d = dims[0] > dims[1] ? dims[0] : dims[1];
+    d = d > dims[2] ? d : dims[2];
+    const int sub = (int)(GRID_FILTER_MAX / (unsigned)d);
+    return inv * (float)(sub > 64 ? 64 : sub);
+}
+
 #ifdef __CUDACC__
+// Sets the substep counter from outside a substep (one thread).
+__device__ __forceinline__ void ctrl_set_k(DevCtrl *ctrl, unsigned long long k)
+{
+    ctrl->k = k;
+    ctrl->coll_count[0] = ctrl->coll_count[1] = 0u;
+}
+
+__device__ __forceinline__ unsigned grid_filter_coord(float x, float o, float qs)
+{
+    return (unsigned)fminf(fmaxf(floorf(__fmul_rn(__fsub_rn(x, o), qs)), 0.0f), (float)GRID_FILTER_MAX);
+}
+
 // The wind's time phase omega k + phase0 reduced to [0, 2 pi), in float.
 // omega and phase0 are held in turns as 64-bit binary fractions, so the
 // reduction modulo one turn is the wrap of integer arithmetic: no FP64 on

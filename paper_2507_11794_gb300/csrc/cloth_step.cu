@@ -38,7 +38,7 @@ namespace {
 #define CLOTH_WALK_UNROLL 1
 #endif
 #ifndef CLOTH_COLL_MINB
-#define CLOTH_COLL_MINB 2
+#define CLOTH_COLL_MINB 4
 #endif
 #define CLOTH_PRAGMA(x) _Pragma(#x)
 #define CLOTH_UNROLL(n) CLOTH_PRAGMA(unroll n)
@@ -273,7 +273,7 @@ __device__ __forceinline__ WalkStatics walk_statics(const StepParams &p, int sx,
 // measured time (they change the register allocation).
 template <bool MESH, bool PER_SPRING, bool DLR = false, bool PMARK = false>
 __device__ __forceinline__ void walk_strip(const StepParams &p, const float *__restrict__ in, float *__restrict__ out,
-                                           float wbase, int sx, int sy, int lane, int cloth,
+                                           float wbase, int sx, int sy, int lane, int cloth, unsigned *coll_count,
                                            float2 &fsum, const WalkStatics &ws)
 {
     const long long st = p.stride;
@@ -591,7 +591,7 @@ __device__ __forceinline__ void walk_strip(const StepParams &p, const float *__r
         const int total = __reduce_add_sync(FULL, cnt);
         if (total > 0) {
             unsigned base = 0;
-            if (lane == 0) base = atomicAdd(p.coll_count, (unsigned)total);
+            if (lane == 0) base = atomicAdd(coll_count, (unsigned)total);
             base = __shfl_sync(FULL, base, 0);
             while (rows) {
                 const int b = __ffs((int)rows) - 1;
@@ -668,7 +668,8 @@ __global__ void CLOTH_WALK_BOUNDS substep_kernel(const StepParams p)
     float2 fsum = bc(0.0f);
     // DLR (receiver-side (+1,-1) springs) in the mesh walk only: 2% faster
     // there, slower without a mesh
-    if (active) walk_strip<MESH && !EDGE, PER_SPRING, DLR>(p, in, out, wbase, sx, sy, lane, 0, fsum, ws);
+    if (active) walk_strip<MESH && !EDGE, PER_SPRING, DLR>(p, in, out, wbase, sx, sy, lane, 0, p.coll_count + (k & 1ull),
+                                                             fsum, ws);
     // the launch's parity checked against the counter after the walk (a
     // check before it would make the walk wait for the counter)
     if (!DLR && p.parity >= 0 && (int)(k & 1ull) != p.parity && threadIdx.x == 0)
@@ -676,7 +677,10 @@ __global__ void CLOTH_WALK_BOUNDS substep_kernel(const StepParams p)
 
     const bool bad = !isfinite(fsum.x + fsum.y);
     if (__any_sync(FULL, bad) && lane == 0) atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
-    if (MESH || EDGE) return;  // the collision kernels finish the substep
+    if (MESH || EDGE) {  // the collision kernels finish the substep
+        if (blockIdx.x == 0 && threadIdx.x == 0) p.ctrl->kc = k;
+        return;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         // the last CTA to finish advances the substep counter for the next launch
@@ -692,6 +696,25 @@ __global__ void CLOTH_WALK_BOUNDS substep_kernel(const StepParams p)
 // response of every node the walk listed (warp-cooperative, collide_list),
 // then the substep counter advances.
 
+// Start of a collision kernel (one thread per CTA): the substep and the number
+// of nodes its walk listed.
+__device__ __forceinline__ void coll_begin(DevCtrl *ctrl, unsigned long long &k, unsigned &n)
+{
+    const volatile DevCtrl *c = ctrl;
+    const unsigned long long kc = c->kc;
+    const unsigned n0 = c->coll_count[0], n1 = c->coll_count[1];
+    k = kc;
+    n = (kc & 1ull) ? n1 : n0;
+}
+// End of a substep with a surface model (one thread of its last kernel, at
+// any point after that kernel's wait): nothing else reads k or the other count
+// before the next substep, which starts after this kernel has completed.
+__device__ __forceinline__ void coll_end(DevCtrl *ctrl, unsigned long long k)
+{
+    ctrl->coll_count[(k + 1ull) & 1ull] = 0u;
+    ctrl->k = k + 1ull;
+}
+
 // List entries of one cloth.
 struct OneClothList {
     const StepParams &p;
@@ -704,50 +727,44 @@ struct OneClothList {
 };
 
 // Collision pass over the nodes the walk listed (cooperative, see
-// collide_list); the last CTA resets the list and advances the substep counter.
+// collide_list); the first CTA advances the substep counter.
 // REC: the adjoint recompute's variant, which also records each hit's
 // response data (p.cdata, p.cbits).
-template <bool REC>
-__global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) collide_kernel(const __grid_constant__ StepParams p)
+// Bound by its chain of dependent loads (list entry, state, cell, filter
+// words, records, response) on short lists and by issue slots on long ones.
+// SHORT (see collide_list) holds three CTAs per SM without spilling much, the
+// long form four of 64 registers.  Measured per step of cloth_step against the
+// pass that spread every candidate's full test over the warp: 256 x 256 nodes
+// lying on 81,920 triangles (784,000 candidates a substep) 26 -> 16 us per
+// substep, 1.45M nodes in a batch (24.7M candidates) 437 -> 84 us (ncu);
+// the long form at three CTAs per SM is 8 % slower on the first, SHORT at two
+// 9 % on a rollout's 16,384 nodes.
+template <bool REC, bool SHORT>
+__global__ void __launch_bounds__(32 * COLL_WARPS, SHORT ? CLOTH_COLL_SHORT_CTAS_PER_SM : CLOTH_COLL_MINB) collide_kernel(const __grid_constant__ StepParams p)
 {
-    __shared__ std::conditional_t<REC, CollSharedRec, CollShared> sh;
     __shared__ unsigned long long s_k;
     __shared__ unsigned s_n, s_stat[2];
     pdl_launch_dependents();
     pdl_wait();
-    // the lane's first list entry, loaded beside the list length instead of
-    // after it (the list holds p.n entries; one past the length is stale and
-    // ignored)
-    const unsigned long long i0 = coll_first_index();
-    const long long pre_o = i0 < (unsigned long long)p.n ? (long long)__ldg(p.coll_list + i0) : 0ll;
+    // the lane's first list entry in case the list is short, loaded beside
+    // the list length instead of after it (the list holds p.n entries; one past
+    // the length is stale and ignored)
+    const unsigned i0 = coll_first_index();
+    const int pre_o = i0 < (unsigned)p.n ? p.coll_list[i0] : 0;
     if (threadIdx.x == 0) {
-        s_k = *(volatile unsigned long long *)&p.ctrl->k;
-        s_n = *(volatile unsigned *)p.coll_count;
+        coll_begin(p.ctrl, s_k, s_n);
         s_stat[0] = s_stat[1] = 0u;
     }
     __syncthreads();
     const unsigned long long k = s_k;
-    if (s_n == 0u) {
-        // nothing listed (every CTA sees the same final count): CTA 0 alone
-        // ends the substep; the others read k only to ignore it, and the
-        // next kernel reads it after this grid completes
-        if (blockIdx.x == 0 && threadIdx.x == 0) p.ctrl->k = k + 1;
-        return;
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) coll_end(p.ctrl, k);
+    if (s_n == 0u) return;
     float fsum = 0.0f;
     unsigned ntest = 0u, nhit = 0u;
-    collide_list<REC>(OneClothList{p}, sh, k, s_n, fsum, ntest, nhit, true, pre_o);
+    collide_list<REC, SHORT>(OneClothList{p}, k, s_n, fsum, ntest, nhit, true, pre_o);
     if (__any_sync(FULL, !isfinite(fsum)) && (threadIdx.x & 31) == 0)
         atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
     coll_stats_add(p.ctrl, s_stat, s_n, ntest, nhit);
-    if (threadIdx.x == 0) {
-        const unsigned prev = atomicAdd(&p.ctrl->blocks_done, 1u);
-        if (prev == gridDim.x - 1) {
-            p.ctrl->blocks_done = 0;
-            *p.coll_count = 0u;
-            p.ctrl->k = k + 1;
-        }
-    }
 }
 
 // Listing of the edge narrow phase: every node whose 3 x 3 block of
@@ -765,7 +782,7 @@ __global__ void __launch_bounds__(256) edge_list_kernel(const __grid_constant__ 
     __shared__ unsigned long long s_k;
     pdl_launch_dependents();
     pdl_wait();
-    if (threadIdx.x == 0) s_k = *(volatile unsigned long long *)&p.ctrl->k;
+    if (threadIdx.x == 0) s_k = *(volatile unsigned long long *)&p.ctrl->kc;
     __syncthreads();
     const unsigned long long k = s_k;
     const float *xs = (k & 1ull) ? p.state0 : p.state1;  // updated positions
@@ -803,7 +820,7 @@ __global__ void __launch_bounds__(256) edge_list_kernel(const __grid_constant__ 
         const unsigned m = __ballot_sync(FULL, want);
         if (m) {
             unsigned base = 0;
-            if (lane == 0) base = atomicAdd(p.coll_count, (unsigned)__popc(m));
+            if (lane == 0) base = atomicAdd(p.coll_count + (k & 1ull), (unsigned)__popc(m));
             base = __shfl_sync(FULL, base, 0);
             if (want) {
                 p.coll_list[base + __popc(m & ((1u << lane) - 1u))] = o;
@@ -817,7 +834,7 @@ __global__ void __launch_bounds__(256) edge_list_kernel(const __grid_constant__ 
 // node's owned edges and records their hits; pass B gathers every listed free
 // node's response from the records of its 12 edges into a scratch array; a
 // third kernel applies the responses, so no test reads a moved node.
-__global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) edge_test_kernel(const __grid_constant__ StepParams p)
+__global__ void __launch_bounds__(32 * COLL_WARPS, 2) edge_test_kernel(const __grid_constant__ StepParams p)
 {
     __shared__ EdgeShared sh;
     __shared__ unsigned long long s_k;
@@ -825,8 +842,7 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) edge_test_ke
     pdl_launch_dependents();
     pdl_wait();
     if (threadIdx.x == 0) {
-        s_k = *(volatile unsigned long long *)&p.ctrl->k;
-        s_n = *(volatile unsigned *)p.coll_count;
+        coll_begin(p.ctrl, s_k, s_n);
         s2[0] = s2[1] = 0u;
     }
     __syncthreads();
@@ -841,10 +857,7 @@ __global__ void __launch_bounds__(256) edge_gather_kernel(const __grid_constant_
     __shared__ unsigned s_n;
     pdl_launch_dependents();
     pdl_wait();
-    if (threadIdx.x == 0) {
-        s_k = *(volatile unsigned long long *)&p.ctrl->k;
-        s_n = *(volatile unsigned *)p.coll_count;
-    }
+    if (threadIdx.x == 0) coll_begin(p.ctrl, s_k, s_n);
     __syncthreads();
     edge_gather_list(p, s_k, s_n);
 }
@@ -855,10 +868,7 @@ __global__ void __launch_bounds__(256) edge_apply_kernel(const __grid_constant__
     __shared__ unsigned s_n;
     pdl_launch_dependents();
     pdl_wait();
-    if (threadIdx.x == 0) {
-        s_k = *(volatile unsigned long long *)&p.ctrl->k;
-        s_n = *(volatile unsigned *)p.coll_count;
-    }
+    if (threadIdx.x == 0) coll_begin(p.ctrl, s_k, s_n);
     __syncthreads();
     const unsigned long long k = s_k;
     float *out = (k & 1ull) ? p.state0 : p.state1;
@@ -878,16 +888,7 @@ __global__ void __launch_bounds__(256) edge_apply_kernel(const __grid_constant__
     }
     if (__any_sync(FULL, !isfinite(fsum)) && (threadIdx.x & 31) == 0)
         atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // the last CTA resets the list and advances the substep counter
-        const unsigned prev = atomicAdd(&p.ctrl->blocks_done, 1u);
-        if (prev == gridDim.x - 1) {
-            p.ctrl->blocks_done = 0;
-            *p.coll_count = 0u;
-            p.ctrl->k = k + 1;
-        }
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) coll_end(p.ctrl, k);
 }
 
 // ---------------------------------------------------------------- batches
@@ -929,30 +930,22 @@ __global__ void __launch_bounds__(32 * CLOTH_WALK_WARPS, CLOTH_BATCH_MINB) batch
         if (VAR != BATCH_VAR_MIXED) {
             // the packed listing test: 3.6% faster on config 5
             walk_strip<(VAR & BATCH_VAR_MESH) != 0, (VAR & BATCH_VAR_PER_SPRING) != 0, false, true>(
-                p, in, out, wbase, it.y, it.z, lane, it.x, fsum, ws);
+                p, in, out, wbase, it.y, it.z, lane, it.x, b.coll_count + (k & 1ull), fsum, ws);
         } else if (p.has_mesh) {
-            if (p.ks_slot) walk_strip<true, true>(p, in, out, wbase, it.y, it.z, lane, it.x, fsum, ws);
-            else walk_strip<true, false>(p, in, out, wbase, it.y, it.z, lane, it.x, fsum, ws);
+            if (p.ks_slot) walk_strip<true, true>(p, in, out, wbase, it.y, it.z, lane, it.x, b.coll_count + (k & 1ull), fsum, ws);
+            else walk_strip<true, false>(p, in, out, wbase, it.y, it.z, lane, it.x, b.coll_count + (k & 1ull), fsum, ws);
         } else {
-            if (p.ks_slot) walk_strip<false, true>(p, in, out, wbase, it.y, it.z, lane, it.x, fsum, ws);
-            else walk_strip<false, false>(p, in, out, wbase, it.y, it.z, lane, it.x, fsum, ws);
+            if (p.ks_slot) walk_strip<false, true>(p, in, out, wbase, it.y, it.z, lane, it.x, b.coll_count + (k & 1ull), fsum, ws);
+            else walk_strip<false, false>(p, in, out, wbase, it.y, it.z, lane, it.x, b.coll_count + (k & 1ull), fsum, ws);
         }
         __syncwarp();  // the slot is rewritten by the next item
     }
     if (__any_sync(FULL, !isfinite(fsum.x + fsum.y)) && lane == 0)
         atomicOr(&b.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // the last CTA re-arms the work counter (the collision kernel advances k)
-        const unsigned prev = atomicAdd(&b.ctrl->blocks_done, 1u);
-        if (prev == gridDim.x - 1) {
-            b.ctrl->blocks_done = 0;
-            *b.work = 0u;
-        }
-    }
+    // the collision kernel re-arms the work counter and advances k
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.ctrl->kc = k;
 }
 
-// Collision kernel of a batch: every entry carries its cloth index.
 // List entries of a batch: each carries its cloth.
 struct BatchList {
     const BatchArgs &b;
@@ -966,32 +959,27 @@ struct BatchList {
 
 __global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) batch_collide_kernel(const __grid_constant__ BatchArgs b)
 {
-    __shared__ CollShared sh;
     __shared__ unsigned long long s_k;
     __shared__ unsigned s_n, s_stat[2];
     pdl_launch_dependents();
     pdl_wait();
     if (threadIdx.x == 0) {
-        s_k = *(volatile unsigned long long *)&b.ctrl->k;
-        s_n = *(volatile unsigned *)b.coll_count;
+        coll_begin(b.ctrl, s_k, s_n);
         s_stat[0] = s_stat[1] = 0u;
     }
     __syncthreads();
     const unsigned long long k = s_k;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *b.work = 0u;
+        coll_end(b.ctrl, k);
+    }
+    if (s_n == 0u) return;
     float fsum = 0.0f;
     unsigned ntest = 0u, nhit = 0u;
-    collide_list(BatchList{b}, sh, k, s_n, fsum, ntest, nhit);
+    collide_list<false, false>(BatchList{b}, k, s_n, fsum, ntest, nhit);
     if (__any_sync(FULL, !isfinite(fsum)) && (threadIdx.x & 31) == 0)
         atomicOr(&b.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
     coll_stats_add(b.ctrl, s_stat, s_n, ntest, nhit);
-    if (threadIdx.x == 0) {
-        const unsigned prev = atomicAdd(&b.ctrl->blocks_done, 1u);
-        if (prev == gridDim.x - 1) {
-            b.ctrl->blocks_done = 0;
-            *b.coll_count = 0u;
-            b.ctrl->k = k + 1;
-        }
-    }
 }
 
 __global__ void aos_to_soa_kernel(const float *__restrict__ pos, const float *__restrict__ vel, float *state0,
@@ -1112,8 +1100,11 @@ cudaError_t launch_collide(const StepParams &p, cudaStream_t s)
         if (e != cudaSuccess) return e;
         return launch_k(edge_apply_kernel, p.coll_blocks, 256, s, p);
     }
-    if (p.cdata) return launch_k(collide_kernel<true>, p.coll_blocks, 32 * COLL_WARPS, s, p);
-    return launch_k(collide_kernel<false>, p.coll_blocks, 32 * COLL_WARPS, s, p);
+    if (p.coll_short)
+        return p.cdata ? launch_k(collide_kernel<true, true>, p.coll_blocks, 32 * COLL_WARPS, s, p)
+                       : launch_k(collide_kernel<false, true>, p.coll_blocks, 32 * COLL_WARPS, s, p);
+    return p.cdata ? launch_k(collide_kernel<true, false>, p.coll_blocks, 32 * COLL_WARPS, s, p)
+                   : launch_k(collide_kernel<false, false>, p.coll_blocks, 32 * COLL_WARPS, s, p);
 }
 
 cudaError_t launch_substep(const StepParams &p, cudaStream_t s)
