@@ -100,6 +100,11 @@ __device__ __forceinline__ bool coll_path(const StepParams &p, float sx, float s
 // path, M = 32767; the boxes overlap iff every lane of T is >= that of N, i.e.
 // iff no guard bit is borrowed from.  A path can only hit a triangle whose
 // box it overlaps, so the test below it runs on the entries that pass.
+// The fourth word has bit a (0, 1, 2) where the entry's cell is the first of
+// the triangle's box along axis a: a triangle listed in several cells of a
+// path's box is tested only in the first cell the two boxes share, which is
+// this one iff along every axis the cell is the path box's first or that bit
+// is set (the same rule coll_candidate applies to the full record).
 struct CollWords {
     unsigned a, b, c;
 };
@@ -117,38 +122,88 @@ __device__ __forceinline__ CollWords coll_words(const StepParams &p, float sx, f
     const unsigned lz = grid_filter_coord(fminf(sz, ez), p.go[2], p.qs), hz = grid_filter_coord(fmaxf(sz, ez), p.go[2], p.qs);
     return {lx | ly << 16, lz | (GRID_FILTER_MAX - hx) << 16, (GRID_FILTER_MAX - hy) | (GRID_FILTER_MAX - hz) << 16};
 }
-__device__ __forceinline__ bool coll_overlap(const uint4 &t, const CollWords &n)
+// need: bit a set where the cell is not the path box's first along axis a.
+__device__ __forceinline__ bool coll_overlap(const uint4 &t, const CollWords &n, unsigned need)
 {
-    return (((t.x - n.a) & (t.y - n.b) & (t.z - n.c)) & GRID_FILTER_GUARD) == GRID_FILTER_GUARD;
+    return (((t.x - n.a) & (t.y - n.b) & (t.z - n.c)) & GRID_FILTER_GUARD) == GRID_FILTER_GUARD && !(need & ~t.w);
+}
+__device__ __forceinline__ unsigned coll_need(const CollBox &bx, int cx, int cy, int cz)
+{
+    return (cx != bx.lox) | (cy != bx.loy) << 1 | (cz != bx.loz) << 2;
 }
 
-// Running sums of one node's hits: K and sum max(t - delta, 0) and, for the
-// adjoint's recompute (REC), over the active hits (t > delta) g1 = sum n/a
-// and g2 = sum t n/a (n = e1 x e2), the derivatives of t w.r.t. S and r.
+__device__ __forceinline__ float coll_shfl(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+// What a path's hits are added to.  add<G>: every lane of a group of G brings
+// one tested candidate (hit: whether it hit; th, over, f, B, C as from
+// coll_candidate) and the group adds the hits in lane order, all of its lanes
+// ending with the same sums; converged warps only for G > 1.  from(l): lane
+// l's, in every lane.
+//
+// A node's: K and sum max(t - delta, 0) and, for the adjoint's recompute (REC),
+// over the active hits (t > delta) g1 = sum n/a and g2 = sum t n/a (n = e1 x e2),
+// the derivatives of t w.r.t. S and r.
 template <bool REC>
-struct CollAcc {
+struct NodeHits {
     int K;
     float acc, g1[REC ? 3 : 1], g2[REC ? 3 : 1];
-};
-template <bool REC>
-__device__ __forceinline__ void coll_add(CollAcc<REC> &s, float val, float th, float f, const float4 &B,
-                                         const float4 &C)
-{
-    s.K++;
-    s.acc += val;
-    if constexpr (REC) {
-        if (val > 0.0f) {
-            const float nx = B.y * C.z - B.z * C.y, ny = B.z * C.x - B.x * C.z, nz = B.x * C.y - B.y * C.x;
-            // products rounded before they are added, in either walk below
-            s.g1[0] = __fadd_rn(s.g1[0], __fmul_rn(nx, f));
-            s.g1[1] = __fadd_rn(s.g1[1], __fmul_rn(ny, f));
-            s.g1[2] = __fadd_rn(s.g1[2], __fmul_rn(nz, f));
-            s.g2[0] = __fadd_rn(s.g2[0], __fmul_rn(__fmul_rn(th, nx), f));
-            s.g2[1] = __fadd_rn(s.g2[1], __fmul_rn(__fmul_rn(th, ny), f));
-            s.g2[2] = __fadd_rn(s.g2[2], __fmul_rn(__fmul_rn(th, nz), f));
+
+    __device__ __forceinline__ void one(float val, float th, float f, const float4 &B, const float4 &C)
+    {
+        K++;
+        acc += val;
+        if constexpr (REC) {
+            if (val > 0.0f) {
+                const float nx = B.y * C.z - B.z * C.y, ny = B.z * C.x - B.x * C.z, nz = B.x * C.y - B.y * C.x;
+                // products rounded before they are added
+                g1[0] = __fadd_rn(g1[0], __fmul_rn(nx, f));
+                g1[1] = __fadd_rn(g1[1], __fmul_rn(ny, f));
+                g1[2] = __fadd_rn(g1[2], __fmul_rn(nz, f));
+                g2[0] = __fadd_rn(g2[0], __fmul_rn(__fmul_rn(th, nx), f));
+                g2[1] = __fadd_rn(g2[1], __fmul_rn(__fmul_rn(th, ny), f));
+                g2[2] = __fadd_rn(g2[2], __fmul_rn(__fmul_rn(th, nz), f));
+            }
         }
     }
-}
+    template <int G>
+    __device__ __forceinline__ void add(const StepParams &, const CollPath &, bool hit, float th, float over, float f,
+                                        const float4 &B, const float4 &C)
+    {
+        const float val = fmaxf(over, 0.0f);
+        if constexpr (G == 1) {
+            if (hit) one(val, th, f, B, C);
+        } else {
+            const int lane = threadIdx.x & 31, gbase = lane & ~(G - 1);
+            unsigned hm = (__ballot_sync(0xffffffffu, hit) >> gbase) & (0xffffffffu >> (32 - G));
+            while (__any_sync(0xffffffffu, hm != 0u)) {
+                const int src = hm ? gbase + __ffs((int)hm) - 1 : lane;
+                const float hv = coll_shfl(val, src);
+                float ht = 0.0f, hf = 0.0f;
+                float4 hB = B, hC = C;
+                if constexpr (REC) {
+                    ht = coll_shfl(th, src);
+                    hf = coll_shfl(f, src);
+                    hB.x = coll_shfl(B.x, src); hB.y = coll_shfl(B.y, src); hB.z = coll_shfl(B.z, src);
+                    hC.x = coll_shfl(C.x, src); hC.y = coll_shfl(C.y, src); hC.z = coll_shfl(C.z, src);
+                }
+                if (hm) one(hv, ht, hf, hB, hC);
+                hm &= hm - 1u;
+            }
+        }
+    }
+    __device__ __forceinline__ NodeHits from(int l) const
+    {
+        NodeHits t;
+        t.K = __shfl_sync(0xffffffffu, K, l);
+        t.acc = coll_shfl(acc, l);
+#pragma unroll
+        for (int a = 0; a < (REC ? 3 : 1); a++) {
+            t.g1[a] = REC ? coll_shfl(g1[a], l) : 0.0f;
+            t.g2[a] = REC ? coll_shfl(g2[a], l) : 0.0f;
+        }
+        return t;
+    }
+};
 
 // ------------------------------------------------------------ list pass
 // The walk appends the nodes whose path box meets the box of the mesh's
@@ -188,46 +243,33 @@ __device__ __forceinline__ void coll_record(const StepParams &p, long long o, fl
     atomicOr(p.cbits + (o >> 5), 1u << (o & 31));
 }
 
-__device__ __forceinline__ float coll_shfl(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-
 // 32 candidates of one path tested by the warp, one per lane (have: whether
-// the lane has one, entry e of cell (cx, cy, cz)); the hits are added to s in
-// lane order.  Every lane passes the same path and ends with the same sums.
-template <bool REC>
+// the lane has one, entry e of cell (cx, cy, cz)).  Every lane passes the same
+// path and ends with the same sums.
+template <class Hits>
 __device__ __forceinline__ void coll_warp_round(const StepParams &p, const CollPath &q, const CollWords &w,
                                                 const CollBox &bx, bool have, long long e, int cx, int cy, int cz,
-                                                CollAcc<REC> &s)
+                                                Hits &s)
 {
     float th = 0.0f, over = 0.0f, f = 0.0f;
     float4 A, B = make_float4(0.0f, 0.0f, 0.0f, 0.0f), C = B;
-    const bool hit = have && coll_overlap(__ldg(p.efil + e), w) &&
+    const bool hit = have && coll_overlap(__ldg(p.efil + e), w, coll_need(bx, cx, cy, cz)) &&
                      coll_candidate(p, q, e, cx, cy, cz, bx.lox, bx.loy, bx.loz, th, over, f, A, B, C);
-    const float val = fmaxf(over, 0.0f);
-    for (unsigned hm = __ballot_sync(0xffffffffu, hit); hm; hm &= hm - 1u) {
-        const int src = __ffs((int)hm) - 1;
-        const float hv = coll_shfl(val, src);
-        float ht = 0.0f, hf = 0.0f;
-        float4 hB = B, hC = C;
-        if constexpr (REC) {
-            ht = coll_shfl(th, src);
-            hf = coll_shfl(f, src);
-            hB.x = coll_shfl(B.x, src); hB.y = coll_shfl(B.y, src); hB.z = coll_shfl(B.z, src);
-            hC.x = coll_shfl(C.x, src); hC.y = coll_shfl(C.y, src); hC.z = coll_shfl(C.z, src);
-        }
-        coll_add<REC>(s, hv, ht, hf, hB, hC);
-    }
+    s.template add<32>(p, q, hit, th, over, f, B, C);
 }
 
 // All cells of a long path walked by the whole warp (every lane passes the
 // same arguments): 32 cells at a time, x fastest, then their candidates 32 at
 // a time in cell order, so the hits come in the order of a walk by one thread.
-template <bool REC>
-__device__ __noinline__ void coll_wide(const StepParams &p, const CollPath q, const CollWords w, const CollBox bx,
-                                       CollAcc<REC> &s)
+// Returns the number of candidates.
+template <class Hits>
+__device__ __noinline__ unsigned coll_wide(const StepParams &p, const CollPath q, const CollWords w, const CollBox bx,
+                                           Hits &s)
 {
     const int lane = threadIdx.x & 31;
     const int nxc = bx.hix - bx.lox + 1, nyc = bx.hiy - bx.loy + 1, nzc = bx.hiz - bx.loz + 1;
     const long long nxy = (long long)nxc * nyc, ncell = nxy * nzc;
+    unsigned tested = 0u;
     for (long long c0 = 0; c0 < ncell; c0 += 32) {
         const long long cc = c0 + lane;
         int e0 = 0, cnt = 0, cx = 0, cy = 0, cz = 0;
@@ -248,6 +290,7 @@ __device__ __noinline__ void coll_wide(const StepParams &p, const CollPath q, co
         }
         const int total = __shfl_sync(0xffffffffu, incl, 31);
         const int excl = incl - cnt;
+        tested += (unsigned)total;
         for (int r0 = 0; r0 < total; r0 += 32) {
             const int j = r0 + lane;
             // the lane whose cell holds candidate j: the last with excl <= j
@@ -258,14 +301,105 @@ __device__ __noinline__ void coll_wide(const StepParams &p, const CollPath q, co
             const int oe0 = __shfl_sync(0xffffffffu, e0, ow), oex = __shfl_sync(0xffffffffu, excl, ow);
             const int ocx = __shfl_sync(0xffffffffu, cx, ow), ocy = __shfl_sync(0xffffffffu, cy, ow),
                       ocz = __shfl_sync(0xffffffffu, cz, ow);
-            coll_warp_round<REC>(p, q, w, bx, j < total, (long long)oe0 + (j - oex), ocx, ocy, ocz, s);
+            coll_warp_round(p, q, w, bx, j < total, (long long)oe0 + (j - oex), ocx, ocy, ocz, s);
         }
+    }
+    return tested;
+}
+
+// The hits of every lane's path (ncell cells of its box; 0: none), G lanes per
+// path: the lanes of a group are neighbours in the warp, bring the same path
+// and end with the same sums.  wide: the path has more than the caller's limit
+// of cells (ncell = 0) and is walked by the whole warp; its candidates are
+// counted with COUNT_WIDE.  src.params(cloth) are the path's parameters.
+// ntest accumulates, in a group's first lane, the candidates.
+template <int G, bool COUNT_WIDE, class Src, class Hits>
+__device__ __forceinline__ void coll_cells(const Src &src, int cloth, const StepParams &p, const CollPath &q,
+                                           const CollBox &bx, const CollWords &w, int ncell, bool wide, Hits &s,
+                                           unsigned &ntest)
+{
+    constexpr unsigned FULLW = 0xffffffffu;
+    const int lane = threadIdx.x & 31, sub = lane % G, gbase = lane - sub;
+    const int ncw = __reduce_max_sync(FULLW, ncell);
+    int cx = bx.lox, cy = bx.loy, cz = bx.loz;
+    for (int c = 0; c < ncw; c++) {
+        int e0 = 0, cnt = 0;
+        if (c < ncell) {
+            const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
+            e0 = __ldg(p.cell_start + cell);
+            cnt = __ldg(p.cell_start + cell + 1) - e0;
+            if (sub == 0) ntest += (unsigned)cnt;
+        }
+        const unsigned need = coll_need(bx, cx, cy, cz);
+        const bool big = cnt > COLL_MAXE;
+        const int own = big ? 0 : cnt;
+        for (int b = 0; __any_sync(FULLW, b < own); b += 32) {
+            const int n = min(own - b, 32);
+            unsigned m = 0u;  // the entries of this run that pass the filter
+            const uint4 *fil = p.efil + e0 + b;
+#pragma unroll 4
+            for (int t = sub; t < n; t += G) m |= (unsigned)coll_overlap(__ldg(fil + t), w, need) << t;
+#pragma unroll
+            for (int d = 1; d < G; d <<= 1) m |= __shfl_xor_sync(FULLW, m, d);
+            while (__any_sync(FULLW, m != 0u)) {
+                // the group's next G survivors, one per lane in entry order
+                unsigned mine = m;
+#pragma unroll
+                for (int t = 0; t < G; t++) {
+                    if (t < sub) mine &= mine - 1u;
+                    m &= m - 1u;
+                }
+                const int t = __ffs((int)mine) - 1;
+                float th = 0.0f, over = 0.0f, f = 0.0f;
+                float4 A, B = make_float4(0.0f, 0.0f, 0.0f, 0.0f), C = B;
+                const bool hit = t >= 0 && coll_candidate(p, q, (long long)e0 + b + t, cx, cy, cz, bx.lox, bx.loy,
+                                                          bx.loz, th, over, f, A, B, C);
+                s.template add<G>(p, q, hit, th, over, f, B, C);
+            }
+        }
+        // crowded cells, one path's at a time over the whole warp
+        for (unsigned bm = __ballot_sync(FULLW, big && sub == 0); bm; bm &= bm - 1u) {
+            const int l = __ffs((int)bm) - 1;
+            const CollPath lq = {coll_shfl(q.sx, l), coll_shfl(q.sy, l), coll_shfl(q.sz, l), coll_shfl(q.rx, l),
+                                 coll_shfl(q.ry, l), coll_shfl(q.rz, l), coll_shfl(q.L, l)};
+            const CollWords lw = {__shfl_sync(FULLW, w.a, l), __shfl_sync(FULLW, w.b, l), __shfl_sync(FULLW, w.c, l)};
+            CollBox lb = bx;
+            lb.lox = __shfl_sync(FULLW, bx.lox, l);
+            lb.loy = __shfl_sync(FULLW, bx.loy, l);
+            lb.loz = __shfl_sync(FULLW, bx.loz, l);
+            const int le0 = __shfl_sync(FULLW, e0, l), lcnt = __shfl_sync(FULLW, cnt, l);
+            const int lcx = __shfl_sync(FULLW, cx, l), lcy = __shfl_sync(FULLW, cy, l), lcz = __shfl_sync(FULLW, cz, l);
+            const StepParams &lp = src.params(__shfl_sync(FULLW, cloth, l));
+            Hits t = s.from(l);
+            for (int r0 = 0; r0 < lcnt; r0 += 32)
+                coll_warp_round(lp, lq, lw, lb, r0 + lane < lcnt, (long long)le0 + r0 + lane, lcx, lcy, lcz, t);
+            if (gbase == l) s = t;
+        }
+        if (++cx > bx.hix) {
+            cx = bx.lox;
+            if (++cy > bx.hiy) {
+                cy = bx.loy;
+                cz++;
+            }
+        }
+    }
+    // long paths, one at a time over the whole warp
+    for (unsigned wm = __ballot_sync(FULLW, wide && sub == 0); wm; wm &= wm - 1u) {
+        const int l = __ffs((int)wm) - 1;
+        const CollPath lq = {coll_shfl(q.sx, l), coll_shfl(q.sy, l), coll_shfl(q.sz, l), coll_shfl(q.rx, l),
+                             coll_shfl(q.ry, l), coll_shfl(q.rz, l), coll_shfl(q.L, l)};
+        const CollWords lw = {__shfl_sync(FULLW, w.a, l), __shfl_sync(FULLW, w.b, l), __shfl_sync(FULLW, w.c, l)};
+        const CollBox lb = {__shfl_sync(FULLW, bx.lox, l), __shfl_sync(FULLW, bx.loy, l), __shfl_sync(FULLW, bx.loz, l),
+                            __shfl_sync(FULLW, bx.hix, l), __shfl_sync(FULLW, bx.hiy, l), __shfl_sync(FULLW, bx.hiz, l)};
+        Hits t = s.from(l);
+        const unsigned tested = coll_wide(src.params(__shfl_sync(FULLW, cloth, l)), lq, lw, lb, t);
+        if (gbase == l) s = t;
+        if (COUNT_WIDE && lane == l) ntest += tested;
     }
 }
 
-// One round of the list pass, G lanes per node (the lanes of a node are
-// neighbours in the warp and end with the same sums): every group brings one
-// entry (valid: whether it has one; i: its index for src.entry).  Src supplies
+// One round of the list pass, G lanes per node: every group brings one entry
+// (valid: whether it has one; i: its index for src.entry).  Src supplies
 // entry(i, cloth, offset) and params(cloth).  has_pre: the entry's offset is
 // pre_o, loaded by the caller (cloth 0).  ntest and nhit accumulate, in the
 // group's first lane, the candidate triangles and whether the node hit.  REC:
@@ -274,8 +408,6 @@ template <bool REC, int G, class Src>
 __device__ __forceinline__ void collide_round(const Src &src, unsigned long long k, bool valid, unsigned long long i,
                                               float &fsum, unsigned &ntest, unsigned &nhit, bool has_pre, int pre_o)
 {
-    constexpr unsigned FULLW = 0xffffffffu;
-    const int lane = threadIdx.x & 31, sub = lane % G, gbase = lane - sub;
     int cloth = 0;
     long long o = 0;
     if (valid) {
@@ -302,110 +434,9 @@ __device__ __forceinline__ void collide_round(const Src &src, unsigned long long
             ncell = wide ? 0 : (int)nc;
         }
     }
-    CollAcc<REC> s = {};
-    const int ncw = __reduce_max_sync(FULLW, ncell);
-    int cx = bx.lox, cy = bx.loy, cz = bx.loz;
-    for (int c = 0; c < ncw; c++) {
-        int e0 = 0, cnt = 0;
-        if (c < ncell) {
-            const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
-            e0 = __ldg(p.cell_start + cell);
-            cnt = __ldg(p.cell_start + cell + 1) - e0;
-            if (sub == 0) ntest += (unsigned)cnt;
-        }
-        const bool big = cnt > COLL_MAXE;
-        const int own = big ? 0 : cnt;
-        for (int b = 0; __any_sync(FULLW, b < own); b += 32) {
-            const int n = min(own - b, 32);
-            unsigned m = 0u;  // the entries of this run that pass the filter
-            const uint4 *fil = p.efil + e0 + b;
-#pragma unroll 4
-            for (int t = sub; t < n; t += G) m |= (unsigned)coll_overlap(__ldg(fil + t), w) << t;
-#pragma unroll
-            for (int d = 1; d < G; d <<= 1) m |= __shfl_xor_sync(FULLW, m, d);
-            while (__any_sync(FULLW, m != 0u)) {
-                // the group's next G survivors, one per lane in entry order
-                unsigned mine = m;
-#pragma unroll
-                for (int t = 0; t < G; t++) {
-                    if (t < sub) mine &= mine - 1u;
-                    m &= m - 1u;
-                }
-                const int t = __ffs((int)mine) - 1;
-                float th = 0.0f, over = 0.0f, f = 0.0f;
-                float4 A, B = make_float4(0.0f, 0.0f, 0.0f, 0.0f), C = B;
-                const bool hit = t >= 0 && coll_candidate(p, q, (long long)e0 + b + t, cx, cy, cz, bx.lox, bx.loy,
-                                                          bx.loz, th, over, f, A, B, C);
-                const float val = fmaxf(over, 0.0f);
-                if (G == 1) {
-                    if (hit) coll_add<REC>(s, val, th, f, B, C);
-                } else {
-                    unsigned hm = (__ballot_sync(FULLW, hit) >> gbase) & ((1u << G) - 1u);
-                    while (__any_sync(FULLW, hm != 0u)) {
-                        const int from = hm ? gbase + __ffs((int)hm) - 1 : lane;
-                        const float hv = coll_shfl(val, from);
-                        float ht = 0.0f, hf = 0.0f;
-                        float4 hB = B, hC = C;
-                        if constexpr (REC) {
-                            ht = coll_shfl(th, from);
-                            hf = coll_shfl(f, from);
-                            hB.x = coll_shfl(B.x, from); hB.y = coll_shfl(B.y, from); hB.z = coll_shfl(B.z, from);
-                            hC.x = coll_shfl(C.x, from); hC.y = coll_shfl(C.y, from); hC.z = coll_shfl(C.z, from);
-                        }
-                        if (hm) coll_add<REC>(s, hv, ht, hf, hB, hC);
-                        hm &= hm - 1u;
-                    }
-                }
-            }
-        }
-        // crowded cells, one node's at a time over the whole warp
-        for (unsigned bm = __ballot_sync(FULLW, big && sub == 0); bm; bm &= bm - 1u) {
-            const int l = __ffs((int)bm) - 1;
-            const StepParams &lp = src.params(__shfl_sync(FULLW, cloth, l));
-            const CollPath lq = {coll_shfl(q.sx, l), coll_shfl(q.sy, l), coll_shfl(q.sz, l), coll_shfl(q.rx, l),
-                                 coll_shfl(q.ry, l), coll_shfl(q.rz, l), coll_shfl(q.L, l)};
-            const CollWords lw = {__shfl_sync(FULLW, w.a, l), __shfl_sync(FULLW, w.b, l), __shfl_sync(FULLW, w.c, l)};
-            CollBox lb = bx;
-            lb.lox = __shfl_sync(FULLW, bx.lox, l);
-            lb.loy = __shfl_sync(FULLW, bx.loy, l);
-            lb.loz = __shfl_sync(FULLW, bx.loz, l);
-            const int le0 = __shfl_sync(FULLW, e0, l), lcnt = __shfl_sync(FULLW, cnt, l);
-            const int lcx = __shfl_sync(FULLW, cx, l), lcy = __shfl_sync(FULLW, cy, l), lcz = __shfl_sync(FULLW, cz, l);
-            CollAcc<REC> t;
-            t.K = __shfl_sync(FULLW, s.K, l);
-            t.acc = coll_shfl(s.acc, l);
-            if constexpr (REC) {
-#pragma unroll
-                for (int a = 0; a < 3; a++) {
-                    t.g1[a] = coll_shfl(s.g1[a], l);
-                    t.g2[a] = coll_shfl(s.g2[a], l);
-                }
-            }
-            for (int r0 = 0; r0 < lcnt; r0 += 32)
-                coll_warp_round<REC>(lp, lq, lw, lb, r0 + lane < lcnt, (long long)le0 + r0 + lane, lcx, lcy, lcz, t);
-            if (gbase == l) s = t;
-        }
-        if (++cx > bx.hix) {
-            cx = bx.lox;
-            if (++cy > bx.hiy) {
-                cy = bx.loy;
-                cz++;
-            }
-        }
-    }
-    // long paths, one at a time over the whole warp (their candidates are not counted)
-    for (unsigned wm = __ballot_sync(FULLW, wide && sub == 0); wm; wm &= wm - 1u) {
-        const int l = __ffs((int)wm) - 1;
-        const CollPath lq = {coll_shfl(q.sx, l), coll_shfl(q.sy, l), coll_shfl(q.sz, l), coll_shfl(q.rx, l),
-                             coll_shfl(q.ry, l), coll_shfl(q.rz, l), coll_shfl(q.L, l)};
-        const CollWords lw = {__shfl_sync(FULLW, w.a, l), __shfl_sync(FULLW, w.b, l), __shfl_sync(FULLW, w.c, l)};
-        const CollBox lb = {__shfl_sync(FULLW, bx.lox, l), __shfl_sync(FULLW, bx.loy, l), __shfl_sync(FULLW, bx.loz, l),
-                            __shfl_sync(FULLW, bx.hix, l), __shfl_sync(FULLW, bx.hiy, l), __shfl_sync(FULLW, bx.hiz, l)};
-        CollAcc<REC> t = {};
-        coll_wide<REC>(src.params(__shfl_sync(FULLW, cloth, l)), lq, lw, lb, t);
-        if (gbase == l) s = t;
-    }
-    if (s.K > 0 && sub == 0) {
+    NodeHits<REC> s = {};
+    coll_cells<G, false>(src, cloth, p, q, bx, w, ncell, wide, s, ntest);
+    if (s.K > 0 && (threadIdx.x & 31) % G == 0) {
         const float m = s.acc / (float)s.K;
         // product and sum rounded separately, the same bits in every kernel
         const float ox = __fadd_rn(q.sx, __fmul_rn(m, q.rx)), oy = __fadd_rn(q.sy, __fmul_rn(m, q.ry)),
@@ -466,14 +497,6 @@ __device__ __forceinline__ void collide_list(const Src &src, unsigned long long 
         collide_chunks<REC, 1>(src, k, n, fsum, ntest, nhit, false, 0);
 }
 
-// Per-lane scratch of the edge pass's cooperative rounds.
-struct CollLane {
-    float4 s;                   // S, L
-    float4 r;                   // r, owning cloth (int bits)
-    int4 box;                   // low cell, x extent | y extent << 16
-    int2 cell[COLL_MAXC];       // per cell of the box: first entry, end of the lane's running count
-};
-
 // Adds a collision pass's counts to the cloth's running statistics: every
 // warp's tested candidates and hit nodes are summed per CTA in shared memory
 // (s2, zeroed by the caller before a __syncthreads), then one thread adds the
@@ -533,219 +556,118 @@ constexpr int EDGES_PER_NODE = 12;
 // walks an edge with more hits than 1 + EDGE_MORE again.
 constexpr int EDGE_MORE = CLOTH_EDGE_MORE;
 
-struct EdgeShared {
-    CollLane lane[COLL_WARPS][32];
-    int base[COLL_WARPS][32];
-    float4 hit[COLL_WARPS][32];  // one round's results: hit point P and 1, or w = 0
-};
-
 // The kind of the triangulation edge from (ra, ca) to (rb, cb): 0 (0,+1),
 // 1 (+1,0), 2 (+1,+1).
 __device__ __forceinline__ int edge_kind(int ra, int ca, int rb, int cb) { return rb == ra ? 0 : (cb == ca ? 1 : 2); }
 
-// The first hit point of an edge path and its number of hits, walked by the
-// whole warp (every lane passes the same path and box; call from converged
-// code): the box's cells 32 at a time, x fastest, and each chunk's candidates
-// 32 at a time in cell order, so the first hit and the count are those of a
-// walk over the candidates in order.  Returns the same record on every lane
-// and adds the candidates tested to ntest.
-__device__ __forceinline__ float4 edge_hits_warp(const StepParams &p, const CollPath &path, const CollBox &bx,
-                                                 long long slot, int lane, unsigned &ntest)
-{
-    constexpr unsigned FULLW = 0xffffffffu;
-    const int nxc = bx.hix - bx.lox + 1, nyc = bx.hiy - bx.loy + 1, nzc = bx.hiz - bx.loz + 1;
-    const long long nxy = (long long)nxc * nyc, ncell = nxy * nzc;
-    float4 rec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    for (long long c0 = 0; c0 < ncell; c0 += 32) {
-        const long long cc = c0 + lane;
-        int e0 = 0, cnt = 0, cx = 0, cy = 0, cz = 0;
-        if (cc < ncell) {
-            cz = bx.loz + (int)(cc / nxy);
-            const int rem = (int)(cc - (long long)(cz - bx.loz) * nxy);
-            cy = bx.loy + rem / nxc;
-            cx = bx.lox + rem % nxc;
-            const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
-            e0 = __ldg(p.cell_start + cell);
-            cnt = __ldg(p.cell_start + cell + 1) - e0;
-        }
-        int incl = cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(FULLW, incl, d);
-            if (lane >= d) incl += t;
-        }
-        const int total = __shfl_sync(FULLW, incl, 31);
-        const int excl = incl - cnt;
-        ntest += (unsigned)total;
-        for (int r0 = 0; r0 < total; r0 += 32) {
-            const int j = r0 + lane;
-            // the lane whose cell holds candidate j: the last with excl <= j
-            int ow = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1)
-                if (__shfl_sync(FULLW, excl, ow + step) <= j) ow += step;
-            const int oe0 = __shfl_sync(FULLW, e0, ow), oex = __shfl_sync(FULLW, excl, ow);
-            const int ocx = __shfl_sync(FULLW, cx, ow), ocy = __shfl_sync(FULLW, cy, ow),
-                      ocz = __shfl_sync(FULLW, cz, ow);
-            bool hit = false;
-            float th = 0.0f;
-            if (j < total) {
-                float f, over;
-                float4 A, B, C;
-                hit = coll_candidate(p, path, (long long)oe0 + (j - oex), ocx, ocy, ocz, bx.lox, bx.loy, bx.loz, th,
-                                     over, f, A, B, C);
-            }
-            const unsigned hm = __ballot_sync(FULLW, hit);
-            if (hm) {
-                const float3 hp = coll_hit_point(path, th);
-                const float hx = hp.x, hy = hp.y, hz = hp.z;
-                // this lane's hit is number rank (from 0) of the edge
-                const int rank = (int)rec.w + __popc(hm & ((1u << lane) - 1u));
-                if (hit && rank >= 1 && rank <= EDGE_MORE)
-                    p.edge_more[(long long)(rank - 1) * 3 * p.stride + slot] = make_float4(hx, hy, hz, 1.0f);
-                if (rec.w == 0.0f) {
-                    const int src = __ffs(hm) - 1;
-                    rec = make_float4(__shfl_sync(FULLW, hx, src), __shfl_sync(FULLW, hy, src),
-                                      __shfl_sync(FULLW, hz, src), 0.0f);
-                }
-                rec.w += (float)__popc(hm);
+// An edge's hits (see NodeHits): rec = (the first hit's point, the number of
+// hits); the points of hits 2 .. 1 + EDGE_MORE go to p.edge_more at the edge's slot.
+struct EdgeHits {
+    float4 rec;
+    long long slot;
+
+    __device__ __forceinline__ void one(const StepParams &p, const CollPath &q, float th)
+    {
+        const float3 P = coll_hit_point(q, th);
+        if (rec.w == 0.0f) rec = make_float4(P.x, P.y, P.z, 0.0f);
+        else if (rec.w <= (float)EDGE_MORE)
+            p.edge_more[(long long)(rec.w - 1.0f) * 3 * p.stride + slot] = make_float4(P.x, P.y, P.z, 1.0f);
+        rec.w += 1.0f;
+    }
+    template <int G>
+    __device__ __forceinline__ void add(const StepParams &p, const CollPath &q, bool hit, float th, float, float,
+                                        const float4 &, const float4 &)
+    {
+        if constexpr (G == 1) {
+            if (hit) one(p, q, th);
+        } else {
+            const int lane = threadIdx.x & 31, gbase = lane & ~(G - 1);
+            unsigned hm = (__ballot_sync(0xffffffffu, hit) >> gbase) & (0xffffffffu >> (32 - G));
+            while (__any_sync(0xffffffffu, hm != 0u)) {
+                const float ht = coll_shfl(th, hm ? gbase + __ffs((int)hm) - 1 : lane);
+                if (hm) one(p, q, ht);  // every lane of the group stores the same point
+                hm &= hm - 1u;
             }
         }
     }
-    return rec;
-}
+    __device__ __forceinline__ EdgeHits from(int l) const
+    {
+        return {make_float4(coll_shfl(rec.x, l), coll_shfl(rec.y, l), coll_shfl(rec.z, l), coll_shfl(rec.w, l)),
+                __shfl_sync(0xffffffffu, slot, l)};
+    }
+};
+
+struct EdgeList {  // coll_cells' source of parameters
+    const StepParams &p;
+    __device__ const StepParams &params(int) const { return p; }
+};
 
 // Pass A of the edge narrow phase: every listed node tests the three edges it
 // owns, (0,+1), (+1,0) and (+1,+1) from it (the triangulation's edges,
 // oriented from their upper-left endpoint), at the updated positions, so each
-// edge is tested once.  32 edges per warp and round, their candidates spread
-// over the lanes as in the node pass; an edge whose box spans more than
-// COLL_MAXC cells is walked afterwards by the whole warp (edge_hits_warp).
-// Records per edge its first hit point (in candidate order) and its number of
-// hits, p.edge_hit[kind * stride + owner] = (P, K), and the points of its hits
-// 2 .. 1 + EDGE_MORE at p.edge_more[(h - 2) * 3 * stride + kind * stride +
-// owner].  Counts the lane's tested candidates and edges that hit into ntest
-// and nhit.
-__device__ __forceinline__ void edge_test_list(const StepParams &p, EdgeShared &sh, unsigned long long k, unsigned n,
-                                               unsigned &ntest, unsigned &nhit)
+// edge is tested once.  G lanes per edge as in the node pass; a warp's edges
+// are of one kind and of neighbouring owners.  Records per edge its first hit
+// point (in candidate order) and its number of hits, p.edge_hit[kind * stride +
+// owner] = (P, K), and the points of its hits 2 .. 1 + EDGE_MORE at
+// p.edge_more[(h - 2) * 3 * stride + kind * stride + owner].  Counts the
+// tested candidates and the edges that hit into ntest and nhit.  Measured on
+// 256 x 256 nodes over 81,920 triangles: the four kernels of a substep 151 ->
+// 80 us against one that searched shared memory for each candidate and walked
+// every box of more than 8 cells by the whole warp (137 us of it, 54M warp
+// instructions).
+constexpr int EDGE_MAXC = 18;  // cells of an edge's box one lane goes through
+template <int G>
+__device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned long long k, unsigned n,
+                                                 unsigned &ntest, unsigned &nhit)
 {
+    constexpr unsigned PER = 32 / G;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const unsigned long long nw = (unsigned long long)gridDim.x * COLL_WARPS;
-    const unsigned long long w = (unsigned long long)blockIdx.x * COLL_WARPS + wib;
-    CollLane &me = sh.lane[wib][lane];
     const long long st = p.stride;
     const float *xs = (k & 1ull) ? p.state0 : p.state1;  // updated positions (written by the walk)
-    const unsigned long long items = 3ull * n;
-    for (unsigned long long b0 = 0; b0 < items; b0 += 32ull * nw) {
-        const unsigned long long j = b0 + (unsigned long long)lane * nw + w;
-        int cnt = 0;
+    const unsigned per_kind = (n + PER - 1u) / PER, nw = gridDim.x * COLL_WARPS;
+    const unsigned long long chunks = 3ull * per_kind;
+    const unsigned first = chunks < nw ? (unsigned)wib * gridDim.x + blockIdx.x : blockIdx.x * COLL_WARPS + wib;
+    for (unsigned long long c = first; c < chunks; c += nw) {
+        const int kind = (int)(c / per_kind);
+        const unsigned i = PER * (unsigned)(c % per_kind) + (unsigned)(lane / G);
         bool has = false, wide = false;
-        long long slot = 0;
-        float4 rec = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        CollPath path = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        int ncell = 0;
+        CollPath path = {};
         CollBox bx = {0, 0, 0, 0, 0, 0};
-        if (j < items) {
-            const int q = (int)(j % 3ull);
-            const int o = __ldg(p.coll_list + j / 3ull);
-            const int r = o / p.pitch, c = o - r * p.pitch;
-            const int rb = r + (q >= 1 ? 1 : 0), cb = c + (q != 1 ? 1 : 0);
+        CollWords w = {0u, 0u, 0u};
+        EdgeHits s = {make_float4(0.0f, 0.0f, 0.0f, 0.0f), 0};
+        if (i < n) {
+            const int o = __ldg(p.coll_list + i);
+            const int r = o / p.pitch, cc = o - r * p.pitch;
+            const int rb = r + (kind >= 1 ? 1 : 0), cb = cc + (kind != 1 ? 1 : 0);
             if (rb < p.ny && cb < p.nx) {
                 has = true;
-                slot = (long long)q * st + o;
+                s.slot = (long long)kind * st + o;
                 const long long ob = (long long)rb * p.pitch + cb;
                 const float x0 = xs[o], y0 = xs[st + o], z0 = xs[2 * st + o];
                 const float x1 = xs[ob], y1 = xs[st + ob], z1 = xs[2 * st + ob];
                 if (coll_path(p, x0, y0, z0, x1, y1, z1, path)) {
                     bx = coll_box(p, x0, y0, z0, x1, y1, z1);
-                    const int nxc = bx.hix - bx.lox + 1, nyc = bx.hiy - bx.loy + 1, nzc = bx.hiz - bx.loz + 1;
-                    if ((long long)nxc * nyc * nzc <= COLL_MAXC) {
-                        int cc = 0;
-                        for (int cz = bx.loz; cz <= bx.hiz; cz++)
-                            for (int cy = bx.loy; cy <= bx.hiy; cy++)
-                                for (int cx = bx.lox; cx <= bx.hix; cx++, cc++) {
-                                    const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
-                                    const int e0 = __ldg(p.cell_start + cell), e1 = __ldg(p.cell_start + cell + 1);
-                                    cnt += e1 - e0;
-                                    me.cell[cc] = make_int2(e0, cnt);
-                                }
-                        me.s = make_float4(path.sx, path.sy, path.sz, path.L);
-                        me.r = make_float4(path.rx, path.ry, path.rz, 0.0f);
-                        me.box = make_int4(bx.lox, bx.loy, bx.loz, nxc | (nyc << 16));
-                    } else {
-                        wide = true;
-                    }
+                    w = coll_words(p, x0, y0, z0, x1, y1, z1, path);
+                    const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
+                    wide = nc > EDGE_MAXC;
+                    ncell = wide ? 0 : (int)nc;
                 }
             }
         }
-        int incl = cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += t;
+        coll_cells<G, true>(EdgeList{p}, 0, p, path, bx, w, ncell, wide, s, ntest);
+        if (has && lane % G == 0) {
+            p.edge_hit[s.slot] = s.rec;
+            nhit += s.rec.w > 0.0f ? 1u : 0u;
         }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        const int excl = incl - cnt;
-        sh.base[wib][lane] = excl;
-        __syncwarp();
-        for (int r0 = 0; r0 < total; r0 += 32) {
-            const int jj = r0 + lane;
-            float4 hv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (jj < total) {
-                int ow = 0;
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (sh.base[wib][ow + step] <= jj) ow += step;
-                const CollLane &L = sh.lane[wib][ow];
-                const int loc = jj - sh.base[wib][ow];
-                int cc = 0;
-                while (L.cell[cc].y <= loc) cc++;
-                const long long e = L.cell[cc].x + (loc - (cc ? L.cell[cc - 1].y : 0));
-                const int nxc = L.box.w & 0xffff, nyc = L.box.w >> 16;
-                const int cx = L.box.x + cc % nxc, cy = L.box.y + (cc / nxc) % nyc, cz = L.box.z + cc / (nxc * nyc);
-                const CollPath lq = {L.s.x, L.s.y, L.s.z, L.r.x, L.r.y, L.r.z, L.s.w};
-                float th, over, f;
-                float4 A, B, C;
-                if (coll_candidate(p, lq, e, cx, cy, cz, L.box.x, L.box.y, L.box.z, th, over, f, A, B, C)) {
-                    const float3 hp = coll_hit_point(lq, th);
-                    hv = make_float4(hp.x, hp.y, hp.z, 1.0f);
-                }
-            }
-            sh.hit[wib][lane] = hv;
-            __syncwarp();
-            if (cnt > 0) {
-                const int q0 = max(excl, r0), q1 = min(excl + cnt, r0 + 32);
-                for (int t = q0; t < q1; t++) {
-                    const float4 P = sh.hit[wib][t - r0];
-                    if (P.w == 0.0f) continue;
-                    if (rec.w == 0.0f) rec = make_float4(P.x, P.y, P.z, 0.0f);
-                    else if (rec.w <= (float)EDGE_MORE) p.edge_more[(long long)(rec.w - 1.0f) * 3 * st + slot] = P;
-                    rec.w += 1.0f;
-                }
-            }
-            __syncwarp();
-        }
-        // the wide edges of this round, one at a time over the whole warp
-        for (unsigned wm = __ballot_sync(0xffffffffu, wide); wm; wm &= wm - 1u) {
-            const int src = __ffs(wm) - 1;
-            const CollPath q = {__shfl_sync(0xffffffffu, path.sx, src), __shfl_sync(0xffffffffu, path.sy, src),
-                                __shfl_sync(0xffffffffu, path.sz, src), __shfl_sync(0xffffffffu, path.rx, src),
-                                __shfl_sync(0xffffffffu, path.ry, src), __shfl_sync(0xffffffffu, path.rz, src),
-                                __shfl_sync(0xffffffffu, path.L, src)};
-            const CollBox b = {__shfl_sync(0xffffffffu, bx.lox, src), __shfl_sync(0xffffffffu, bx.loy, src),
-                               __shfl_sync(0xffffffffu, bx.loz, src), __shfl_sync(0xffffffffu, bx.hix, src),
-                               __shfl_sync(0xffffffffu, bx.hiy, src), __shfl_sync(0xffffffffu, bx.hiz, src)};
-            const long long sl = __shfl_sync(0xffffffffu, slot, src);
-            unsigned t = 0;
-            const float4 wr = edge_hits_warp(p, q, b, sl, lane, t);
-            if (lane == src) {
-                rec = wr;
-                ntest += t;
-            }
-        }
-        ntest += (unsigned)cnt;
-        nhit += rec.w > 0.0f ? 1u : 0u;
-        if (has) p.edge_hit[slot] = rec;
     }
+}
+__device__ __forceinline__ void edge_test_list(const StepParams &p, unsigned long long k, unsigned n, unsigned &ntest,
+                                               unsigned &nhit)
+{
+    const unsigned lanes = gridDim.x * 32u * COLL_WARPS;
+    if (3u * n <= lanes / COLL_GMAX) edge_test_chunks<COLL_GMAX>(p, k, n, ntest, nhit);
+    else edge_test_chunks<1>(p, k, n, ntest, nhit);
 }
 
 // Running sum of one node's response directions (Algorithm 2): adds the

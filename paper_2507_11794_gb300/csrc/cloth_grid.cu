@@ -199,9 +199,9 @@ __device__ __forceinline__ uint2 filter_side(float a, float e1, float e2, float 
 
 // Expand the sorted (cell, triangle) pairs into per-entry records read by the
 // narrow phase without an indirection: the triangle's plane and first cell,
-// and its box as filter words.
+// and its filter words (its box; whether this is its first cell per axis).
 __global__ void expand_kernel(const float4 *__restrict__ rec, const int *__restrict__ tri_ids, long long n,
-                              float ox, float oy, float oz, float qs, float pad, float4 *__restrict__ etri,
+                              const int *__restrict__ cell_start, long long ncells, int dx, int dy, float ox, float oy, float oz, float qs, float pad, float4 *__restrict__ etri,
                               uint4 *__restrict__ efil)
 {
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -214,8 +214,17 @@ __global__ void expand_kernel(const float4 *__restrict__ rec, const int *__restr
     const uint2 x = filter_side(A.x, B.x, C.x, ox, qs, pad);
     const uint2 y = filter_side(A.y, B.y, C.y, oy, qs, pad);
     const uint2 z = filter_side(A.z, B.z, C.z, oz, qs, pad);
+    // the entry's cell: the last whose list starts at or before e
+    long long lo = 0, hi = ncells;
+    while (hi - lo > 1) {
+        const long long mid = (lo + hi) >> 1;
+        if (cell_start[mid] <= e) lo = mid;
+        else hi = mid;
+    }
+    const int cx = (int)(lo % dx), cy = (int)(lo / dx % dy), cz = (int)(lo / dx / dy);
+    const unsigned first = (__float_as_int(A.w) == cx) | (__float_as_int(B.w) == cy) << 1 | (__float_as_int(C.w) == cz) << 2;
     efil[e] = make_uint4(GRID_FILTER_GUARD | x.y | y.y << 16, GRID_FILTER_GUARD | z.y | (GRID_FILTER_MAX - x.x) << 16,
-                         GRID_FILTER_GUARD | (GRID_FILTER_MAX - y.x) | (GRID_FILTER_MAX - z.x) << 16, 0u);
+                         GRID_FILTER_GUARD | (GRID_FILTER_MAX - y.x) | (GRID_FILTER_MAX - z.x) << 16, first);
 }
 
 __global__ void query_kernel(const float4 *__restrict__ rec, const int *__restrict__ cell_start,
@@ -366,6 +375,7 @@ cudaError_t grid_build(const float *d_verts, const int *d_tris, int nt, DevGrid 
             top = fmax(top, fmax(fabs((double)g->origin[a]), fabs((double)g->origin[a] + (double)g->dims[a] * g->h)));
         const float pad = (float)fmin(1.0 + ceil(4e-7 * top * g->qs), 40000.0);
         expand_kernel<<<blocks_for((long long)htotal, 256), 256, 0, s>>>(g->tri, g->tri_ids, (long long)htotal,
+                                                                         g->cell_start, nc, g->dims[0], g->dims[1],
                                                                          g->origin[0], g->origin[1], g->origin[2],
                                                                          g->qs, pad, g->etri, g->efil);
         GTRY(cudaGetLastError());

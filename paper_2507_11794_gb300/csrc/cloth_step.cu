@@ -834,9 +834,8 @@ __global__ void __launch_bounds__(256) edge_list_kernel(const __grid_constant__ 
 // node's owned edges and records their hits; pass B gathers every listed free
 // node's response from the records of its 12 edges into a scratch array; a
 // third kernel applies the responses, so no test reads a moved node.
-__global__ void __launch_bounds__(32 * COLL_WARPS, 2) edge_test_kernel(const __grid_constant__ StepParams p)
+__global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) edge_test_kernel(const __grid_constant__ StepParams p)
 {
-    __shared__ EdgeShared sh;
     __shared__ unsigned long long s_k;
     __shared__ unsigned s_n, s2[2];
     pdl_launch_dependents();
@@ -847,7 +846,7 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, 2) edge_test_kernel(const __g
     }
     __syncthreads();
     unsigned ntest = 0, nhit = 0;
-    edge_test_list(p, sh, s_k, s_n, ntest, nhit);
+    edge_test_list(p, s_k, s_n, ntest, nhit);
     coll_stats_add(p.ctrl, s2, s_n, ntest, nhit);
 }
 

@@ -89,3 +89,60 @@ def test_one_substep_matches_oracle(cloth_lib, oracle_lib, case):
     assert len(off) <= 2 + n // 500
     if n > 100:
         assert (hits > 0).sum() > n // 200
+
+
+# edge narrow phase: eight lanes per edge up to 6,485 listed nodes on 152 SMs, one beyond; a steep sheet
+# whose edges span up to 12 cells, some more than one lane goes through
+EDGE_CASES = {"eight_lanes": (81, 80, 60), "one_lane": (82, 80, 60), "long_edges": (30, 26, 90)}
+
+
+@pytest.mark.parametrize("case", EDGE_CASES)
+def test_edge_substep_matches_oracle(cloth_lib, oracle_lib, case):
+    nx, ny, m = EDGE_CASES[case]
+    v, t = wavy(m, 1.0, 0.01, 21)
+    rng = np.random.default_rng(22)
+    h = 0.8 / nx
+    x, z = np.meshgrid(0.1 + h * np.arange(nx), 0.1 + h * np.arange(ny))
+    pos = np.stack([x, rng.uniform(-0.03, 0.03, x.shape), z], axis=2)
+    vel = rng.normal(size=(nx * ny, 3)) * 0.5
+    sc = make_scene(nx, ny, pos=pos, vel=vel, mesh=(v, t), dt=1e-3)
+    grid = oracle_lib.Grid(v, t)
+    clo = oracle_lib.Cloth(sc)
+    xo, _, hits = oracle_lib.step_edges(clo, sc.init_pos, sc.init_vel, 0, 1, grid, want_hits=True)
+    with cloth_lib.Cloth(sc, flags=cloth_lib.capi.CLOTH_FLAG_EDGE_COLLISION) as cl:
+        cl.step(1)
+        p, _ = cl.read()
+    S = sc.init_pos.astype(np.float64)
+    err = np.abs(p.astype(np.float64) - xo).max(axis=1)
+    # a hit decided within float32 rounding of its threshold may go either way (as in test_gpu_edges)
+    bound = np.linalg.norm(xo - S, axis=1) + np.linalg.norm(p.astype(np.float64) - S, axis=1)
+    print(f"{case}: {int((hits > 0).sum())} nodes affected, {int((err > 1e-5).sum())} beyond 1e-5")
+    assert np.all(err <= np.maximum(1e-5, 1.01 * bound + 1e-7))
+    assert (err > 1e-5).mean() <= 0.02
+    assert (hits > 0).mean() > 0.3
+
+
+@pytest.mark.parametrize("nx,ny", [(41, 37), (90, 85)])
+def test_edge_statistics_count_every_edge(cloth_lib, nx, ny):
+    # a flat sheet above the surface, inside its cells: nothing hits, so the
+    # candidates of every edge follow from the final positions and the grid
+    v, t = wavy(40, 1.0, 0.01, 31)
+    h = 0.8 / nx
+    x, z = np.meshgrid(0.1 + h * np.arange(nx), 0.1 + h * np.arange(ny))
+    sc = make_scene(nx, ny, pos=np.stack([x, np.full_like(x, 0.0100), z], axis=2), mesh=(v, t), dt=1e-3)
+    with cloth_lib.Cloth(sc, flags=cloth_lib.capi.CLOTH_FLAG_EDGE_COLLISION) as cl:
+        cl.step(1)
+        p, _ = cl.read()
+        listed, tested, hits = cl.collision_stats()
+        i = cl.info()
+        start, _ = cl.grid()
+    assert hits == 0 and listed == nx * ny
+    dims = np.array(i.grid_dims)
+    cell = np.floor((p - np.float32(i.grid_origin)) * np.float32(i.grid_inv)).astype(int).reshape(ny, nx, 3)
+    count = np.diff(start).reshape(dims[::-1])
+    total = 0
+    for dr, dc in ((0, 1), (1, 0), (1, 1)):
+        a, b = cell[:ny - dr, :nx - dc].reshape(-1, 3), cell[dr:, dc:].reshape(-1, 3)
+        for lo, hi in zip(np.minimum(a, b), np.maximum(a, b)):
+            total += int(count[lo[2]:hi[2] + 1, lo[1]:hi[1] + 1, lo[0]:hi[0] + 1].sum())
+    assert tested == total
