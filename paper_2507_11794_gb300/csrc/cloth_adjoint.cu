@@ -392,7 +392,11 @@ cudaError_t enqueue_forward(ClothRollout *ro, cudaStream_t s)
     for (int g = 0; g < ro->nseg && e == cudaSuccess; g++) {
         e = copy_planes(cur_state(h, ro->kseg[g]), ro->ckpt + (size_t)g * 6 * st, 6 * st, s);
         const int n = seg_steps(ro, g) * h->desc.substeps;
-        for (int q = 0; q < n && e == cudaSuccess; q++) e = launch_substep(h->params, s);
+        for (int q = 0; q < n && e == cudaSuccess; q++) {
+            StepParams p = h->params;
+            p.parity = (int)((ro->kseg[g] + (unsigned long long)q) & 1ull);
+            e = launch_substep(p, s);
+        }
     }
     if (e == cudaSuccess) e = copy_planes(cur_state(h, ro->k_final), ro->final_state, 6 * st, s);
     return e;
@@ -432,7 +436,8 @@ cudaError_t recompute_segment(ClothRollout *ro, int g, cudaStream_t s)
         float *in = j == 0 ? const_cast<float *>(ck) : seg_slot(ro, b, j);
         float *out = seg_slot(ro, b, j + 1);
         // the kernels read (k odd ? state1 : state0) and write the other
-        if ((kg + (unsigned long long)j) & 1ull) {
+        q.parity = (int)((kg + (unsigned long long)j) & 1ull);
+        if (q.parity) {
             q.state1 = in;
             q.state0 = out;
         } else {

@@ -124,7 +124,7 @@ void cloth_fill_params(ClothHandle *h)
     p.rows_per_warp = substep_rows_per_warp(d.nx, d.ny, h->sm_count);
     substep_shape(p);
     p.stride = h->stride;
-    p.parity = -1;
+    p.parity = 0;
     p.state0 = h->state;
     p.state1 = h->state + 6 * h->stride;
     p.pin_bits = h->pin_bits;
@@ -201,6 +201,7 @@ void cloth_fill_params(ClothHandle *h)
     p.coll_count = h->ctrl ? h->ctrl->coll_count : nullptr;
     p.coll_blocks = coll_ctas(h->n, h->sm_count);
     p.coll_short = coll_short(h->n, h->sm_count);
+    p.sms = h->sm_count;
 }
 
 namespace {
@@ -604,9 +605,11 @@ int cloth_profile_substeps(ClothHandle *h, int32_t nsub, float *walk_us, float *
         auto rec = [&](cudaEvent_t x) { return cudaEventRecordWithFlags(x, h->cap_stream, cudaEventRecordExternal); };
         for (int i = 0; i < nsub && le == cudaSuccess; i++) {
             le = rec(ev[3 * i]);
-            if (le == cudaSuccess) le = launch_walk(h->params, h->cap_stream);
+            StepParams q = h->params;
+            q.parity = (int)((h->substeps_done + i) & 1);
+            if (le == cudaSuccess) le = launch_walk(q, h->cap_stream);
             if (le == cudaSuccess) le = rec(ev[3 * i + 1]);
-            if (le == cudaSuccess && h->has_mesh) le = launch_collide(h->params, h->cap_stream);
+            if (le == cudaSuccess && h->has_mesh) le = launch_collide(q, h->cap_stream);
             if (le == cudaSuccess) le = rec(ev[3 * i + 2]);
         }
         e = cudaStreamEndCapture(h->cap_stream, &g);
@@ -653,10 +656,12 @@ int cloth_get_collision_stats(ClothHandle *h, int64_t *listed, int64_t *tested, 
     int rc = check_handle(h);
     if (rc) return rc;
     DeviceScope ds(h->device);
-    unsigned long long v[3] = {0ull, 0ull, 0ull};
-    CTRY(h, cudaMemcpyAsync(v, &h->ctrl->stat_listed, sizeof(v), cudaMemcpyDeviceToHost, h->stream),
+    unsigned long long slots[CLOTH_STAT_SLOTS][4] = {}, v[3] = {0ull, 0ull, 0ull};
+    CTRY(h, cudaMemcpyAsync(slots, h->ctrl->stat, sizeof(slots), cudaMemcpyDeviceToHost, h->stream),
          "read collision statistics");
     CTRY(h, cudaStreamSynchronize(h->stream), "synchronize");
+    for (const auto &q : slots)
+        for (int a = 0; a < 3; a++) v[a] += q[a];
     if (listed) *listed = (int64_t)v[0];
     if (tested) *tested = (int64_t)v[1];
     if (hits) *hits = (int64_t)v[2];

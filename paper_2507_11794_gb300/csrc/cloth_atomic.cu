@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(SPRING_THREADS) spring_atomic_kernel(const __g
     __shared__ unsigned long long s_k;
     pdl_launch_dependents();
     pdl_wait();
-    if (threadIdx.x == 0) s_k = *(volatile unsigned long long *)&p.ctrl->k;
+    if (threadIdx.x == 0) s_k = ctrl_k(p.ctrl);
     __syncthreads();
     const unsigned long long k = s_k;
     const float *__restrict__ in = (k & 1ull) ? p.state1 : p.state0;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(NODE_THREADS) node_integrate_kernel(const __gr
     pdl_launch_dependents();
     pdl_wait();
     if (threadIdx.x == 0) {
-        const unsigned long long k = *(volatile unsigned long long *)&p.ctrl->k;
+        const unsigned long long k = ctrl_k(p.ctrl);
         s_k = k;
         float sw = 0.0f, cw = 1.0f;
         if (p.has_wind) sincosf(wind_base(p.w_turn_step, p.w_turn0, k), &sw, &cw);
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(NODE_THREADS) node_integrate_kernel(const __gr
         const unsigned prev = atomicAdd(&p.ctrl->blocks_done, 1u);
         if (prev == gridDim.x - 1) {
             p.ctrl->blocks_done = 0;
-            p.ctrl->k = k + 1;
+            ctrl_end_k(p.ctrl, k);
         }
     }
 }

@@ -437,10 +437,12 @@ int cloth_batch_get_collision_stats(ClothBatch *b, int64_t *listed, int64_t *tes
 {
     int rc = check_batch(b);
     if (rc) return rc;
-    unsigned long long v[3] = {0ull, 0ull, 0ull};
-    BTRY(b, cudaMemcpyAsync(v, &b->ctrl->stat_listed, sizeof(v), cudaMemcpyDeviceToHost, b->stream),
+    unsigned long long slots[CLOTH_STAT_SLOTS][4] = {}, v[3] = {0ull, 0ull, 0ull};
+    BTRY(b, cudaMemcpyAsync(slots, b->ctrl->stat, sizeof(slots), cudaMemcpyDeviceToHost, b->stream),
          "read collision statistics");
     BTRY(b, cudaStreamSynchronize(b->stream), "synchronize");
+    for (const auto &q : slots)
+        for (int a = 0; a < 3; a++) v[a] += q[a];
     if (listed) *listed = (int64_t)v[0];
     if (tested) *tested = (int64_t)v[1];
     if (hits) *hits = (int64_t)v[2];

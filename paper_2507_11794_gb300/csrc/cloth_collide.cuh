@@ -37,6 +37,15 @@ __device__ __forceinline__ CollBox coll_box(const StepParams &p, float sx, float
     return b;
 }
 
+// a b - c d and a b + c d + e f with every rounding written out: what the
+// compiler contracts differs from kernel to kernel, and a node's response has to
+// come out the same in all of them.
+__device__ __forceinline__ float det_rn(float a, float b, float c, float d) { return __fmaf_rn(a, b, -__fmul_rn(c, d)); }
+__device__ __forceinline__ float dot_rn(float a, float b, float c, float d, float e, float f)
+{
+    return __fmaf_rn(e, f, __fmaf_rn(a, b, __fmul_rn(c, d)));
+}
+
 // One candidate: grid entry e met in cell (cx, cy, cz) of a box whose low
 // corner is (lox, loy, loz).  Returns true on a hit, with th the distance
 // along r, over = th - delta (of the rounded th, whichever lane adds it up) and
@@ -53,21 +62,20 @@ __device__ __forceinline__ bool coll_candidate(const StepParams &p, const CollPa
         max(__float_as_int(C.w), loz) != cz)
         return false;
     // extended Moller-Trumbore: edge S -> E, direction r, length L
-    const float hx = q.ry * C.z - q.rz * C.y;
-    const float hy = q.rz * C.x - q.rx * C.z;
-    const float hz = q.rx * C.y - q.ry * C.x;
-    const float a = B.x * hx + B.y * hy + B.z * hz;
+    const float hx = det_rn(q.ry, C.z, q.rz, C.y);
+    const float hy = det_rn(q.rz, C.x, q.rx, C.z);
+    const float hz = det_rn(q.rx, C.y, q.ry, C.x);
+    const float a = dot_rn(B.x, hx, B.y, hy, B.z, hz);
     if (fabsf(a) < p.eps) return false;
     f = 1.0f / a;
-    const float qx0 = q.sx - A.x, qy0 = q.sy - A.y, qz0 = q.sz - A.z;
-    const float u = f * (qx0 * hx + qy0 * hy + qz0 * hz);
+    const float qx0 = __fsub_rn(q.sx, A.x), qy0 = __fsub_rn(q.sy, A.y), qz0 = __fsub_rn(q.sz, A.z);
+    const float u = __fmul_rn(f, dot_rn(qx0, hx, qy0, hy, qz0, hz));
     if (u < 0.0f || u > 1.0f) return false;
-    const float qx = qy0 * B.z - qz0 * B.y;
-    const float qy = qz0 * B.x - qx0 * B.z;
-    const float qz = qx0 * B.y - qy0 * B.x;
-    const float v = f * (q.rx * qx + q.ry * qy + q.rz * qz);
-    const float e2q = C.x * qx + C.y * qy + C.z * qz;
-    th = __fmul_rn(f, e2q);
+    const float qx = det_rn(qy0, B.z, qz0, B.y);
+    const float qy = det_rn(qz0, B.x, qx0, B.z);
+    const float qz = det_rn(qx0, B.y, qy0, B.x);
+    const float v = __fmul_rn(f, dot_rn(q.rx, qx, q.ry, qy, q.rz, qz));
+    th = __fmul_rn(f, dot_rn(C.x, qx, C.y, qy, C.z, qz));
     over = __fsub_rn(th, p.delta);
     if (v < 0.0f || u + v > 1.0f) return false;
     return th > p.tmin && th < q.L;
@@ -84,13 +92,18 @@ __device__ __forceinline__ float3 coll_hit_point(const CollPath &q, float th)
 __device__ __forceinline__ bool coll_path(const StepParams &p, float sx, float sy, float sz, float ex, float ey,
                                           float ez, CollPath &q)
 {
-    const float dx = ex - sx, dy = ey - sy, dz = ez - sz;
-    q.L = sqrtf(dx * dx + dy * dy + dz * dz);
+    const float dx = __fsub_rn(ex, sx), dy = __fsub_rn(ey, sy), dz = __fsub_rn(ez, sz);
+    q.L = sqrtf(dot_rn(dx, dx, dy, dy, dz, dz));
     if (!(q.L >= p.eps)) return false;
     q.sx = sx; q.sy = sy; q.sz = sz;
     q.rx = dx / q.L; q.ry = dy / q.L; q.rz = dz / q.L;
     return true;
 }
+
+struct OneCloth {  // coll_cells' source of parameters for one cloth
+    const StepParams &p;
+    __device__ const StepParams &params(int) const { return p; }
+};
 
 // Candidate filter: every grid entry carries its triangle's box in 16-bit
 // units of 1 / grid_filter_sub of a cell (grown by p.qpad units), laid out so
@@ -154,7 +167,7 @@ struct NodeHits {
         acc += val;
         if constexpr (REC) {
             if (val > 0.0f) {
-                const float nx = B.y * C.z - B.z * C.y, ny = B.z * C.x - B.x * C.z, nz = B.x * C.y - B.y * C.x;
+                const float nx = det_rn(B.y, C.z, B.z, C.y), ny = det_rn(B.z, C.x, B.x, C.z), nz = det_rn(B.x, C.y, B.y, C.x);
                 // products rounded before they are added
                 g1[0] = __fadd_rn(g1[0], __fmul_rn(nx, f));
                 g1[1] = __fadd_rn(g1[1], __fmul_rn(ny, f));
@@ -398,6 +411,37 @@ __device__ __forceinline__ void coll_cells(const Src &src, int cloth, const Step
     }
 }
 
+// The response of every group's path S -> E (valid: whether it has one; o: its
+// node's plane offset), G lanes per path.  True in the group's first lane if
+// the node hits, with its position x; REC also records the response data.
+template <bool REC, int G, class Src>
+__device__ __forceinline__ bool collide_path(const Src &src, int cloth, const StepParams &p, bool valid, float sx,
+                                             float sy, float sz, float ex, float ey, float ez, long long o, float3 &x,
+                                             unsigned &ntest)
+{
+    CollPath q = {};
+    CollBox bx = {0, 0, 0, 0, 0, 0};
+    CollWords w = {0u, 0u, 0u};
+    int ncell = 0;
+    bool wide = false;
+    if (valid && coll_path(p, sx, sy, sz, ex, ey, ez, q)) {
+        bx = coll_box(p, sx, sy, sz, ex, ey, ez);
+        w = coll_words(p, sx, sy, sz, ex, ey, ez, q);
+        const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
+        wide = nc > COLL_MAXC;
+        ncell = wide ? 0 : (int)nc;
+    }
+    NodeHits<REC> s = {};
+    coll_cells<G, false>(src, cloth, p, q, bx, w, ncell, wide, s, ntest);
+    if (s.K == 0 || (threadIdx.x & 31) % G != 0) return false;
+    const float m = s.acc / (float)s.K;
+    // product and sum rounded separately, the same bits in every kernel
+    x = make_float3(__fadd_rn(q.sx, __fmul_rn(m, q.rx)), __fadd_rn(q.sy, __fmul_rn(m, q.ry)),
+                    __fadd_rn(q.sz, __fmul_rn(m, q.rz)));
+    if constexpr (REC) coll_record(p, o, m, (float)s.K, q.rx, q.ry, q.rz, s.g1, s.g2);
+    return true;
+}
+
 // One round of the list pass, G lanes per node: every group brings one entry
 // (valid: whether it has one; i: its index for src.entry).  Src supplies
 // entry(i, cloth, offset) and params(cloth).  has_pre: the entry's offset is
@@ -418,37 +462,20 @@ __device__ __forceinline__ void collide_round(const Src &src, unsigned long long
     const long long st = p.stride;
     const float *in = (k & 1ull) ? p.state1 : p.state0;
     float *out = (k & 1ull) ? p.state0 : p.state1;
-    CollPath q = {};
-    CollBox bx = {0, 0, 0, 0, 0, 0};
-    CollWords w = {0u, 0u, 0u};
-    int ncell = 0;
-    bool wide = false;
+    float sx = 0.0f, sy = 0.0f, sz = 0.0f, ex = 0.0f, ey = 0.0f, ez = 0.0f;
     if (valid) {
-        const float sx = __ldg(in + o), sy = __ldg(in + st + o), sz = __ldg(in + 2 * st + o);
-        const float ex = out[o], ey = out[st + o], ez = out[2 * st + o];
-        if (coll_path(p, sx, sy, sz, ex, ey, ez, q)) {
-            bx = coll_box(p, sx, sy, sz, ex, ey, ez);
-            w = coll_words(p, sx, sy, sz, ex, ey, ez, q);
-            const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
-            wide = nc > COLL_MAXC;
-            ncell = wide ? 0 : (int)nc;
-        }
+        sx = __ldg(in + o); sy = __ldg(in + st + o); sz = __ldg(in + 2 * st + o);
+        ex = out[o]; ey = out[st + o]; ez = out[2 * st + o];
     }
-    NodeHits<REC> s = {};
-    coll_cells<G, false>(src, cloth, p, q, bx, w, ncell, wide, s, ntest);
-    if (s.K > 0 && (threadIdx.x & 31) % G == 0) {
-        const float m = s.acc / (float)s.K;
-        // product and sum rounded separately, the same bits in every kernel
-        const float ox = __fadd_rn(q.sx, __fmul_rn(m, q.rx)), oy = __fadd_rn(q.sy, __fmul_rn(m, q.ry)),
-                    oz = __fadd_rn(q.sz, __fmul_rn(m, q.rz));
-        if constexpr (REC) coll_record(p, o, m, (float)s.K, q.rx, q.ry, q.rz, s.g1, s.g2);
-        out[o] = ox;
-        out[st + o] = oy;
-        out[2 * st + o] = oz;
+    float3 x;
+    if (collide_path<REC, G>(src, cloth, p, valid, sx, sy, sz, ex, ey, ez, o, x, ntest)) {
+        out[o] = x.x;
+        out[st + o] = x.y;
+        out[2 * st + o] = x.z;
         out[3 * st + o] *= p.restitution;
         out[4 * st + o] *= p.restitution;
         out[5 * st + o] *= p.restitution;
-        fsum += ox + oy + oz;
+        fsum += x.x + x.y + x.z;
         nhit++;
     }
 }
@@ -497,11 +524,20 @@ __device__ __forceinline__ void collide_list(const Src &src, unsigned long long 
         collide_chunks<REC, 1>(src, k, n, fsum, ntest, nhit, false, 0);
 }
 
+// One thread of a CTA adds its counts to the cloth's running statistics.  The
+// adds return nothing, so no thread waits on them.
+__device__ __forceinline__ void coll_stats_store(DevCtrl *ctrl, unsigned listed, unsigned tested, unsigned hits)
+{
+    unsigned long long *q = ctrl->stat[blockIdx.x % CLOTH_STAT_SLOTS];
+    if (listed) atomicAdd(q, (unsigned long long)listed);
+    if (tested) atomicAdd(q + 1, (unsigned long long)tested);
+    if (hits) atomicAdd(q + 2, (unsigned long long)hits);
+}
+
 // Adds a collision pass's counts to the cloth's running statistics: every
 // warp's tested candidates and hit nodes are summed per CTA in shared memory
 // (s2, zeroed by the caller before a __syncthreads), then one thread adds the
-// CTA's totals; CTA 0 also adds the list length n.  The adds return nothing,
-// so no thread waits on them.
+// CTA's totals; CTA 0 also adds the list length n.
 __device__ __forceinline__ void coll_stats_add(DevCtrl *ctrl, unsigned *s2, unsigned n, unsigned ntest, unsigned nhit)
 {
     const unsigned h = __reduce_add_sync(0xffffffffu, nhit), q = __reduce_add_sync(0xffffffffu, ntest);
@@ -511,9 +547,7 @@ __device__ __forceinline__ void coll_stats_add(DevCtrl *ctrl, unsigned *s2, unsi
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        if (s2[0]) atomicAdd(&ctrl->stat_tested, (unsigned long long)s2[0]);
-        if (s2[1]) atomicAdd(&ctrl->stat_hits, (unsigned long long)s2[1]);
-        if (blockIdx.x == 0) atomicAdd(&ctrl->stat_listed, (unsigned long long)n);
+        coll_stats_store(ctrl, blockIdx.x == 0 ? n : 0u, s2[0], s2[1]);
     }
 }
 
@@ -597,11 +631,6 @@ struct EdgeHits {
     }
 };
 
-struct EdgeList {  // coll_cells' source of parameters
-    const StepParams &p;
-    __device__ const StepParams &params(int) const { return p; }
-};
-
 // Pass A of the edge narrow phase: every listed node tests the three edges it
 // owns, (0,+1), (+1,0) and (+1,+1) from it (the triangulation's edges,
 // oriented from their upper-left endpoint), at the updated positions, so each
@@ -655,7 +684,7 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
                 }
             }
         }
-        coll_cells<G, true>(EdgeList{p}, 0, p, path, bx, w, ncell, wide, s, ntest);
+        coll_cells<G, true>(OneCloth{p}, 0, p, path, bx, w, ncell, wide, s, ntest);
         if (has && lane % G == 0) {
             p.edge_hit[s.slot] = s.rec;
             nhit += s.rec.w > 0.0f ? 1u : 0u;

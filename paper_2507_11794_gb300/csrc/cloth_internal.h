@@ -6,26 +6,31 @@
 
 #include "cloth.h"
 
+#define CLOTH_STAT_SLOTS 16
 // Device-side control block of one cloth (one per handle, in device memory).
 struct DevCtrl {
-    unsigned long long k;     // global substep counter: selects time and ping-pong buffer
-    unsigned int blocks_done; // completion counter of the running substep launch (substeps without a mesh)
-    unsigned int flags;       // CTRL_FLAG_* (sticky until set_state)
-    // With a surface model a substep needs no completion count: the walk
-    // copies k to kc, which the collision kernels read, so their first CTA can
-    // advance k at once; they list into coll_count[k & 1] and zero the other
-    // one, which the next substep uses.  Whoever sets k from outside zeroes
-    // both (ctrl_set_k).
+    // The substep counter k (selects time and ping-pong buffer), as two words:
+    // kk[k & 1] = k and the other one lower, so k is the larger (ctrl_k).  A
+    // launch that knows its parity reads kk[parity], which nothing writes while
+    // it runs, and its first CTA stores k + 1 in the other word at once: no
+    // count of finished CTAs is needed to know when everybody has read k.
+    unsigned long long kk[2];
+    // The walk of a substep with collision kernels copies k to kc, which those
+    // read; they list into coll_count[k & 1] and zero the other one, which the
+    // next substep uses.  Whoever sets k from outside zeroes both (ctrl_set_k).
     unsigned long long kc;
     unsigned int coll_count[2];
+    unsigned int blocks_done; // completion counter (the atomic path's substeps without a mesh)
+    unsigned int flags;       // CTRL_FLAG_* (sticky until set_state)
     // running collision statistics since create: listed nodes, candidate
-    // triangles tested, nodes that hit (summed over substeps)
-    unsigned long long stat_listed, stat_tested, stat_hits;
+    // triangles tested, nodes that hit (summed over substeps), in slots that
+    // the CTAs spread their additions over
+    unsigned long long stat[CLOTH_STAT_SLOTS][4];
 };
 
 // NONFINITE: a stored value was NaN/Inf; TIMEOUT: a bounded wait gave up;
-// PARITY: a walk launched with a buffer parity that the substep counter
-// contradicts (a host bookkeeping error; its results are wrong)
+// PARITY: a walk launched with a parity that the substep counter contradicts
+// (a host bookkeeping error; its results are wrong)
 enum : unsigned int { CTRL_FLAG_NONFINITE = 1u, CTRL_FLAG_TIMEOUT = 2u, CTRL_FLAG_PARITY = 4u };
 
 // Spring directions (drow, dcol) of the canonical order; each node owns the
@@ -38,8 +43,7 @@ struct StepParams {
     int nx, ny, n;
     int pitch;                 // floats per row (nx rounded up to 4): node (r,c) at r*pitch + c
     int rows_per_warp;         // rows walked by one warp
-    int parity;                // walk launches: k & 1 as the host knows it when it enqueues the launch (the
-                               // walk then picks its buffers without waiting for k), or -1: read k first
+    int parity;                // k & 1 of the launch, which the host knows when it enqueues it
     int strips_x, strips_y;    // warp strips across columns / rows
     long long stride;          // floats between SoA planes
     float *state0, *state1;    // 6 planes each: px py pz vx vy vz
@@ -85,6 +89,7 @@ struct StepParams {
     unsigned *coll_count;      // entries in coll_list, by substep parity (DevCtrl.coll_count)
     int coll_blocks;           // CTAs of the collision kernel
     int coll_short;            // its form (see coll_short())
+    int sms;                   // multiprocessors of the device
     float delta, eps, tmin, restitution;
     DevCtrl *ctrl;
 };
@@ -112,8 +117,13 @@ inline int coll_ctas(long long n, int sms)
     return (int)(want < 1 ? 1 : (want > most ? most : want));
 }
 
-// Launch one substep (reads state k&1, writes the other, advances ctrl->k).
+// Launch one substep (reads state k&1, writes the other, advances k); p.parity
+// is k & 1 of that substep.
 cudaError_t launch_substep(const StepParams &p, cudaStream_t s);
+// One substep of a small cloth as one kernel (cloth_node.cu), where
+// node_kernel_fits; launch_substep takes it there.
+bool node_kernel_fits(const StepParams &p);
+cudaError_t launch_node_substep(const StepParams &p, cudaStream_t s);
 // The two kernels of a substep separately (with a surface model, the walk
 // leaves the counter to the collision kernel).  With p.force set, the "walk"
 // is the atomic spring kernel followed by the per-node integration kernel.
@@ -203,10 +213,20 @@ inline float grid_filter_scale(const int dims[3], float inv)
 }
 
 #ifdef __CUDACC__
+// The substep counter, where no substep without collision kernels is running.
+__device__ __forceinline__ unsigned long long ctrl_k(const DevCtrl *ctrl)
+{
+    const volatile DevCtrl *c = ctrl;
+    const unsigned long long a = c->kk[0], b = c->kk[1];
+    return a > b ? a : b;
+}
+// End of substep k, by one thread.
+__device__ __forceinline__ void ctrl_end_k(DevCtrl *ctrl, unsigned long long k) { ctrl->kk[(k + 1ull) & 1ull] = k + 1ull; }
 // Sets the substep counter from outside a substep (one thread).
 __device__ __forceinline__ void ctrl_set_k(DevCtrl *ctrl, unsigned long long k)
 {
-    ctrl->k = k;
+    ctrl->kk[k & 1ull] = k;
+    ctrl->kk[(k + 1ull) & 1ull] = k ? k - 1ull : 0ull;
     ctrl->coll_count[0] = ctrl->coll_count[1] = 0u;
 }
 

@@ -22,9 +22,9 @@
 // results are bitwise reproducible.  The first two rows of each walk only
 // produce the springs that reach into the strip.
 #include <type_traits>
-#include <utility>
 
 #include "cloth_collide.cuh"
+#include "cloth_force.cuh"
 #include "cloth_internal.h"
 
 namespace {
@@ -43,35 +43,6 @@ namespace {
 #define CLOTH_PRAGMA(x) _Pragma(#x)
 #define CLOTH_UNROLL(n) CLOTH_PRAGMA(unroll n)
 
-constexpr unsigned FULL = 0xffffffffu;
-
-// Programmatic dependent launch: each kernel of a substep lets the next one
-// be launched once all its CTAs are running (launch_dependents), and waits
-// for the previous one to complete, with its writes visible, before it
-// touches any state (wait).  The next kernel's launch and CTA start-up then
-// overlap this kernel's tail instead of following it.
-#ifndef CLOTH_PDL
-#define CLOTH_PDL 1
-#endif
-// Substep completion: the last CTA of the kernel that ends a substep (found by
-// an atomic count of finished CTAs) advances the substep counter and resets
-// the per-substep counters.  It reads nothing the other CTAs wrote, and every
-// CTA has read those control words before its increment; the next kernel
-// reads them only after this one has completed (or after griddepcontrol.wait),
-// which makes all writes visible.  So no memory fence is taken: a fence would
-// make each CTA wait for its own stores to drain, about 1 us per launch.
-__device__ __forceinline__ void pdl_wait()
-{
-#if CLOTH_PDL
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-#endif
-}
-__device__ __forceinline__ void pdl_launch_dependents()
-{
-#if CLOTH_PDL
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-#endif
-}
 // One warp per CTA: the walk's warps fill one wave, and with 4-warp CTAs
 // 403 CTAs of the 800 x 800 walk put 12 warps on two thirds of the SMs and 8
 // on the rest, so the crowded SMs set the time; single-warp CTAs spread 10
@@ -93,58 +64,6 @@ constexpr int WARPS_PER_CTA = CLOTH_WALK_WARPS;
 #endif
 constexpr int STRIP_COLS = 60;
 
-// Packed FP32x2 arithmetic as explicitly rounded PTX instructions (add.rn,
-// mul.rn, fma.rn on .f32x2).  Each is one IEEE operation per component that
-// no optimizer fuses or reorders, so a node's arithmetic is the same whichever
-// copy of the unrolled row loop computes it; with the CUDA 13.0 packed
-// intrinsics (__fadd2_rn, __fmul2_rn, __ffma2_rn) the four copies of the loop
-// gave results one ulp apart, so a cloth's bits depended on its strip height.
-__device__ __forceinline__ float2 add2(float2 a, float2 b)
-{
-    float2 r;
-    asm("{.reg .b64 x, y, d;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 d, x, y;\n\t"
-        "mov.b64 {%0, %1}, d;}"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    float2 r;
-    asm("{.reg .b64 x, y, d;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 d, x, y;\n\t"
-        "mov.b64 {%0, %1}, d;}"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 r;
-    asm("{.reg .b64 x, y, z, d;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
-        "fma.rn.f32x2 d, x, y, z;\n\tmov.b64 {%0, %1}, d;}"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return r;
-}
-// a - b, exact as one rounding: fma(b, -1, a)
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, make_float2(-1.0f, -1.0f), a); }
-__device__ __forceinline__ float2 bc(float s) { return make_float2(s, s); }
-
-struct Node2 {  // two nodes (A = .x, B = .y)
-    float2 px, py, pz, vx, vy, vz;
-};
-struct Vec2 {  // one 3-vector per node of the pair
-    float2 x, y, z;
-};
-
-__device__ __forceinline__ Vec2 vadd(Vec2 a, Vec2 b) { return {add2(a.x, b.x), add2(a.y, b.y), add2(a.z, b.z)}; }
-__device__ __forceinline__ Vec2 vsub(Vec2 a, Vec2 b) { return {sub2(a.x, b.x), sub2(a.y, b.y), sub2(a.z, b.z)}; }
-
-__device__ __forceinline__ float2 shfl_down2(float2 v, int d)
-{
-    return make_float2(__shfl_down_sync(FULL, v.x, d), __shfl_down_sync(FULL, v.y, d));
-}
-__device__ __forceinline__ float2 shfl_up2(float2 v, int d)
-{
-    return make_float2(__shfl_up_sync(FULL, v.x, d), __shfl_up_sync(FULL, v.y, d));
-}
 // Row r of the lane's two columns.  The row and the column pair are clamped
 // into the grid's memory, so every load is in bounds; the values of a row
 // outside [0, ny) or a pair outside the pitch are finite stand-ins that only
@@ -164,56 +83,6 @@ __device__ __forceinline__ Node2 load_row(const float *in, unsigned st, int r, i
     n.vz = __ldg((const float2 *)(in + (o + 5u * st)));
     return n;
 }
-
-// Hooke's law plus damping along the spring (Algorithm 1) for the pair:
-// d = q - p, F_p = (ks (|d| - L0) + kd (v_q - v_p).d / |d|) d / |d|, written
-// as F_p = s d with s = (ks (|d| - L0) + kd il (v_q - v_p).d) il, il = 1/|d|
-// (zero force for |d|^2 <= 1e-24).
-// The same from the differences d = q - p (dx, dy, dz) and v_q - v_p (ux,
-// uy, uz).
-__device__ __forceinline__ Vec2 spring2d(float2 dx, float2 dy, float2 dz, float2 ux, float2 uy, float2 uz, float2 ks,
-                                         float2 kd, float L0)
-{
-    const float2 l2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-    float2 il;
-    il.x = l2.x > 1e-24f ? rsqrtf(l2.x) : 0.0f;
-    il.y = l2.y > 1e-24f ? rsqrtf(l2.y) : 0.0f;
-    const float2 dvd = fma2(uz, dz, fma2(uy, dy, mul2(ux, dx)));
-    const float2 e = fma2(l2, il, bc(-L0));  // |d| - L0
-    const float2 sc = mul2(fma2(mul2(kd, il), dvd, mul2(ks, e)), il);
-    return {mul2(sc, dx), mul2(sc, dy), mul2(sc, dz)};
-}
-__device__ __forceinline__ Vec2 spring2(const Node2 &P, const Node2 &Q, float2 ks, float2 kd, float L0)
-{
-    return spring2d(sub2(Q.px, P.px), sub2(Q.py, P.py), sub2(Q.pz, P.pz), sub2(Q.vx, P.vx), sub2(Q.vy, P.vy),
-                    sub2(Q.vz, P.vz), ks, kd, L0);
-}
-// A spring of each node of the pair P towards the pair Q = (a.y, b.x) that
-// straddles two column pairs: the differences are formed one component at a
-// time, so Q is never assembled.
-__device__ __forceinline__ float2 dstr(float ay, float bx, float2 p) { return make_float2(__fsub_rn(ay, p.x), __fsub_rn(bx, p.y)); }
-__device__ __forceinline__ Vec2 spring2s(const Node2 &P, const Node2 &a, const Node2 &b, float2 ks, float2 kd,
-                                         float L0)
-{
-    return spring2d(dstr(a.px.y, b.px.x, P.px), dstr(a.py.y, b.py.x, P.py), dstr(a.pz.y, b.pz.x, P.pz),
-                    dstr(a.vx.y, b.vx.x, P.vx), dstr(a.vy.y, b.vy.x, P.vy), dstr(a.vz.y, b.vz.x, P.vz), ks, kd, L0);
-}
-
-// Sign bits set (node A in .x, node B in .y) where the segment from s to e
-// lies on the far side of one face of the slab [lo, hi]: both ends below lo
-// or both above hi.
-__device__ __forceinline__ uint2 box_out_bits(float2 s, float2 e, float lo, float hi)
-{
-    const float2 a = sub2(s, bc(lo)), b = sub2(e, bc(lo)), c = sub2(bc(hi), s), d = sub2(bc(hi), e);
-    return make_uint2((__float_as_uint(a.x) & __float_as_uint(b.x)) | (__float_as_uint(c.x) & __float_as_uint(d.x)),
-                      (__float_as_uint(a.y) & __float_as_uint(b.y)) | (__float_as_uint(c.y) & __float_as_uint(d.y)));
-}
-
-// q - (ay, bx) for a pair q and the straddling pair (a.y, b.x), one
-// component at a time.
-__device__ __forceinline__ float2 rdstr(float2 q, float ay, float bx) { return make_float2(__fsub_rn(q.x, ay), __fsub_rn(q.y, bx)); }
-__device__ __forceinline__ Vec2 vscale(Vec2 a, float2 s) { return {mul2(a.x, s), mul2(a.y, s), mul2(a.z, s)}; }
-
 
 // Inputs of a strip that do not change from substep to substep (the wind
 // tables and the pin bits): the lane's column wind terms and the first output
@@ -492,10 +361,7 @@ __device__ __forceinline__ void walk_strip(const StepParams &p, const float *__r
             float2 ay = fma2(F.y, bc(p.inv_mass), bc(p.g[1]));
             float2 az = fma2(F.z, bc(p.inv_mass), bc(p.g[2]));
             if (p.has_wind) {
-                // sin(a + b) = sin(a) cos(b) + cos(a) sin(b), a = base + alpha_r
-                const float sinR = sinW * tr.y + cosW * tr.x;
-                const float cosR = cosW * tr.y - sinW * tr.x;
-                const float2 w = mul2(bc(p.w_amp), fma2(bc(cosR), sinB, mul2(bc(sinR), cosB)));
+                const float2 w = wind_pair(sinW, cosW, tr, sinB, cosB, p.w_amp);
                 ax = fma2(w, bc(p.w_dir[0]), ax);
                 ay = fma2(w, bc(p.w_dir[1]), ay);
                 az = fma2(w, bc(p.w_dir[2]), az);
@@ -636,20 +502,19 @@ __global__ void CLOTH_WALK_BOUNDS substep_kernel(const StepParams p)
     WalkStatics ws{};
     if (active) ws = walk_statics(p, sx, sy, lane);  // before the wait: static tables only
     pdl_wait();
-    // Every lane reads the substep counter itself and, with the parity known
-    // at launch (p.parity >= 0), picks its buffers without waiting for it:
-    // the row loads then overlap the counter's read, which only the wind
-    // phase and the end of the substep need.  The mesh walk (DLR) keeps the
-    // counter read by one thread and the buffers picked from it: there the
-    // other form spilled and was 1.6% slower.
+    // The launch's parity picks the buffers, so the row loads overlap the
+    // counter's read, which only the wind phase and the end of the substep
+    // need.  The mesh walk (DLR) has it read by one thread per CTA and picks
+    // the buffers from it: there the other form was 2% slower.
     constexpr bool DLR = MESH && !EDGE && !PER_SPRING;
+    const int par = p.parity & 1;
     unsigned long long k;
     float wbase;
     if (DLR) {
         __shared__ unsigned long long s_k;
         __shared__ float s_wbase;
         if (threadIdx.x == 0) {
-            k = *(volatile unsigned long long *)&p.ctrl->k;
+            k = *(volatile unsigned long long *)&p.ctrl->kk[par];
             s_k = k;
             s_wbase = p.has_wind ? wind_base(p.w_turn_step, p.w_turn0, k) : 0.0f;
         }
@@ -657,10 +522,10 @@ __global__ void CLOTH_WALK_BOUNDS substep_kernel(const StepParams p)
         k = s_k;
         wbase = s_wbase;
     } else {
-        k = *(volatile unsigned long long *)&p.ctrl->k;
+        k = *(volatile unsigned long long *)&p.ctrl->kk[par];
         wbase = p.has_wind ? wind_base(p.w_turn_step, p.w_turn0, k) : 0.0f;
     }
-    const bool odd = p.parity >= 0 && !DLR ? p.parity != 0 : (k & 1ull) != 0ull;
+    const bool odd = DLR ? (k & 1ull) != 0ull : par != 0;
     const float *__restrict__ in = odd ? p.state1 : p.state0;
     float *__restrict__ out = odd ? p.state0 : p.state1;
     // sum of the stored positions: non-finite iff one of them is or a stored
@@ -668,27 +533,16 @@ __global__ void CLOTH_WALK_BOUNDS substep_kernel(const StepParams p)
     float2 fsum = bc(0.0f);
     // DLR (receiver-side (+1,-1) springs) in the mesh walk only: 2% faster
     // there, slower without a mesh
-    if (active) walk_strip<MESH && !EDGE, PER_SPRING, DLR>(p, in, out, wbase, sx, sy, lane, 0, p.coll_count + (k & 1ull),
+    if (active) walk_strip<MESH && !EDGE, PER_SPRING, DLR>(p, in, out, wbase, sx, sy, lane, 0, p.coll_count + (int)odd,
                                                              fsum, ws);
-    // the launch's parity checked against the counter after the walk (a
-    // check before it would make the walk wait for the counter)
-    if (!DLR && p.parity >= 0 && (int)(k & 1ull) != p.parity && threadIdx.x == 0)
-        atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_PARITY);
 
     const bool bad = !isfinite(fsum.x + fsum.y);
     if (__any_sync(FULL, bad) && lane == 0) atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
-    if (MESH || EDGE) {  // the collision kernels finish the substep
-        if (blockIdx.x == 0 && threadIdx.x == 0) p.ctrl->kc = k;
-        return;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // the last CTA to finish advances the substep counter for the next launch
-        const unsigned prev = atomicAdd(&p.ctrl->blocks_done, 1u);
-        if (prev == gridDim.x - 1) {
-            p.ctrl->blocks_done = 0;
-            p.ctrl->k = k + 1;
-        }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // the other word is lower until this launch ends the substep
+        if (*(volatile unsigned long long *)&p.ctrl->kk[par ^ 1] > k) atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_PARITY);
+        if (MESH || EDGE) p.ctrl->kc = k;  // the collision kernels finish the substep
+        else ctrl_end_k(p.ctrl, k);
     }
 }
 
@@ -712,7 +566,7 @@ __device__ __forceinline__ void coll_begin(DevCtrl *ctrl, unsigned long long &k,
 __device__ __forceinline__ void coll_end(DevCtrl *ctrl, unsigned long long k)
 {
     ctrl->coll_count[(k + 1ull) & 1ull] = 0u;
-    ctrl->k = k + 1ull;
+    ctrl_end_k(ctrl, k);
 }
 
 // List entries of one cloth.
@@ -906,7 +760,7 @@ __global__ void __launch_bounds__(32 * CLOTH_WALK_WARPS, CLOTH_BATCH_MINB) batch
     __shared__ unsigned long long s_k;
     pdl_launch_dependents();
     pdl_wait();
-    if (threadIdx.x == 0) s_k = *(volatile unsigned long long *)&b.ctrl->k;
+    if (threadIdx.x == 0) s_k = ctrl_k(b.ctrl);
     __syncthreads();
     const unsigned long long k = s_k;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -984,7 +838,7 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) batch_collid
 __global__ void aos_to_soa_kernel(const float *__restrict__ pos, const float *__restrict__ vel, float *state0,
                                   float *state1, long long st, int n, int nx, int pitch, DevCtrl *ctrl)
 {
-    const unsigned long long k = *(volatile unsigned long long *)&ctrl->k;
+    const unsigned long long k = ctrl_k(ctrl);
     float *dst = (k & 1ull) ? state1 : state0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const long long o = (long long)(i / nx) * pitch + (i % nx);
@@ -1005,7 +859,7 @@ __global__ void aos_to_soa_kernel(const float *__restrict__ pos, const float *__
 __global__ void soa_to_aos_kernel(const float *state0, const float *state1, long long st, int n, int nx, int pitch,
                                   const DevCtrl *ctrl, float *__restrict__ pos, float *__restrict__ vel)
 {
-    const unsigned long long k = *(volatile const unsigned long long *)&ctrl->k;
+    const unsigned long long k = ctrl_k(ctrl);
     const float *src = (k & 1ull) ? state1 : state0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const long long o = (long long)(i / nx) * pitch + (i % nx);
@@ -1051,25 +905,6 @@ void substep_shape(StepParams &p)
     p.strips_y = (p.ny + p.rows_per_warp - 1) / p.rows_per_warp;
 }
 
-namespace {
-// Kernel launch with the programmatic-serialisation attribute (see pdl_wait).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_k(void (*kern)(KArgs...), int blocks, int threads, cudaStream_t s, Args &&...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = CLOTH_PDL;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-}
-}  // namespace
-
 cudaError_t launch_walk(const StepParams &p, cudaStream_t s)
 {
     if (p.force) return launch_atomic_forces_and_integrate(p, s);
@@ -1108,6 +943,7 @@ cudaError_t launch_collide(const StepParams &p, cudaStream_t s)
 
 cudaError_t launch_substep(const StepParams &p, cudaStream_t s)
 {
+    if (node_kernel_fits(p)) return launch_node_substep(p, s);
     cudaError_t e = launch_walk(p, s);
     if (e == cudaSuccess && p.has_mesh) e = launch_collide(p, s);
     return e;
