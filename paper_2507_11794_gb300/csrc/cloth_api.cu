@@ -78,6 +78,7 @@ void free_all(ClothHandle *h)
     cudaFree(h->kd_slot);
     cudaFree(h->ctrl);
     cudaFree(h->staging);
+    bounce_release(&h->bounce);
     cudaFree(h->coll_list);
     h->coll_list = nullptr;
     cudaFree(h->wind_tab);
@@ -537,22 +538,13 @@ int cloth_read(ClothHandle *h, float *pos_out, float *vel_out)
     int rc = check_handle(h);
     if (rc) return rc;
     DeviceScope ds(h->device);
-    const long long N = h->n;
     unsigned flags = 0;
     if (pos_out || vel_out) {
-        CTRY(h, launch_soa_to_aos(h->state, h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, h->ctrl,
-                                  pos_out ? h->staging : nullptr, vel_out ? h->staging + 3 * N : nullptr, h->stream),
-             "state gather");
-        if (pos_out)
-            CTRY(h, cudaMemcpyAsync(pos_out, h->staging, sizeof(float) * 3 * N, cudaMemcpyDeviceToHost, h->stream),
-                 "copy positions");
-        if (vel_out)
-            CTRY(h, cudaMemcpyAsync(vel_out, h->staging + 3 * N, sizeof(float) * 3 * N, cudaMemcpyDeviceToHost,
-                                    h->stream),
-                 "copy velocities");
+        CTRY(h, state_to_host(h, h->ctrl, &h->bounce, pos_out, vel_out, &flags, h->stream), "read state");
+    } else {
+        rc = read_flags(h, &flags);
+        if (rc) return rc;
     }
-    rc = read_flags(h, &flags);
-    if (rc) return rc;
     return flags_status(flags);
 }
 
@@ -562,12 +554,7 @@ int cloth_set_state(ClothHandle *h, const float *pos, const float *vel)
     if (rc) return rc;
     if (!pos && !vel) return CLOTH_OK;
     DeviceScope ds(h->device);
-    const long long N = h->n;
-    if (pos) CTRY(h, upload(h->staging, pos, sizeof(float) * 3 * N, h->stream), "upload positions");
-    if (vel) CTRY(h, upload(h->staging + 3 * N, vel, sizeof(float) * 3 * N, h->stream), "upload velocities");
-    CTRY(h, launch_aos_to_soa(pos ? h->staging : nullptr, vel ? h->staging + 3 * N : nullptr, h->state,
-                              h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, h->ctrl, h->stream),
-         "state scatter");
+    CTRY(h, state_from_host(h, h->ctrl, pos, vel, h->stream), "set state");
     return CLOTH_OK;
 }
 

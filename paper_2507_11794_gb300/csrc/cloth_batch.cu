@@ -21,6 +21,7 @@ struct ClothBatch {
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
     DevCtrl *ctrl = nullptr;
+    HostBounce bounce;
     unsigned *work = nullptr;
     int *coll_list = nullptr;
     int *coll_cloth = nullptr;
@@ -154,6 +155,7 @@ void free_batch(ClothBatch *b)
     for (ClothHandle *h : b->cl) cloth_destroy(h);
     b->cl.clear();
     cudaFree(b->ctrl);
+    bounce_release(&b->bounce);
     cudaFree(b->work);
     cudaFree(b->coll_list);
     cudaFree(b->coll_cloth);
@@ -162,15 +164,20 @@ void free_batch(ClothBatch *b)
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
 }
 
+int batch_flags_status(unsigned flags)
+{
+    if (flags & CTRL_FLAG_TIMEOUT) return bfail(CLOTH_ERR_TIMEOUT, "a device-side wait timed out");
+    if (flags & CTRL_FLAG_NONFINITE) return bfail(CLOTH_ERR_NONFINITE, "a cloth of the batch became non-finite");
+    return CLOTH_OK;
+}
+
 int read_batch_flags(ClothBatch *b)
 {
     unsigned flags = 0;
     BTRY(b, cudaMemcpyAsync(&flags, &b->ctrl->flags, sizeof(flags), cudaMemcpyDeviceToHost, b->stream),
          "read flags");
     BTRY(b, cudaStreamSynchronize(b->stream), "synchronize");
-    if (flags & CTRL_FLAG_TIMEOUT) return bfail(CLOTH_ERR_TIMEOUT, "a device-side wait timed out");
-    if (flags & CTRL_FLAG_NONFINITE) return bfail(CLOTH_ERR_NONFINITE, "a cloth of the batch became non-finite");
-    return CLOTH_OK;
+    return batch_flags_status(flags);
 }
 
 }  // namespace
@@ -283,21 +290,10 @@ int cloth_batch_read(ClothBatch *b, int32_t index, float *pos_out, float *vel_ou
     int rc = check_batch(b);
     if (rc) return rc;
     if (index < 0 || index >= (int)b->cl.size()) return bfail(CLOTH_ERR_INVALID_ARG, "cloth index %d", index);
-    ClothHandle *h = b->cl[index];
-    const long long N = h->n;
-    if (pos_out || vel_out) {
-        BTRY(b, launch_soa_to_aos(h->state, h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, b->ctrl,
-                                  pos_out ? h->staging : nullptr, vel_out ? h->staging + 3 * N : nullptr, b->stream),
-             "state gather");
-        if (pos_out)
-            BTRY(b, cudaMemcpyAsync(pos_out, h->staging, sizeof(float) * 3 * N, cudaMemcpyDeviceToHost, b->stream),
-                 "copy positions");
-        if (vel_out)
-            BTRY(b, cudaMemcpyAsync(vel_out, h->staging + 3 * N, sizeof(float) * 3 * N, cudaMemcpyDeviceToHost,
-                                    b->stream),
-                 "copy velocities");
-    }
-    return read_batch_flags(b);
+    unsigned flags = 0;
+    if (!pos_out && !vel_out) return read_batch_flags(b);
+    BTRY(b, state_to_host(b->cl[index], b->ctrl, &b->bounce, pos_out, vel_out, &flags, b->stream), "read state");
+    return batch_flags_status(flags);
 }
 
 int cloth_batch_set_state(ClothBatch *b, int32_t index, const float *pos, const float *vel)
@@ -306,17 +302,7 @@ int cloth_batch_set_state(ClothBatch *b, int32_t index, const float *pos, const 
     if (rc) return rc;
     if (index < 0 || index >= (int)b->cl.size()) return bfail(CLOTH_ERR_INVALID_ARG, "cloth index %d", index);
     if (!pos && !vel) return CLOTH_OK;
-    ClothHandle *h = b->cl[index];
-    const long long N = h->n;
-    if (pos)
-        BTRY(b, cudaMemcpyAsync(h->staging, pos, sizeof(float) * 3 * N, cudaMemcpyHostToDevice, b->stream),
-             "upload positions");
-    if (vel)
-        BTRY(b, cudaMemcpyAsync(h->staging + 3 * N, vel, sizeof(float) * 3 * N, cudaMemcpyHostToDevice, b->stream),
-             "upload velocities");
-    BTRY(b, launch_aos_to_soa(pos ? h->staging : nullptr, vel ? h->staging + 3 * N : nullptr, h->state,
-                              h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, b->ctrl, b->stream),
-         "state scatter");
+    BTRY(b, state_from_host(b->cl[index], b->ctrl, pos, vel, b->stream), "set state");
     return CLOTH_OK;
 }
 
