@@ -32,7 +32,8 @@ struct ClothBatch {
     int ctas_per_sm = 2;
     int substeps = 1;
     BatchArgs args{};
-    cudaGraphExec_t graph = nullptr;
+    int2 *d_groups = nullptr;
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};  // one step, by the parity of its first substep
     long long substeps_done = 0;
     bool dead = false;
 };
@@ -69,12 +70,19 @@ int check_batch(ClothBatch *b)
     return CLOTH_OK;
 }
 
+void drop_graphs(ClothBatch *b)
+{
+    for (cudaGraphExec_t &g : b->graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+}
+
 // Parameters of every cloth for the current tuning, and the item list sorted
 // longest first (ties: cloth, strip row, strip column).
 cudaError_t rebuild(ClothBatch *b)
 {
-    if (b->graph) cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
+    drop_graphs(b);
     const int scols = substep_strip_cols();
     std::vector<StepParams> prm(b->cl.size());
     std::vector<int4> items;
@@ -127,16 +135,46 @@ cudaError_t rebuild(ClothBatch *b)
         var = var < 0 || var == v ? v : BATCH_VAR_MIXED;
     }
     b->args.variant = var < 0 ? BATCH_VAR_MIXED : var;
+    // small cloths: a list of 64-position groups for the one-kernel substep
+    cudaFree(b->d_groups);
+    b->d_groups = nullptr;
+    std::vector<int2> groups;
+    long long ng = 0;
+    for (const StepParams &q : prm) ng += ((long long)q.ny * q.pitch + 63) / 64;
+    if (node_batch_fits(ng, b->args.variant, b->sm_count))
+        for (size_t i = 0; i < prm.size(); i++)
+            for (long long j = 0; 64 * j < (long long)prm[i].ny * prm[i].pitch; j++)
+                groups.push_back(make_int2((int)i, (int)j));
+    if (e == cudaSuccess && !groups.empty()) {
+        e = cudaMalloc(&b->d_groups, sizeof(int2) * groups.size());
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(b->d_groups, groups.data(), sizeof(int2) * groups.size(), cudaMemcpyHostToDevice,
+                                b->stream);
+    }
+    // the other form of the substep leaves the listing counts as they were
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->ctrl->coll_count, 0, sizeof(b->ctrl->coll_count), b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    b->args.groups = b->d_groups;
+    b->args.n_groups = (int)groups.size();
+    b->args.sms = b->sm_count;
+    b->args.parity = 0;
     return e;
 }
 
-cudaError_t ensure_graph(ClothBatch *b)
+cudaError_t launch_parity(const ClothBatch *b, long long k, cudaStream_t s)
 {
-    if (b->graph) return cudaSuccess;
+    BatchArgs a = b->args;
+    a.parity = (int)(k & 1);
+    return launch_batch_substep(a, s);
+}
+
+cudaError_t ensure_graph(ClothBatch *b, int par)
+{
+    if (b->graph[par]) return cudaSuccess;
     cudaError_t e = cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     cudaError_t le = cudaSuccess;
-    for (int s = 0; s < b->substeps && le == cudaSuccess; s++) le = launch_batch_substep(b->args, b->cap_stream);
+    for (int s = 0; s < b->substeps && le == cudaSuccess; s++) le = launch_parity(b, par + s, b->cap_stream);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(b->cap_stream, &g);
     if (le != cudaSuccess) {
@@ -144,14 +182,14 @@ cudaError_t ensure_graph(ClothBatch *b)
         return le;
     }
     if (e != cudaSuccess) return e;
-    e = cudaGraphInstantiate(&b->graph, g, 0);
+    e = cudaGraphInstantiate(&b->graph[par], g, 0);
     cudaGraphDestroy(g);
     return e;
 }
 
 void free_batch(ClothBatch *b)
 {
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    drop_graphs(b);
     for (ClothHandle *h : b->cl) cloth_destroy(h);
     b->cl.clear();
     cudaFree(b->ctrl);
@@ -161,6 +199,7 @@ void free_batch(ClothBatch *b)
     cudaFree(b->coll_cloth);
     cudaFree(b->d_params);
     cudaFree(b->d_items);
+    cudaFree(b->d_groups);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
 }
 
@@ -168,6 +207,7 @@ int batch_flags_status(unsigned flags)
 {
     if (flags & CTRL_FLAG_TIMEOUT) return bfail(CLOTH_ERR_TIMEOUT, "a device-side wait timed out");
     if (flags & CTRL_FLAG_NONFINITE) return bfail(CLOTH_ERR_NONFINITE, "a cloth of the batch became non-finite");
+    if (flags & CTRL_FLAG_PARITY) return bfail(CLOTH_ERR_STATE, "a substep ran on the wrong state buffer (internal)");
     return CLOTH_OK;
 }
 
@@ -279,8 +319,12 @@ int cloth_batch_step(ClothBatch *b, int32_t nsteps)
     int rc = check_batch(b);
     if (rc) return rc;
     if (nsteps < 0) return bfail(CLOTH_ERR_INVALID_ARG, "nsteps < 0");
-    BTRY(b, ensure_graph(b), "graph capture");
-    for (int s = 0; s < nsteps; s++) BTRY(b, cudaGraphLaunch(b->graph, b->stream), "graph launch");
+    BTRY(b, ensure_graph(b, (int)(b->substeps_done & 1)), "graph capture");
+    for (long long s = 0; s < nsteps; s++) {
+        const int par = (int)((b->substeps_done + s * b->substeps) & 1);
+        BTRY(b, ensure_graph(b, par), "graph capture");
+        BTRY(b, cudaGraphLaunch(b->graph[par], b->stream), "graph launch");
+    }
     b->substeps_done += (long long)nsteps * b->substeps;
     return CLOTH_OK;
 }
@@ -345,6 +389,7 @@ int cloth_batch_tune(ClothBatch *b, int32_t trial_substeps, ClothBatchTuning *ou
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     const int Rs[] = {4, 6, 8, 12, 16, 24, 32};
+    long long k = b->substeps_done;
     for (int c = 1; c <= batch_min_ctas() && e == cudaSuccess; c++)
         for (int R : Rs) {
             if (e != cudaSuccess) break;
@@ -355,9 +400,9 @@ int cloth_batch_tune(ClothBatch *b, int32_t trial_substeps, ClothBatchTuning *ou
             } catch (...) {
                 e = cudaErrorMemoryAllocation;
             }
-            if (e == cudaSuccess) e = launch_batch_substep(b->args, b->stream);  // warm-up
+            if (e == cudaSuccess) e = launch_parity(b, k++, b->stream);  // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-            for (int s = 0; s < trial_substeps && e == cudaSuccess; s++) e = launch_batch_substep(b->args, b->stream);
+            for (int s = 0; s < trial_substeps && e == cudaSuccess; s++) e = launch_parity(b, k++, b->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float ms = 0.0f;

@@ -146,9 +146,16 @@ struct BatchArgs {
     unsigned *coll_count;
     int walk_blocks, coll_blocks;
     int variant;               // BATCH_VAR_* shared by every cloth, or BATCH_VAR_MIXED
+    const int2 *groups;        // batches of small cloths: (cloth, 64 plane positions), or nullptr
+    int n_groups;
+    int parity;                // k & 1 of the launch
+    int sms;                   // multiprocessors of the device
 };
 enum : int { BATCH_VAR_MESH = 1, BATCH_VAR_PER_SPRING = 2, BATCH_VAR_MIXED = 4 };
 cudaError_t launch_batch_substep(const BatchArgs &b, cudaStream_t s);
+// One substep of a batch of small cloths as one kernel (cloth_node.cu).
+bool node_batch_fits(long long groups, int variant, int sms);
+cudaError_t launch_node_batch(const BatchArgs &b, cudaStream_t s);
 int substep_strip_cols();
 int substep_warps_per_cta();
 int substep_min_ctas();

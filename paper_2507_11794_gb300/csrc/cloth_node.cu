@@ -199,20 +199,19 @@ enum { NODE_FREE = 0, NODE_MESH = 1, NODE_EDGE = 2, NODE_LIST = 3 };
 // kernels follow (cloth_step.cu); or a surface model whose nodes are listed
 // for the collision pass that follows.  W warps per CTA: the first computes the
 // CTA's 32 pairs, all of them collide.  REC: the adjoint's recompute.
+//
+// The CTA's nodes are the 64 plane positions from `base`.
 template <int MODE, bool PS, bool REC, int W>
-__global__ void __launch_bounds__(32 * W, W == 1 ? 12 : W == 2 ? CLOTH_NODE_W2 : W == 4 ? 3 : 1) node_kernel(const __grid_constant__ StepParams p)
+__device__ __forceinline__ void node_substep(const StepParams &p, const int par, const unsigned base)
 {
     // per node of the CTA: start and end of the path, end velocity
     __shared__ float s_x[MODE == NODE_MESH ? 9 : 1][64];
     __shared__ int s_list[64], s_n;
     __shared__ unsigned s_stat[2];
-    pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const unsigned st = (unsigned)p.stride;
-    const int par = p.parity & 1;
     const float *in = par ? p.state1 : p.state0;
     float *out = par ? p.state0 : p.state1;
-    const unsigned base = 64u * blockIdx.x;
     float fs = 0.0f;
     if (threadIdx.x < 32) {
         const unsigned total = (unsigned)p.ny * (unsigned)p.pitch;
@@ -367,6 +366,36 @@ __global__ void __launch_bounds__(32 * W, W == 1 ? 12 : W == 2 ? CLOTH_NODE_W2 :
     if (__any_sync(FULL, !isfinite(fs)) && lane == 0) atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
 }
 
+constexpr int node_min_ctas(int W) { return W == 1 ? CLOTH_NODE_MAX : W == 2 ? CLOTH_NODE_W2 : W == 4 ? CLOTH_NODE_W4 : CLOTH_NODE_W8; }
+
+template <int MODE, bool PS, bool REC, int W>
+__global__ void __launch_bounds__(32 * W, node_min_ctas(W)) node_kernel(const __grid_constant__ StepParams p)
+{
+    pdl_launch_dependents();
+    node_substep<MODE, PS, REC, W>(p, p.parity & 1, 64u * blockIdx.x);
+}
+
+// A batch of small cloths: a CTA per (cloth, 64 positions) of the list b.groups.
+template <int MODE, bool PS, int W>
+__global__ void __launch_bounds__(32 * W, node_min_ctas(W)) node_batch_kernel(const __grid_constant__ BatchArgs b)
+{
+    __shared__ StepParams p;
+    pdl_launch_dependents();
+    const int2 g = __ldg(b.groups + blockIdx.x);
+    const unsigned *src = (const unsigned *)(b.params + g.x);  // does not change from substep to substep
+    for (int w = threadIdx.x; w < (int)(sizeof(StepParams) / 4); w += 32 * W) ((unsigned *)&p)[w] = __ldg(src + w);
+    if (W == 1) __syncwarp();
+    else __syncthreads();
+    node_substep<MODE, PS, false, W>(p, b.parity & 1, 64u * (unsigned)g.y);
+}
+
+template <int MODE, int W>
+cudaError_t launch_batch_mode(const BatchArgs &b, cudaStream_t s)
+{
+    return b.variant & BATCH_VAR_PER_SPRING ? launch_k(node_batch_kernel<MODE, true, W>, b.n_groups, 32 * W, s, b)
+                                            : launch_k(node_batch_kernel<MODE, false, W>, b.n_groups, 32 * W, s, b);
+}
+
 template <int MODE, int W>
 cudaError_t launch_mode(const StepParams &p, int blocks, cudaStream_t s)
 {
@@ -397,4 +426,19 @@ cudaError_t launch_node_substep(const StepParams &p, cudaStream_t s)
     if (blocks <= CLOTH_NODE_W2 * p.sms) return launch_mode<NODE_MESH, 2>(p, blocks, s);
     const cudaError_t e = launch_mode<NODE_LIST, 1>(p, blocks, s);
     return e == cudaSuccess ? launch_collide(p, s) : e;
+}
+
+// As for one cloth, by the batch's number of groups; a batch that mixes walk
+// variants or has more groups than are resident takes the persistent walk.
+bool node_batch_fits(long long groups, int variant, int sms)
+{
+    return variant != BATCH_VAR_MIXED && groups <= (long long)(variant & BATCH_VAR_MESH ? CLOTH_NODE_W2 : CLOTH_NODE_MAX) * sms;
+}
+
+cudaError_t launch_node_batch(const BatchArgs &b, cudaStream_t s)
+{
+    if (!(b.variant & BATCH_VAR_MESH)) return launch_batch_mode<NODE_FREE, 1>(b, s);
+    if (b.n_groups <= CLOTH_NODE_W8 * b.sms) return launch_batch_mode<NODE_MESH, 8>(b, s);
+    if (b.n_groups <= CLOTH_NODE_W4 * b.sms) return launch_batch_mode<NODE_MESH, 4>(b, s);
+    return launch_batch_mode<NODE_MESH, 2>(b, s);
 }

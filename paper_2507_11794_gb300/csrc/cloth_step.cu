@@ -946,6 +946,7 @@ cudaError_t launch_substep(const StepParams &p, cudaStream_t s)
 
 cudaError_t launch_batch_substep(const BatchArgs &b, cudaStream_t s)
 {
+    if (b.groups) return launch_node_batch(b, s);
     cudaError_t e;
     switch (b.variant) {
     case 0: e = launch_k(batch_substep_kernel<0>, b.walk_blocks, 32 * WARPS_PER_CTA, s, b); break;

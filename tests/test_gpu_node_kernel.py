@@ -100,3 +100,57 @@ def test_rollout_recompute(cloth_lib, nx, ny):
             ro.close()
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+# (sides, cloths): groups of 64 positions on 152 SMs: below one, three and eight CTAs per SM, and above (the walk)
+BATCHES = {"few": ((5, 17, 31), 1), "eight_warps": ((16, 33, 40), 3), "four_warps": ((24, 61, 70), 4),
+           "two_warps": ((40, 61, 90), 7), "walk": ((100, 120, 121), 5)}
+
+
+@pytest.mark.parametrize("case", BATCHES)
+@pytest.mark.parametrize("springs", [False, True])
+@pytest.mark.parametrize("mesh", [False, True])
+def test_batches(cloth_lib, case, springs, mesh):
+    """Every cloth of a batch as stepped alone by the walk, over an odd number
+    of substeps per step (both parities)."""
+    sides, times = BATCHES[case]
+    scs = [scene(n + i, n, mesh, True, seed=n + i) for i in range(times) for n in sides]
+    for sc in scs:
+        sc.substeps, sc.dt = 3, 3 / 4800
+        if springs:
+            per_spring(sc)
+    b = cloth_lib.ClothBatch(scs)
+    b.step(1)
+    b.step(2)
+    total = np.zeros(3, int)
+    for i, sc in enumerate(scs):
+        with cloth_lib.Cloth(sc) as cl:
+            cl.profile_substeps(9)
+            (pa, va), (pb, vb) = b.read(i), cl.read()
+            total += cl.collision_stats()
+        np.testing.assert_array_equal(pa, pb)
+        np.testing.assert_array_equal(va, vb)
+    assert tuple(total) == b.collision_stats()
+    b.close()
+
+
+def test_batch_changes_form(cloth_lib):
+    """Meshes set and cleared between steps take a batch from one form of the
+    substep to the other (one walk variant or mixed) and back."""
+    scs = [scene(30, 28, True, False, seed=i) for i in range(3)]
+    b = cloth_lib.ClothBatch(scs)
+    cls = [cloth_lib.Cloth(sc) for sc in scs]
+    for clear in (None, 1, 2, None):
+        for i, (cl, sc) in enumerate(zip(cls, scs)):
+            v, t = (None, None) if i == clear else (sc.mesh_verts, sc.mesh_tris)
+            cl.set_mesh(v, t)
+            cloth_lib.capi.cloth_batch_set_mesh(b.h, i, v, t)
+        b.step(3)
+        for i, cl in enumerate(cls):
+            cl.step(3)
+            (pa, va), (pb, vb) = b.read(i), cl.read()
+            np.testing.assert_array_equal(pa, pb)
+            np.testing.assert_array_equal(va, vb)
+    b.close()
+    for cl in cls:
+        cl.close()
