@@ -306,9 +306,10 @@ void cloth_batch_destroy(ClothBatch *b);
  * velocities.  The contact set of every substep is frozen at the one the
  * forward pass finds (the response is differentiated as a smooth map of the
  * start point and the path direction).  The forward pass stores the state
- * every checkpoint_every steps; the backward pass recomputes one segment at
- * a time into one of two slot sets while the previous segment is reversed,
- * so device memory grows as nsteps/checkpoint_every states plus
+ * every checkpoint_every steps and records the last two segments into the two
+ * slot sets; the backward pass starts from those and recomputes the earlier
+ * segments, one at a time into a set that has been reversed (a second backward
+ * pass recomputes all but up to two segments in all), so device memory grows as nsteps/checkpoint_every states plus
  * 2 x (checkpoint_every x substeps + 1) slots of 19 planes.  The forward and
  * backward passes run as CUDA graphs captured on first use (rebuilt after
  * cloth_set_mesh) unless the cloth has CLOTH_FLAG_NO_GRAPH; the backward

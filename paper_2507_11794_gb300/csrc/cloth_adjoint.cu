@@ -89,21 +89,20 @@ __device__ __forceinline__ void contact_adj(const StepParams &p, const float *__
     lF[o] = sc * q0; lF[st + o] = sc * q1; lF[2 * st + o] = sc * q2;
 }
 
-// Adjoint of one spring seen from its owner o (forward spring o -> e):
-// mu = lF_o - lF_e; returns gd = (dF/dd)^T mu, gv = (dF/ddv)^T mu and the
-// ks / kd gradient terms.
-__device__ __forceinline__ void spring_adj(const float *xo, const float *vo, const float *xe, const float *ve,
+// Adjoint of one spring seen from its end i (the other end n): mu = lF_i - lF_n;
+// returns gd = (dF/dd)^T mu, gv = (dF/ddv)^T mu for d = x_n - x_i, and the
+// ks / kd gradient terms.  Seen from the other end d, dv and mu change sign,
+// so gd and gv do, exactly, and the gradients stay: it does not matter which
+// end owns the spring.
+__device__ __forceinline__ void spring_adj(const float *xi, const float *vi, const float *xn, const float *vn,
                                            const float *mu, float ks, float kd, float L0, float gd[3], float gv[3],
                                            float &gks, float &gkd)
 {
-    const float dx = xe[0] - xo[0], dy = xe[1] - xo[1], dz = xe[2] - xo[2];
+    const float dx = xn[0] - xi[0], dy = xn[1] - xi[1], dz = xn[2] - xi[2];
     const float l2 = dx * dx + dy * dy + dz * dz;
-    gd[0] = gd[1] = gd[2] = gv[0] = gv[1] = gv[2] = 0.0f;
-    gks = gkd = 0.0f;
-    if (!(l2 > 1e-24f)) return;
-    const float il = rsqrtf(l2), l = l2 * il;
+    const float il = l2 > 1e-24f ? rsqrtf(l2) : 0.0f, l = l2 * il;
     const float ux = dx * il, uy = dy * il, uz = dz * il;
-    const float dvx = ve[0] - vo[0], dvy = ve[1] - vo[1], dvz = ve[2] - vo[2];
+    const float dvx = vn[0] - vi[0], dvy = vn[1] - vi[1], dvz = vn[2] - vi[2];
     const float ud = ux * dvx + uy * dvy + uz * dvz;
     const float um = ux * mu[0] + uy * mu[1] + uz * mu[2];
     const float phi = ks * (l - L0) + kd * ud;
@@ -122,64 +121,56 @@ __device__ __forceinline__ void spring_adj(const float *xo, const float *vo, con
 // lane q (0..3) of the node's group of four lanes: the lane takes springs
 // u = q, q + 4, q + 8 of the node's twelve in the order (owned d, incoming d,
 // owned d + 1, ...), so lanes 0 and 2 take owned springs and write their
-// ks / kd gradients, lanes 1 and 3 incoming ones.  xs is the substep's start
-// state, lF its force adjoints (all nodes).  Returns the lane's part of the
-// adjoints of the node's start position (gx) and velocity (gv).  Loads are
-// issued unconditionally (a missing neighbour reads the node itself) so that
-// the lane's gathers overlap; a missing spring's terms are discarded.
+// ks / kd gradients, lanes 1 and 3 incoming ones; all compute them from their
+// own end, so the warp does not diverge (with one branch for each it issued
+// both: 2.04M warp instructions a launch on 16,384 nodes).  xs is the substep's
+// start state, lF its force adjoints (all nodes).  Returns the lane's part of
+// the adjoints of the node's start position (gx) and velocity (gv).  Loads are
+// issued unconditionally (a missing neighbour reads the node itself: d = 0,
+// whose terms are 0) so that the lane's gathers overlap.
 __device__ __forceinline__ void spring_adj_lane(const StepParams &p, const float *__restrict__ xs,
-                                                const float *__restrict__ lF, long long o, int r, int c, int q,
+                                                const float *__restrict__ lF, unsigned o, int r, int c, int q,
                                                 double *__restrict__ gks, double *__restrict__ gkd, float gx[3],
                                                 float gv[3])
 {
-    const long long st = p.stride;
-    const float xi[3] = {xs[o], xs[st + o], xs[2 * st + o]};
-    const float vi[3] = {xs[3 * st + o], xs[4 * st + o], xs[5 * st + o]};
-    const float fi[3] = {lF[o], lF[st + o], lF[2 * st + o]};
+    const unsigned st = (unsigned)p.stride;  // six planes are below 2^32 floats
+    const float xi[3] = {xs[o], xs[st + o], xs[2u * st + o]};
+    const float vi[3] = {xs[3u * st + o], xs[4u * st + o], xs[5u * st + o]};
+    const float fi[3] = {lF[o], lF[st + o], lF[2u * st + o]};
     const bool own = (q & 1) == 0;
-    float xn[3][3], vn[3][3], ln[3][3], ksn[3], kdn[3];
+    const int sgn = own ? 1 : -1;
+    float xn[3][3], vn[3][3], ln[3][3], ksn[3], kdn[3], L0[3];
     double sk[3], sd[3];
     bool ok[3];
-    int dd[3];
+    unsigned so[3];
 #pragma unroll
     for (int t = 0; t < 3; t++) {
         const int d = (q >> 1) + 2 * t;
-        dd[t] = d;
-        const int r2 = own ? r + dev_dr(d) : r - dev_dr(d);
-        const int c2 = own ? c + dev_dc(d) : c - dev_dc(d);
+        const int r2 = r + sgn * dev_dr(d), c2 = c + sgn * dev_dc(d);
         ok[t] = r2 >= 0 && r2 < p.ny && c2 >= 0 && c2 < p.nx;
-        const long long e = ok[t] ? (long long)r2 * p.pitch + c2 : o;
-        xn[t][0] = xs[e]; xn[t][1] = xs[st + e]; xn[t][2] = xs[2 * st + e];
-        vn[t][0] = xs[3 * st + e]; vn[t][1] = xs[4 * st + e]; vn[t][2] = xs[5 * st + e];
-        ln[t][0] = lF[e]; ln[t][1] = lF[st + e]; ln[t][2] = lF[2 * st + e];
-        const long long so = d * st + (own ? o : e);  // the spring's slot: its owner's offset
-        ksn[t] = p.ks_slot[so];
-        kdn[t] = p.kd_slot[so];
-        sk[t] = own ? gks[so] : 0.0;
-        sd[t] = own ? gkd[so] : 0.0;
+        const unsigned e = ok[t] ? (unsigned)(r2 * p.pitch + c2) : o;
+        xn[t][0] = xs[e]; xn[t][1] = xs[st + e]; xn[t][2] = xs[2u * st + e];
+        vn[t][0] = xs[3u * st + e]; vn[t][1] = xs[4u * st + e]; vn[t][2] = xs[5u * st + e];
+        ln[t][0] = lF[e]; ln[t][1] = lF[st + e]; ln[t][2] = lF[2u * st + e];
+        so[t] = (unsigned)d * st + (own ? o : e);  // the spring's slot: its owner's offset
+        ksn[t] = p.ks_slot[so[t]];
+        kdn[t] = p.kd_slot[so[t]];
+        sk[t] = own ? gks[so[t]] : 0.0;
+        sd[t] = own ? gkd[so[t]] : 0.0;
+        L0[t] = (q >> 1) ? p.L0[2 * t + 1] : p.L0[2 * t];
     }
     gx[0] = gx[1] = gx[2] = gv[0] = gv[1] = gv[2] = 0.0f;
 #pragma unroll
     for (int t = 0; t < 3; t++) {
-        const int d = dd[t];
         float a[3], b[3], g1, g2;
-        if (own) {
-            const float mu[3] = {fi[0] - ln[t][0], fi[1] - ln[t][1], fi[2] - ln[t][2]};
-            spring_adj(xi, vi, xn[t], vn[t], mu, ksn[t], kdn[t], p.L0[d], a, b, g1, g2);
-            if (ok[t]) {
-                gx[0] -= a[0]; gx[1] -= a[1]; gx[2] -= a[2];
-                gv[0] -= b[0]; gv[1] -= b[1]; gv[2] -= b[2];
-                // per-spring sums over the substeps in double: FP64 only in these reductions
-                gks[d * st + o] = sk[t] + (double)g1;
-                gkd[d * st + o] = sd[t] + (double)g2;
-            }
-        } else {
-            const float mu[3] = {ln[t][0] - fi[0], ln[t][1] - fi[1], ln[t][2] - fi[2]};
-            spring_adj(xn[t], vn[t], xi, vi, mu, ksn[t], kdn[t], p.L0[d], a, b, g1, g2);
-            if (ok[t]) {
-                gx[0] += a[0]; gx[1] += a[1]; gx[2] += a[2];
-                gv[0] += b[0]; gv[1] += b[1]; gv[2] += b[2];
-            }
+        const float mu[3] = {fi[0] - ln[t][0], fi[1] - ln[t][1], fi[2] - ln[t][2]};
+        spring_adj(xi, vi, xn[t], vn[t], mu, ksn[t], kdn[t], L0[t], a, b, g1, g2);
+        gx[0] -= a[0]; gx[1] -= a[1]; gx[2] -= a[2];
+        gv[0] -= b[0]; gv[1] -= b[1]; gv[2] -= b[2];
+        if (own && ok[t]) {
+            // per-spring sums over the substeps in double: FP64 only in these reductions
+            gks[so[t]] = sk[t] + (double)g1;
+            gkd[so[t]] = sd[t] + (double)g2;
         }
     }
 }
@@ -223,7 +214,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_kernel(const StepParams p, co
     float l[3], m[3];
     if (SPRING) {
         const unsigned gm = 0xFu << (threadIdx.x & 28u);  // the group's lanes
-        spring_adj_lane(p, a.xs_s, a.lF_s, o, r, c, q, a.gks, a.gkd, l, m);
+        spring_adj_lane(p, a.xs_s, a.lF_s, (unsigned)o, r, c, q, a.gks, a.gkd, l, m);
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             l[k] += __shfl_xor_sync(gm, l[k], 1);
@@ -255,12 +246,12 @@ __global__ void copy_planes_kernel(const float4 *__restrict__ src, float4 *__res
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x)
         dst[i] = src[i];
 }
-// Start of a segment's recompute: the substep counter, and the hit bits of
-// all its substeps cleared.
-__global__ void segment_begin_kernel(DevCtrl *ctrl, unsigned long long k, uint32_t *bits, long long nwords)
+// Start of a recorded segment: the hit bits of all its substeps cleared and,
+// for a recompute (set_k), the substep counter.
+__global__ void segment_begin_kernel(DevCtrl *ctrl, int set_k, unsigned long long k, uint32_t *bits, long long nwords)
 {
     const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i0 == 0) ctrl_set_k(ctrl, k);
+    if (i0 == 0 && set_k) ctrl_set_k(ctrl, k);
     for (long long i = i0; i < nwords; i += (long long)gridDim.x * blockDim.x) bits[i] = 0u;
 }
 
@@ -325,10 +316,12 @@ struct ClothRollout {
     float *final_state = nullptr;          // 6 planes
     int *map = nullptr;                    // canonical spring -> slot
     bool forward_done = false;
-    // the forward chain and the reverse pass as CUDA graphs (captured on first
-    // use; rebuilt when the cloth's kernel parameters change)
-    cudaGraphExec_t fwd_graph = nullptr, bwd_graph = nullptr;
-    unsigned long long fwd_gen = 0, bwd_gen = 0;
+    bool slots_hold_last = false;          // the slot sets hold the last segments as the forward pass recorded them
+    // the forward chain and the reverse pass (without and with slots_hold_last)
+    // as CUDA graphs (captured on first use; rebuilt when the cloth's kernel
+    // parameters change)
+    cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};
+    unsigned long long graph_gen[3] = {0, 0, 0};
 };
 
 namespace {
@@ -381,27 +374,6 @@ cudaError_t copy_planes(const float *src, float *dst, long long nfloats, cudaStr
     return cudaGetLastError();
 }
 
-// The forward chain from the restored initial state: a checkpoint before
-// every segment, the segment's substeps (the cloth's own launches), and a
-// copy of the final state.
-cudaError_t enqueue_forward(ClothRollout *ro, cudaStream_t s)
-{
-    ClothHandle *h = ro->h;
-    const long long st = h->stride;
-    cudaError_t e = cudaSuccess;
-    for (int g = 0; g < ro->nseg && e == cudaSuccess; g++) {
-        e = copy_planes(cur_state(h, ro->kseg[g]), ro->ckpt + (size_t)g * 6 * st, 6 * st, s);
-        const int n = seg_steps(ro, g) * h->desc.substeps;
-        for (int q = 0; q < n && e == cudaSuccess; q++) {
-            StepParams p = h->params;
-            p.parity = (int)((ro->kseg[g] + (unsigned long long)q) & 1ull);
-            e = launch_substep(p, s);
-        }
-    }
-    if (e == cudaSuccess) e = copy_planes(cur_state(h, ro->k_final), ro->final_state, 6 * st, s);
-    return e;
-}
-
 // Slot j of recompute set b (segments alternate between the two sets).
 float *seg_slot(const ClothRollout *ro, int b, int j)
 {
@@ -412,13 +384,13 @@ uint32_t *seg_bits(const ClothRollout *ro, int b, int j)
     return ro->cbits + ((size_t)b * ro->seg_slots + (size_t)j) * (size_t)(ro->h->stride / 32);
 }
 
-// Recompute of segment g from its checkpoint into slot set g & 1, with the
-// substep kernels redirected: substep j reads slot j (the checkpoint for
-// j = 0) and writes slot j + 1, its post-integration velocity and, for the
-// nodes that hit, the response data into slot j; every substep's start state
-// stays in place without copies and the cloth's state buffers are not
-// touched.
-cudaError_t recompute_segment(ClothRollout *ro, int g, cudaStream_t s)
+// Segment g from its checkpoint into slot set g & 1, with the substep kernels
+// redirected: substep j reads slot j (the checkpoint for j = 0) and writes
+// slot j + 1, its post-integration velocity and, for the nodes that hit, the
+// response data into slot j; every substep's start state stays in place without
+// copies and the cloth's state buffers are not touched.  set_k: a recompute,
+// which starts from the segment's substep counter.
+cudaError_t record_segment(ClothRollout *ro, int g, bool set_k, cudaStream_t s)
 {
     ClothHandle *h = ro->h;
     const long long st = h->stride;
@@ -428,7 +400,7 @@ cudaError_t recompute_segment(ClothRollout *ro, int g, cudaStream_t s)
     const StepParams &p = h->params;
     const long long nwords = (long long)nsub * (st / 32);
     const int zb = nblk(nwords, 256);
-    segment_begin_kernel<<<zb < 1 ? 1 : (zb > 1024 ? 1024 : zb), 256, 0, s>>>(h->ctrl, kg, seg_bits(ro, b, 0),
+    segment_begin_kernel<<<zb < 1 ? 1 : (zb > 1024 ? 1024 : zb), 256, 0, s>>>(h->ctrl, set_k, kg, seg_bits(ro, b, 0),
                                                                                nwords);
     cudaError_t e = cudaGetLastError();
     for (int j = 0; j < nsub && e == cudaSuccess; j++) {
@@ -451,6 +423,37 @@ cudaError_t recompute_segment(ClothRollout *ro, int g, cudaStream_t s)
         }
         e = launch_substep(q, s);
     }
+    return e;
+}
+
+// The forward chain from the restored initial state: a checkpoint before
+// every segment, the segment's substeps (the cloth's own launches), and a copy
+// of the final state.  The last two segments, the first that the reverse pass
+// needs, are recorded into the two slot sets as they run, so it has nothing to
+// recompute for them.
+cudaError_t enqueue_forward(ClothRollout *ro, cudaStream_t s)
+{
+    ClothHandle *h = ro->h;
+    const long long st = h->stride;
+    cudaError_t e = cudaSuccess;
+    const float *cur = cur_state(h, ro->kseg[0]);
+    for (int g = 0; g < ro->nseg && e == cudaSuccess; g++) {
+        e = copy_planes(cur, ro->ckpt + (size_t)g * 6 * st, 6 * st, s);
+        const int n = seg_steps(ro, g) * h->desc.substeps;
+        if (g + 2 >= ro->nseg) {
+            if (e == cudaSuccess) e = record_segment(ro, g, false, s);
+            cur = seg_slot(ro, g & 1, n);
+            continue;
+        }
+        for (int q = 0; q < n && e == cudaSuccess; q++) {
+            StepParams p = h->params;
+            p.parity = (int)((ro->kseg[g] + (unsigned long long)q) & 1ull);
+            e = launch_substep(p, s);
+        }
+        cur = cur_state(h, ro->kseg[g + 1]);
+    }
+    if (e == cudaSuccess) e = copy_planes(cur, ro->final_state, 6 * st, s);
+    if (e == cudaSuccess) e = copy_planes(cur, cur_state(h, ro->k_final), 6 * st, s);
     return e;
 }
 
@@ -502,8 +505,9 @@ cudaError_t reverse_segment(ClothRollout *ro, int g, cudaStream_t s)
 // The reverse of segment g waits for its recompute; the recompute of
 // segment g - 1 runs meanwhile (into the other slot set) and the one of
 // g - 2 waits until the reverse of g has released its set.  Both chains are
-// latency-bound and occupy few SMs, so they overlap.
-cudaError_t enqueue_backward(ClothRollout *ro, cudaStream_t s)
+// latency-bound and occupy few SMs, so they overlap.  recorded: the slot sets
+// hold the last two segments from the forward pass.
+cudaError_t enqueue_backward(ClothRollout *ro, bool recorded, cudaStream_t s)
 {
     cudaStream_t v = ro->side;
     cudaError_t e = cudaEventRecord(ro->ev_fork, s);
@@ -511,9 +515,11 @@ cudaError_t enqueue_backward(ClothRollout *ro, cudaStream_t s)
     if (e != cudaSuccess) return e;
     for (int g = ro->nseg - 1; g >= 0 && e == cudaSuccess; g--) {
         if (g + 2 < ro->nseg) e = cudaStreamWaitEvent(s, ro->ev_rev[g & 1], 0);
-        if (e == cudaSuccess) e = recompute_segment(ro, g, s);
-        if (e == cudaSuccess) e = cudaEventRecord(ro->ev_rec[g & 1], s);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(v, ro->ev_rec[g & 1], 0);
+        if (!(recorded && g + 2 >= ro->nseg)) {
+            if (e == cudaSuccess) e = record_segment(ro, g, true, s);
+            if (e == cudaSuccess) e = cudaEventRecord(ro->ev_rec[g & 1], s);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(v, ro->ev_rec[g & 1], 0);
+        }
         if (e == cudaSuccess) e = reverse_segment(ro, g, v);
         if (e == cudaSuccess) e = cudaEventRecord(ro->ev_rev[g & 1], v);
     }
@@ -544,16 +550,17 @@ cudaError_t capture_graph(ClothHandle *h, cudaGraphExec_t *exec, F &&body)
 
 // Runs the forward chain or the reverse pass on s, through a cached graph
 // unless the cloth was created with CLOTH_FLAG_NO_GRAPH.
-cudaError_t run_pass(ClothRollout *ro, bool backward, cudaStream_t s)
+enum { PASS_FORWARD = 0, PASS_BACKWARD = 1, PASS_BACKWARD_RECORDED = 2 };
+cudaError_t run_pass(ClothRollout *ro, int pass, cudaStream_t s)
 {
     ClothHandle *h = ro->h;
-    auto body = [ro, backward](cudaStream_t cs) {
-        return backward ? enqueue_backward(ro, cs) : enqueue_forward(ro, cs);
+    auto body = [ro, pass](cudaStream_t cs) {
+        return pass == PASS_FORWARD ? enqueue_forward(ro, cs)
+                                    : enqueue_backward(ro, pass == PASS_BACKWARD_RECORDED, cs);
     };
     if (h->desc.flags & CLOTH_FLAG_NO_GRAPH) return body(s);
-    cudaGraphExec_t &gx = backward ? ro->bwd_graph : ro->fwd_graph;
-    unsigned long long &gen = backward ? ro->bwd_gen : ro->fwd_gen;
-    if (gx && gen != h->params_gen) {
+    cudaGraphExec_t &gx = ro->graph[pass];
+    if (gx && ro->graph_gen[pass] != h->params_gen) {
         cudaGraphExecDestroy(gx);
         gx = nullptr;
     }
@@ -563,7 +570,7 @@ cudaError_t run_pass(ClothRollout *ro, bool backward, cudaStream_t s)
             gx = nullptr;
             return e;
         }
-        gen = h->params_gen;
+        ro->graph_gen[pass] = h->params_gen;
     }
     return cudaGraphLaunch(gx, s);
 }
@@ -697,7 +704,9 @@ int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd
     RTRY(h, launch_aos_to_soa(ro->x0, d_v0 ? d_v0 : ro->v0, h->state, h->state + 6 * st, st, h->n, h->desc.nx,
                               h->pitch, h->ctrl, s),
          "initial state");
-    RTRY(h, run_pass(ro, false, s), "forward chain");
+    ro->slots_hold_last = false;
+    RTRY(h, run_pass(ro, PASS_FORWARD, s), "forward chain");
+    ro->slots_hold_last = true;
     h->substeps_done = (long long)ro->k_final;
     if (d_pos_out || d_vel_out)
         RTRY(h, launch_soa_to_aos(h->state, h->state + 6 * st, st, h->n, h->desc.nx, h->pitch, h->ctrl, d_pos_out,
@@ -723,7 +732,9 @@ int cloth_rollout_backward(ClothRollout *ro, const float *d_gpos, const float *d
     aos_planes_kernel<<<nblk(n, 256), 256, 0, s>>>(d_gpos, n, nx, h->pitch, st, lx);
     aos_planes_kernel<<<nblk(n, 256), 256, 0, s>>>(d_gvel, n, nx, h->pitch, st, lv);
     RTRY(h, cudaGetLastError(), "load output adjoints");
-    RTRY(h, run_pass(ro, true, s), "reverse pass");
+    const bool recorded = ro->slots_hold_last;
+    ro->slots_hold_last = recorded && ro->nseg <= 2;  // earlier segments' recomputes overwrite the sets
+    RTRY(h, run_pass(ro, recorded ? PASS_BACKWARD_RECORDED : PASS_BACKWARD, s), "reverse pass");
     if (d_gv0) planes_aos_kernel<<<nblk(n, 256), 256, 0, s>>>(lv, n, nx, h->pitch, st, d_gv0);
     if (d_gks && ro->S > 0) gather_kernel<<<nblk(ro->S, 256), 256, 0, s>>>(ro->gslot, ro->map, ro->S, d_gks);
     if (d_gkd && ro->S > 0)
@@ -741,8 +752,8 @@ void cloth_rollout_destroy(ClothRollout *ro)
     if (!ro) return;
     if (ro->h) cudaStreamSynchronize(ro->h->stream);
     if (ro->side) cudaStreamSynchronize(ro->side);
-    if (ro->fwd_graph) cudaGraphExecDestroy(ro->fwd_graph);
-    if (ro->bwd_graph) cudaGraphExecDestroy(ro->bwd_graph);
+    for (cudaGraphExec_t g : ro->graph)
+        if (g) cudaGraphExecDestroy(g);
     cudaFree(ro->x0);
     cudaFree(ro->v0);
     cudaFree(ro->ckpt);

@@ -154,3 +154,34 @@ def test_batch_changes_form(cloth_lib):
     b.close()
     for cl in cls:
         cl.close()
+
+
+@pytest.mark.parametrize("steps,every", [(3, 1), (3, 2), (4, 2), (5, 2), (6, 6)])
+@pytest.mark.parametrize("graph", [True, False])
+def test_rollout_reverse_twice(cloth_lib, steps, every, graph):
+    """The forward pass records the last two segments; a second reverse pass
+    (with more than two, of recomputed ones) and one after another forward
+    pass with other inputs in between give the same gradients."""
+    import torch
+    from paper_2507_11794_gb300.rollout import Rollout
+    sc = per_spring(scene(23, 19, mesh=True, wind=False))
+    with cloth_lib.Cloth(sc, flags=0 if graph else cloth_lib.capi.CLOTH_FLAG_NO_GRAPH) as cl:
+        ro = Rollout(cl, steps, every)
+        args = [torch.tensor(a, device="cuda", requires_grad=True) for a in (sc.ks_spring, sc.kd_spring, sc.init_vel)]
+
+        def loss():
+            pos, vel = ro(*args)
+            return (pos ** 2).sum() + vel.sum()
+
+        L = loss()
+        first = torch.autograd.grad(L, args, retain_graph=True)
+        again = torch.autograd.grad(L, args)
+        state = cl.read()
+        with torch.no_grad():
+            ro(args[0] * 1.1, args[1], args[2])
+        third = torch.autograd.grad(loss(), args)
+        after = cl.read()
+        ro.close()
+    for a, b, c in zip(first, again, third):
+        assert torch.equal(a, b) and torch.equal(a, c)
+    assert np.array_equal(state[0], after[0]) and np.array_equal(state[1], after[1])
