@@ -457,36 +457,60 @@ int cloth_set_mesh(ClothHandle *h, const float *verts, int32_t nverts, const int
     if (rc) return rc;
     if (ntris < 0 || nverts < 0) return fail(CLOTH_ERR_BAD_MESH, "negative mesh size");
     if (ntris > 0 && (!verts || !tris || nverts < 1)) return fail(CLOTH_ERR_BAD_MESH, "missing mesh arrays");
-    for (long long i = 0; i < 3 * (long long)ntris; i++)
-        if (tris[i] < 0 || tris[i] >= nverts)
-            return fail(CLOTH_ERR_BAD_MESH, "triangle index %d at %lld out of range [0, %d)", tris[i], i, nverts);
-    for (long long i = 0; i < 3 * (long long)nverts && ntris > 0; i++)
-        if (!isfinite(verts[i])) return fail(CLOTH_ERR_BAD_MESH, "non-finite vertex coordinate at %lld", i);
+    // A mesh is looked over on the host when it is small, on the device (beside
+    // the upload it needs anyway) when it is not: a triangle takes the host about
+    // 20 ns, 1.7 of 1.9 ms on 81,920 triangles; the scan's launch, read-back and
+    // wait cost what some 4,000 take.
+    const bool scan = ntris >= 4096;
+    auto bad_index = [&](long long i) {
+        return fail(CLOTH_ERR_BAD_MESH, "triangle index %d at %lld out of range [0, %d)", tris[i], i, nverts);
+    };
+    auto bad_vertex = [&](long long i) { return fail(CLOTH_ERR_BAD_MESH, "non-finite vertex coordinate at %lld", i); };
+    if (!scan) {
+        for (long long i = 0; i < 3 * (long long)ntris; i++)
+            if (tris[i] < 0 || tris[i] >= nverts) return bad_index(i);
+        for (long long i = 0; i < 3 * (long long)nverts && ntris > 0; i++)
+            if (!isfinite(verts[i])) return bad_vertex(i);
+    }
     DeviceScope ds(h->device);
     CTRY(h, cudaStreamSynchronize(h->stream), "synchronize");
     DevGrid g{};
     if (ntris > 0) {
-        if (grid_params(verts, tris, ntris, &g.h, g.origin, g.dims, &g.inv) != 0)
-            return fail(CLOTH_ERR_BAD_MESH, "grid parameters");
-        for (int a = 0; a < 3; a++) {
-            g.lo[a] = INFINITY;
-            g.hi[a] = -INFINITY;
-        }
-        for (long long i = 0; i < 3 * (long long)ntris; i++)
+        if (!scan) {
+            if (grid_params(verts, tris, ntris, &g.h, g.origin, g.dims, &g.inv) != 0)
+                return fail(CLOTH_ERR_BAD_MESH, "grid parameters");
             for (int a = 0; a < 3; a++) {
-                const float x = verts[3 * (long long)tris[i] + a];
-                g.lo[a] = fminf(g.lo[a], x);
-                g.hi[a] = fmaxf(g.hi[a], x);
+                g.lo[a] = INFINITY;
+                g.hi[a] = -INFINITY;
             }
+            for (long long i = 0; i < 3 * (long long)ntris; i++)
+                for (int a = 0; a < 3; a++) {
+                    const float x = verts[3 * (long long)tris[i] + a];
+                    g.lo[a] = fminf(g.lo[a], x);
+                    g.hi[a] = fmaxf(g.hi[a], x);
+                }
+        }
         float *dv = nullptr;
         int *dt = nullptr;
+        MeshInfo m;
+        m.bad_index = m.bad_vertex = -1;
         cudaError_t e = cudaMalloc(&dv, sizeof(float) * 3 * (size_t)nverts);
         if (e == cudaSuccess) e = cudaMalloc(&dt, sizeof(int) * 3 * (size_t)ntris);
         if (e == cudaSuccess) e = upload(dv, verts, sizeof(float) * 3 * (size_t)nverts, h->stream);
         if (e == cudaSuccess) e = upload(dt, tris, sizeof(int) * 3 * (size_t)ntris, h->stream);
-        if (e == cudaSuccess) e = grid_build(dv, dt, ntris, &g, h->stream);
+        if (e == cudaSuccess && scan) {
+            e = mesh_scan(dv, nverts, dt, ntris, &m, h->stream);
+            if (e == cudaSuccess && m.bad_index < 0 && m.bad_vertex < 0) {
+                grid_from_sides(m.sum, ntris, m.lo, m.hi, &g.h, g.origin, g.dims, &g.inv);
+                memcpy(g.lo, m.lo, sizeof(g.lo));
+                memcpy(g.hi, m.hi, sizeof(g.hi));
+            }
+        }
+        const bool good = m.bad_index < 0 && m.bad_vertex < 0;
+        if (e == cudaSuccess && good) e = grid_build(dv, dt, ntris, &g, h->stream);
         cudaFree(dv);
         cudaFree(dt);
+        if (e == cudaSuccess && !good) return m.bad_index >= 0 ? bad_index(m.bad_index) : bad_vertex(m.bad_vertex);
         if (e == cudaErrorInvalidValue) {
             cudaGetLastError();
             return fail(CLOTH_ERR_BAD_MESH, "mesh needs more than 2^31 grid entries");

@@ -11,6 +11,8 @@
 //      that the lists are ascending and the result is deterministic.
 #include <math.h>
 #include <stdio.h>
+#include <stdlib.h>
+#include <string.h>
 
 #include "cloth_internal.h"
 
@@ -197,16 +199,30 @@ __device__ __forceinline__ uint2 filter_side(float a, float e1, float e2, float 
     return make_uint2((unsigned)fminf(fmaxf(lo, 0.0f), top), (unsigned)fminf(fmaxf(hi, 0.0f), top));
 }
 
-// Expand the sorted (cell, triangle) pairs into per-entry records read by the
-// narrow phase without an indirection: the triangle's plane and first cell,
-// and its filter words (its box; whether this is its first cell per axis).
-__global__ void expand_kernel(const float4 *__restrict__ rec, const int *__restrict__ tri_ids, long long n,
-                              const int *__restrict__ cell_start, long long ncells, int dx, int dy, float ox, float oy, float oz, float qs, float pad, float4 *__restrict__ etri,
-                              uint4 *__restrict__ efil)
+// Sorts each cell's triangle ids and expands the pairs into the per-entry
+// records that the narrow phase reads without an indirection: the triangle's
+// plane and first cell, and its filter words (its box; whether this is its
+// first cell per axis).  One thread per entry of the unsorted lists: its place
+// is the number of smaller ids in its cell.  (An insertion sort by one thread
+// per cell took 52 us of the build's 94 on 81,920 triangles.)
+__global__ void expand_kernel(const float4 *__restrict__ rec, const int *__restrict__ unsorted, long long n,
+                              const int *__restrict__ cell_start, long long ncells, int dx, int dy, float ox, float oy, float oz, float qs, float pad, int *__restrict__ tri_ids,
+                              float4 *__restrict__ etri, uint4 *__restrict__ efil)
 {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const int t = tri_ids[e];
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int t = unsorted[i];
+    // the entry's cell: the last whose list starts at or before i
+    long long lo = 0, hi = ncells;
+    while (hi - lo > 1) {
+        const long long mid = (lo + hi) >> 1;
+        if (cell_start[mid] <= i) lo = mid;
+        else hi = mid;
+    }
+    const int b = cell_start[lo], end = cell_start[lo + 1];
+    long long e = b;
+    for (int j = b; j < end; j++) e += unsorted[j] < t;  // a cell lists a triangle once
+    tri_ids[e] = t;
     const float4 A = rec[3 * t], B = rec[3 * t + 1], C = rec[3 * t + 2];
     etri[3 * e] = A;
     etri[3 * e + 1] = B;
@@ -214,13 +230,6 @@ __global__ void expand_kernel(const float4 *__restrict__ rec, const int *__restr
     const uint2 x = filter_side(A.x, B.x, C.x, ox, qs, pad);
     const uint2 y = filter_side(A.y, B.y, C.y, oy, qs, pad);
     const uint2 z = filter_side(A.z, B.z, C.z, oz, qs, pad);
-    // the entry's cell: the last whose list starts at or before e
-    long long lo = 0, hi = ncells;
-    while (hi - lo > 1) {
-        const long long mid = (lo + hi) >> 1;
-        if (cell_start[mid] <= e) lo = mid;
-        else hi = mid;
-    }
     const int cx = (int)(lo % dx), cy = (int)(lo / dx % dy), cz = (int)(lo / dx / dy);
     const unsigned first = (__float_as_int(A.w) == cx) | (__float_as_int(B.w) == cy) << 1 | (__float_as_int(C.w) == cz) << 2;
     efil[e] = make_uint4(GRID_FILTER_GUARD | x.y | y.y << 16, GRID_FILTER_GUARD | z.y | (GRID_FILTER_MAX - x.x) << 16,
@@ -258,14 +267,89 @@ __global__ void query_kernel(const float4 *__restrict__ rec, const int *__restri
 
 inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
+// First look at a mesh on the device (see mesh_scan): the smallest position of an
+// index outside [0, nv) and of a non-finite coordinate, the box of the
+// triangles' vertices (floats in an order-preserving integer form) and each
+// triangle's longest box side, in double.  A triangle with a bad index
+// contributes nothing.
+struct MeshScan {
+    unsigned long long bad_index, bad_vertex;
+    unsigned lo[3], hi[3];
+};
+__device__ __forceinline__ unsigned ordered(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__global__ void __launch_bounds__(256) mesh_scan_kernel(const float *__restrict__ verts, int nv,
+                                                        const int *__restrict__ tris, int nt,
+                                                        double *__restrict__ side, MeshScan *out)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    if (t < nt) {
+        bool ok = true;
+        int id[3];
+        for (int j = 2; j >= 0; j--) {
+            id[j] = tris[3ll * t + j];
+            if (id[j] < 0 || id[j] >= nv) {
+                ok = false;
+                atomicMin(&out->bad_index, 3ull * t + j);
+            }
+        }
+        double s = 0.0;
+        if (ok) {
+            for (int j = 0; j < 3; j++)
+                for (int a = 0; a < 3; a++) {
+                    const float x = verts[3ll * id[j] + a];
+                    lo[a] = x < lo[a] ? x : lo[a];
+                    hi[a] = x > hi[a] ? x : hi[a];
+                }
+            for (int a = 0; a < 3; a++) {
+                const double e = (double)hi[a] - (double)lo[a];
+                s = e > s ? e : s;
+            }
+        }
+        side[t] = s;
+    }
+    for (int a = 0; a < 3; a++) {
+        const unsigned l = __reduce_min_sync(0xffffffffu, ordered(lo[a])), h = __reduce_max_sync(0xffffffffu, ordered(hi[a]));
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&out->lo[a], l);
+            atomicMax(&out->hi[a], h);
+        }
+    }
+    for (long long i = t; i < 3ll * nv; i += (long long)gridDim.x * blockDim.x)
+        if (!isfinite(verts[i])) atomicMin(&out->bad_vertex, (unsigned long long)i);
+}
+
 }  // namespace
+
+// h = (float)(2 * mean longest AABB side), the sides summed in double in
+// triangle order; origin = (float)(min - 1.5h); dims = floor(extent/h) + 4; the
+// cell size doubles while the grid would exceed 2^24 cells.
+void grid_from_sides(double sum, int nt, const float mn[3], const float mx[3], float *h_out, float origin[3],
+                     int dims[3], float *inv_out)
+{
+    float h = (float)(2.0 * (sum / (double)nt));
+    if (!(h > 0.0f)) h = 1.0f;
+    for (;;) {
+        long long cells = 1;
+        for (int a = 0; a < 3; a++) {
+            origin[a] = (float)((double)mn[a] - 1.5 * (double)h);
+            dims[a] = (int)floor(((double)mx[a] - (double)mn[a]) / (double)h) + 4;
+            cells *= dims[a];
+        }
+        if (cells <= (1ll << 24)) break;
+        h = h * 2.0f;
+    }
+    *h_out = h;
+    *inv_out = (float)(1.0 / (double)h);
+}
 
 int grid_params(const float *verts, const int32_t *tris, int32_t nt, float *h_out, float origin[3], int dims[3],
                 float *inv_out)
 {
-    // h = (float)(2 * mean longest AABB side), summed in double in triangle
-    // order; origin = (float)(min - 1.5h); dims = floor(extent/h) + 4; the cell
-    // size doubles while the grid would exceed 2^24 cells.
     if (nt <= 0) return -1;
     double sum = 0.0;
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
@@ -287,21 +371,54 @@ int grid_params(const float *verts, const int32_t *tris, int32_t nt, float *h_ou
         }
         sum += side;
     }
-    float h = (float)(2.0 * (sum / (double)nt));
-    if (!(h > 0.0f)) h = 1.0f;
-    for (;;) {
-        long long cells = 1;
-        for (int a = 0; a < 3; a++) {
-            origin[a] = (float)((double)mn[a] - 1.5 * (double)h);
-            dims[a] = (int)floor(((double)mx[a] - (double)mn[a]) / (double)h) + 4;
-            cells *= dims[a];
-        }
-        if (cells <= (1ll << 24)) break;
-        h = h * 2.0f;
-    }
-    *h_out = h;
-    *inv_out = (float)(1.0 / (double)h);
+    grid_from_sides(sum, nt, mn, mx, h_out, origin, dims, inv_out);
     return 0;
+}
+
+cudaError_t mesh_scan(const float *d_verts, int nv, const int *d_tris, int nt, MeshInfo *m, cudaStream_t s)
+{
+    // triangle sides first, then the scan's words, in one buffer; read back
+    // together and summed here in triangle order, which the cell size is
+    // defined by (a sum in another order could round to another float)
+    const size_t bytes = sizeof(double) * (size_t)nt + sizeof(MeshScan);
+    char *buf = nullptr;
+    char *host = (char *)malloc(bytes);
+    if (!host) return cudaErrorMemoryAllocation;
+    const MeshScan init = {~0ull, ~0ull, {~0u, ~0u, ~0u}, {0u, 0u, 0u}};
+    cudaError_t e = cudaMalloc(&buf, bytes);
+    MeshScan *scan = (MeshScan *)(buf + sizeof(double) * (size_t)nt);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(scan, &init, sizeof(init), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) {
+        mesh_scan_kernel<<<blocks_for(nt, 256), 256, 0, s>>>(d_verts, nv, d_tris, nt, (double *)buf, scan);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(host, buf, bytes, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(buf);
+    if (e != cudaSuccess) {
+        free(host);
+        return e;
+    }
+    MeshScan r;
+    memcpy(&r, host + sizeof(double) * (size_t)nt, sizeof(r));
+    m->bad_index = r.bad_index == ~0ull ? -1 : (long long)r.bad_index;
+    m->bad_vertex = r.bad_vertex == ~0ull ? -1 : (long long)r.bad_vertex;
+    auto plain = [](unsigned b) {
+        b = b & 0x80000000u ? b & 0x7fffffffu : ~b;
+        float x;
+        memcpy(&x, &b, sizeof(x));
+        return x;
+    };
+    for (int a = 0; a < 3; a++) {
+        m->lo[a] = plain(r.lo[a]);
+        m->hi[a] = plain(r.hi[a]);
+    }
+    const double *side = (const double *)host;
+    double sum = 0.0;
+    for (int t = 0; t < nt; t++) sum += side[t];
+    m->sum = sum;
+    free(host);
+    return cudaSuccess;
 }
 
 #define GTRY(x)                          \
@@ -318,6 +435,7 @@ cudaError_t grid_build(const float *d_verts, const int *d_tris, int nt, DevGrid 
     cudaError_t err = cudaSuccess;
     int4 *box_hi = nullptr;
     unsigned *cnt = nullptr, *cursor = nullptr, *sums = nullptr;
+    int *unsorted = nullptr;
     unsigned long long *total = nullptr;
     unsigned long long htotal = 0;
     const long long nc = (long long)g->dims[0] * g->dims[1] * g->dims[2];
@@ -352,6 +470,7 @@ cudaError_t grid_build(const float *d_verts, const int *d_tris, int nt, DevGrid 
     }
     g->nentries = (long long)htotal;
     GTRY(cudaMalloc(&g->tri_ids, sizeof(int) * (size_t)(htotal > 0 ? htotal : 1)));
+    GTRY(cudaMalloc(&unsorted, sizeof(int) * (size_t)(htotal > 0 ? htotal : 1)));
     cell_count_kernel<<<blocks_for(nt, 256), 256, 0, s>>>(g->tri, box_hi, nt, g->dims[0], g->dims[1], cnt);
     GTRY(cudaGetLastError());
     scan_reduce_kernel<<<(int)ntiles, SCAN_THREADS, 0, s>>>(cnt, nc, sums);
@@ -361,9 +480,7 @@ cudaError_t grid_build(const float *d_verts, const int *d_tris, int nt, DevGrid 
     scan_final_kernel<<<(int)ntiles, SCAN_THREADS, 0, s>>>(cnt, nc, sums, g->cell_start);
     GTRY(cudaGetLastError());
     cell_fill_kernel<<<blocks_for(nt, 256), 256, 0, s>>>(g->tri, box_hi, nt, g->dims[0], g->dims[1], g->cell_start,
-                                                         cursor, g->tri_ids);
-    GTRY(cudaGetLastError());
-    cell_sort_kernel<<<blocks_for(nc, 256), 256, 0, s>>>(g->cell_start, nc, g->tri_ids);
+                                                         cursor, unsorted);
     GTRY(cudaGetLastError());
     // records and filter words in one allocation
     GTRY(cudaMalloc(&g->etri, (sizeof(float4) * 3 + sizeof(uint4)) * (size_t)(htotal > 0 ? htotal : 1)));
@@ -374,10 +491,10 @@ cudaError_t grid_build(const float *d_verts, const int *d_tris, int nt, DevGrid 
         for (int a = 0; a < 3; a++)
             top = fmax(top, fmax(fabs((double)g->origin[a]), fabs((double)g->origin[a] + (double)g->dims[a] * g->h)));
         const float pad = (float)fmin(1.0 + ceil(4e-7 * top * g->qs), 40000.0);
-        expand_kernel<<<blocks_for((long long)htotal, 256), 256, 0, s>>>(g->tri, g->tri_ids, (long long)htotal,
+        expand_kernel<<<blocks_for((long long)htotal, 256), 256, 0, s>>>(g->tri, unsorted, (long long)htotal,
                                                                          g->cell_start, nc, g->dims[0], g->dims[1],
                                                                          g->origin[0], g->origin[1], g->origin[2],
-                                                                         g->qs, pad, g->etri, g->efil);
+                                                                         g->qs, pad, g->tri_ids, g->etri, g->efil);
         GTRY(cudaGetLastError());
     }
     GTRY(cudaStreamSynchronize(s));
@@ -386,6 +503,7 @@ done:
     cudaFree(cnt);
     cudaFree(cursor);
     cudaFree(sums);
+    cudaFree(unsorted);
     cudaFree(total);
     if (err != cudaSuccess) grid_free(g);
     return err;

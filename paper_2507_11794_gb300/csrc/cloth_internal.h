@@ -187,6 +187,18 @@ struct DevGrid {
 int grid_params(const float *verts, const int32_t *tris, int32_t nt, float *h, float origin[3], int dims[3],
                 float *inv);
 
+void grid_from_sides(double sum, int nt, const float mn[3], const float mx[3], float *h, float origin[3], int dims[3],
+                     float *inv);
+// What validation and the grid parameters need of a mesh, from device copies:
+// the smallest position of a bad index and of a non-finite coordinate (-1:
+// none), the box and the sum of the triangles' longest box sides.  Waits for s.
+struct MeshInfo {
+    long long bad_index, bad_vertex;
+    float lo[3], hi[3];
+    double sum;
+};
+cudaError_t mesh_scan(const float *d_verts, int nv, const int *d_tris, int nt, MeshInfo *m, cudaStream_t s);
+
 // Build the device grid from device copies of the mesh (d_verts, d_tris).
 // Allocates g->tri, g->cell_start, g->tri_ids; scratch is allocated and
 // freed inside.  Synchronises s.
