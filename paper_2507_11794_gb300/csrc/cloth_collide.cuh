@@ -654,9 +654,14 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
     const long long st = p.stride;
     const float *xs = (k & 1ull) ? p.state0 : p.state1;  // updated positions (written by the walk)
     const unsigned per_kind = (n + PER - 1u) / PER, nw = gridDim.x * COLL_WARPS;
-    const unsigned long long chunks = 3ull * per_kind;
+    const unsigned chunks = 3u * per_kind;  // three chunks of 32 edges per 32 nodes: far below 2^32
     const unsigned first = chunks < nw ? (unsigned)wib * gridDim.x + blockIdx.x : blockIdx.x * COLL_WARPS + wib;
-    for (unsigned long long c = first; c < chunks; c += nw) {
+    unsigned *next = p.ctrl->edge_next + (k & 1ull);
+    // every warp has a first chunk; the others go to whoever is free, since edges
+    // differ in their cells and hits (256 x 256 nodes are 1.3 chunks a warp: with
+    // c += nw the pass took two full rounds, 90 against 80 us per substep; lists
+    // of nodes keep c += nw, whose neighbours share an SM's L1: 4 % faster there)
+    for (unsigned c = first; c < chunks;) {
         const int kind = (int)(c / per_kind);
         const unsigned i = PER * (unsigned)(c % per_kind) + (unsigned)(lane / G);
         bool has = false, wide = false;
@@ -689,6 +694,10 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
             p.edge_hit[s.slot] = s.rec;
             nhit += s.rec.w > 0.0f ? 1u : 0u;
         }
+        if (chunks <= nw) break;
+        c = 0u;
+        if (lane == 0) c = nw + atomicAdd(next, 1u);
+        c = __shfl_sync(0xffffffffu, c, 0);
     }
 }
 __device__ __forceinline__ void edge_test_list(const StepParams &p, unsigned long long k, unsigned n, unsigned &ntest,

@@ -20,6 +20,7 @@ struct DevCtrl {
     // next substep uses.  Whoever sets k from outside zeroes both (ctrl_set_k).
     unsigned long long kc;
     unsigned int coll_count[2];
+    unsigned int edge_next[2]; // next chunk of the edge pass, by substep parity as coll_count
     unsigned int blocks_done; // completion counter (the atomic path's substeps without a mesh)
     unsigned int flags;       // CTRL_FLAG_* (sticky until set_state)
     // running collision statistics since create: listed nodes, candidate
@@ -248,6 +249,7 @@ __device__ __forceinline__ void ctrl_set_k(DevCtrl *ctrl, unsigned long long k)
     ctrl->kk[k & 1ull] = k;
     ctrl->kk[(k + 1ull) & 1ull] = k ? k - 1ull : 0ull;
     ctrl->coll_count[0] = ctrl->coll_count[1] = 0u;
+    ctrl->edge_next[0] = ctrl->edge_next[1] = 0u;
 }
 
 __device__ __forceinline__ unsigned grid_filter_coord(float x, float o, float qs)

@@ -569,6 +569,7 @@ __device__ __forceinline__ void coll_begin(DevCtrl *ctrl, unsigned long long &k,
 __device__ __forceinline__ void coll_end(DevCtrl *ctrl, unsigned long long k)
 {
     ctrl->coll_count[(k + 1ull) & 1ull] = 0u;
+    ctrl->edge_next[(k + 1ull) & 1ull] = 0u;
     ctrl_end_k(ctrl, k);
 }
 
