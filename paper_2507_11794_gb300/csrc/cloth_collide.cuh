@@ -640,10 +640,9 @@ struct EdgeHits {
 // owner] = (P, K), and the points of its hits 2 .. 1 + EDGE_MORE at
 // p.edge_more[(h - 2) * 3 * stride + kind * stride + owner].  Counts the
 // tested candidates and the edges that hit into ntest and nhit.  Measured on
-// 256 x 256 nodes over 81,920 triangles: the four kernels of a substep 151 ->
-// 80 us against one that searched shared memory for each candidate and walked
-// every box of more than 8 cells by the whole warp (137 us of it, 54M warp
-// instructions).
+// 256 x 256 nodes over 81,920 triangles: this kernel 137 -> 41 us (ncu) against
+// one that searched shared memory for each candidate and walked every box of
+// more than 8 cells by the whole warp (54M warp instructions, now 14M).
 constexpr int EDGE_MAXC = 18;  // cells of an edge's box one lane goes through
 template <int G>
 __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned long long k, unsigned n,
