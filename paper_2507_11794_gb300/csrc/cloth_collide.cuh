@@ -635,15 +635,17 @@ struct EdgeHits {
 // owns, (0,+1), (+1,0) and (+1,+1) from it (the triangulation's edges,
 // oriented from their upper-left endpoint), at the updated positions, so each
 // edge is tested once.  G lanes per edge as in the node pass; a warp's edges
-// are of one kind and of neighbouring owners.  Records per edge its first hit
+// are of one kind.  Records per edge its first hit
 // point (in candidate order) and its number of hits, p.edge_hit[kind * stride +
 // owner] = (P, K), and the points of its hits 2 .. 1 + EDGE_MORE at
 // p.edge_more[(h - 2) * 3 * stride + kind * stride + owner].  Counts the
-// tested candidates and the edges that hit into ntest and nhit.  Measured on
-// 256 x 256 nodes over 81,920 triangles: this kernel 137 -> 41 us (ncu) against
-// one that searched shared memory for each candidate and walked every box of
-// more than 8 cells by the whole warp (54M warp instructions, now 14M).
-constexpr int EDGE_MAXC = 18;  // cells of an edge's box one lane goes through
+// tested candidates and the edges that hit into ntest and nhit.  Against one
+// that searched shared memory for each candidate: 256 x 256 nodes lying on
+// 81,920 triangles 669 -> 329 us per step of cloth_step with its copies, falling
+// onto them (steps 150 to 250) 276 -> 271.  Where edges are long the time is
+// that of the slowest warp: a warp's edges from one place of the list made it
+// 309 and 367, from 32 places 346 and 258; up to 18 cells per lane 338 (falling).
+constexpr int EDGE_MAXC = 8;  // cells of an edge's box one lane goes through
 template <int G>
 __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned long long k, unsigned n,
                                                  unsigned &ntest, unsigned &nhit)
@@ -662,7 +664,11 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
     // of nodes keep c += nw, whose neighbours share an SM's L1: 4 % faster there)
     for (unsigned c = first; c < chunks;) {
         const int kind = (int)(c / per_kind);
-        const unsigned i = PER * (unsigned)(c % per_kind) + (unsigned)(lane / G);
+        // long edges come in clusters, so a warp takes pairs of neighbours from
+        // sixteen places of the list (a cluster in one warp held it for 100 us)
+        const unsigned cc0 = c % per_kind;
+        const unsigned i = G > 1 ? PER * cc0 + (unsigned)(lane / G)
+                                 : (unsigned)(lane / 2) * 2u * per_kind + 2u * cc0 + (unsigned)(lane % 2);
         bool has = false, wide = false;
         int ncell = 0;
         CollPath path = {};

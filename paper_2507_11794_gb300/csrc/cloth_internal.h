@@ -141,7 +141,7 @@ struct BatchArgs {
     const StepParams *params;  // one per cloth (device)
     const int4 *items;         // (cloth, strip x, strip y, cost), longest first
     int n_items;
-    unsigned *work;            // next item (re-armed by the last CTA)
+    unsigned *work;            // next item (re-armed by the collision kernel)
     DevCtrl *ctrl;             // shared substep counter and flags
     int *coll_list, *coll_cloth;
     unsigned *coll_count;
