@@ -234,8 +234,9 @@ int cloth_query_candidates(ClothHandle *h, const float *S, const float *E, int32
  * launches run back to back), and report the mean device
  * duration per launch in microseconds: walk_us for the force + integration
  * kernel (Algorithm 1 and Section 3), collide_us for the collision kernel
- * (Section 3 and Algorithm 2; 0 without a surface model).  The state
- * advances exactly as with cloth_step.  nsub in [1, 4096]; either output may
+ * (Section 3 and Algorithm 2; 0 without a surface model).  These two
+ * kernels run here also for small cloths, whose cloth_step runs a substep as one
+ * kernel.  The state advances exactly as with cloth_step.  nsub in [1, 4096]; either output may
  * be NULL.  Synchronises.  Errors: CLOTH_ERR_INVALID_ARG, CLOTH_ERR_CUDA,
  * and the flag errors of cloth_sync. */
 int cloth_profile_substeps(ClothHandle *h, int32_t nsub, float *walk_us, float *collide_us);
@@ -255,8 +256,8 @@ int cloth_compute_normals(ClothHandle *h, float *d_normals);
 /* Many independent cloths (each with its own grid, constants, pins and
  * surface model) stepped together: every substep is one persistent walk
  * launch over a (cloth, strip) work list sorted longest first plus one
- * collision launch over the nodes of all cloths near their meshes, replayed
- * from a CUDA graph holding one step.  Each cloth gets exactly the arithmetic
+ * collision launch over the nodes of all cloths near their meshes (for small
+ * cloths, one launch in all), replayed from a CUDA graph holding one step.  Each cloth gets exactly the arithmetic
  * it gets from cloth_step (bitwise the same results).  Not in the paper. */
 typedef struct ClothBatch ClothBatch;
 
