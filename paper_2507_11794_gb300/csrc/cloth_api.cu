@@ -521,9 +521,6 @@ int cloth_set_mesh(ClothHandle *h, const float *verts, int32_t nverts, const int
         }
         if (e != cudaSuccess) return cuda_fail(h, e, "grid build");
     }
-    // substeps without a mesh advance k and leave the listing counts: both start
-    // again at zero
-    CTRY(h, cudaMemsetAsync(h->ctrl->coll_count, 0, sizeof(h->ctrl->coll_count) + sizeof(h->ctrl->edge_next), h->stream), "clear listing counts");
     grid_free(&h->grid);
     h->grid = g;
     h->has_mesh = ntris > 0;

@@ -151,8 +151,6 @@ cudaError_t rebuild(ClothBatch *b)
             e = cudaMemcpyAsync(b->d_groups, groups.data(), sizeof(int2) * groups.size(), cudaMemcpyHostToDevice,
                                 b->stream);
     }
-    // the other form of the substep leaves the listing counts as they were
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->ctrl->coll_count, 0, sizeof(b->ctrl->coll_count), b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     b->args.groups = b->d_groups;
     b->args.n_groups = (int)groups.size();

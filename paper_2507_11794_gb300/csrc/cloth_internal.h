@@ -16,8 +16,9 @@ struct DevCtrl {
     // count of finished CTAs is needed to know when everybody has read k.
     unsigned long long kk[2];
     // The walk of a substep with collision kernels copies k to kc, which those
-    // read; they list into coll_count[k & 1] and zero the other one, which the
-    // next substep uses.  Whoever sets k from outside zeroes both (ctrl_set_k).
+    // read; they list into coll_count[k & 1].  Every substep, listing or not,
+    // zeroes the other one, which the next substep uses (ctrl_end_k); whoever
+    // sets k from outside zeroes both (ctrl_set_k).
     unsigned long long kc;
     unsigned int coll_count[2];
     unsigned int edge_next[2]; // next chunk of the edge pass, by substep parity as coll_count
@@ -241,8 +242,18 @@ __device__ __forceinline__ unsigned long long ctrl_k(const DevCtrl *ctrl)
     const unsigned long long a = c->kk[0], b = c->kk[1];
     return a > b ? a : b;
 }
-// End of substep k, by one thread.
-__device__ __forceinline__ void ctrl_end_k(DevCtrl *ctrl, unsigned long long k) { ctrl->kk[(k + 1ull) & 1ull] = k + 1ull; }
+// End of substep k, by one thread of its last kernel, at any point after that
+// kernel's wait: nothing reads k + 1 or the other listing counts before the next
+// substep, which starts after this kernel has completed.  Every form of the
+// substep ends here, also those that list nothing: the counts that substep k + 1
+// lists into are zero however substep k - 1 left them.
+__device__ __forceinline__ void ctrl_end_k(DevCtrl *ctrl, unsigned long long k)
+{
+    const unsigned next = (unsigned)(k + 1ull) & 1u;
+    ctrl->coll_count[next] = 0u;
+    ctrl->edge_next[next] = 0u;
+    ctrl->kk[next] = k + 1ull;
+}
 // Sets the substep counter from outside a substep (one thread).
 __device__ __forceinline__ void ctrl_set_k(DevCtrl *ctrl, unsigned long long k)
 {

@@ -566,15 +566,6 @@ __device__ __forceinline__ void coll_begin(DevCtrl *ctrl, unsigned long long &k,
     k = kc;
     n = (kc & 1ull) ? n1 : n0;
 }
-// End of a substep with a surface model (one thread of its last kernel, at
-// any point after that kernel's wait): nothing else reads k or the other count
-// before the next substep, which starts after this kernel has completed.
-__device__ __forceinline__ void coll_end(DevCtrl *ctrl, unsigned long long k)
-{
-    ctrl->coll_count[(k + 1ull) & 1ull] = 0u;
-    ctrl->edge_next[(k + 1ull) & 1ull] = 0u;
-    ctrl_end_k(ctrl, k);
-}
 
 // List entries of one cloth.
 struct OneClothList {
@@ -618,7 +609,7 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, SHORT ? CLOTH_COLL_SHORT_CTAS
     }
     __syncthreads();
     const unsigned long long k = s_k;
-    if (blockIdx.x == 0 && threadIdx.x == 0) coll_end(p.ctrl, k);
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl_end_k(p.ctrl, k);
     if (s_n == 0u) return;
     float fsum = 0.0f;
     unsigned ntest = 0u, nhit = 0u;
@@ -748,7 +739,7 @@ __global__ void __launch_bounds__(256) edge_apply_kernel(const __grid_constant__
     }
     if (__any_sync(FULL, !isfinite(fsum)) && (threadIdx.x & 31) == 0)
         atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
-    if (blockIdx.x == 0 && threadIdx.x == 0) coll_end(p.ctrl, k);
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl_end_k(p.ctrl, k);
 }
 
 // ---------------------------------------------------------------- batches
@@ -831,7 +822,7 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) batch_collid
     const unsigned long long k = s_k;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *b.work = 0u;
-        coll_end(b.ctrl, k);
+        ctrl_end_k(b.ctrl, k);
     }
     if (s_n == 0u) return;
     float fsum = 0.0f;
