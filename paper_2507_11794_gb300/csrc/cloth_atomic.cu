@@ -139,7 +139,8 @@ __global__ void __launch_bounds__(NODE_THREADS) node_integrate_kernel(const __gr
                 xx = fmaf(p.dt, p.pin_vel[0], px); xy = fmaf(p.dt, p.pin_vel[1], py); xz = fmaf(p.dt, p.pin_vel[2], pz);
                 wx = p.pin_vel[0]; wy = p.pin_vel[1]; wz = p.pin_vel[2];
             }
-            if (MESH)
+            // the edge narrow phase lists its nodes itself (edge_list_kernel), into the same list
+            if (MESH && !p.edge_resp)
                 need = !pinned && fmaxf(px, xx) >= p.mlo[0] && fminf(px, xx) <= p.mhi[0] &&
                        fmaxf(py, xy) >= p.mlo[1] && fminf(py, xy) <= p.mhi[1] && fmaxf(pz, xz) >= p.mlo[2] &&
                        fminf(pz, xz) <= p.mhi[2];

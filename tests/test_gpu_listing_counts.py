@@ -52,7 +52,7 @@ def test_profile_and_step_in_turn(cloth_lib, nx, ny, graph):
     np.testing.assert_array_equal(va, vb)
 
 
-@pytest.mark.parametrize("edges,atomic", [(False, False), (True, False), (False, True)])
+@pytest.mark.parametrize("edges,atomic", [(False, False), (True, False), (False, True), (True, True)])
 @pytest.mark.parametrize("free", [1, 2])
 def test_model_taken_away_and_set_again(cloth_lib, edges, atomic, free):
     """Listing substeps, `free` substeps without a model, listing substeps: as
@@ -77,3 +77,21 @@ def test_model_taken_away_and_set_again(cloth_lib, edges, atomic, free):
         assert tuple(x - y for x, y in zip(sa, before)) == sb
         np.testing.assert_array_equal(pa, pb)
         np.testing.assert_array_equal(va, vb)
+
+
+@pytest.mark.parametrize("nx,ny", [(31, 23), (150, 131)])
+def test_atomic_forces_with_edges(cloth_lib, nx, ny):
+    """Both flags together: the edge narrow phase alone fills the list.  Without
+    spring forces the two force paths round alike, so the results are those of
+    the edge flag alone, bit for bit."""
+    P, sc = cloth_lib, scene(nx, ny)
+    sc.ks = sc.kd = (0.0, 0.0, 0.0)
+    got = []
+    for flags in (P.capi.CLOTH_FLAG_EDGE_COLLISION, P.capi.CLOTH_FLAG_EDGE_COLLISION | P.capi.CLOTH_FLAG_ATOMIC_SPRINGS):
+        with P.Cloth(sc, flags=flags) as cl:
+            cl.step(3)
+            got.append((*cl.read(), cl.collision_stats()))
+    (pa, va, sa), (pb, vb, sb) = got
+    assert sa == sb and sa[0] == 3 * sc.n and sa[2] > 0
+    np.testing.assert_array_equal(pa, pb)
+    np.testing.assert_array_equal(va, vb)
