@@ -105,14 +105,19 @@ struct OneCloth {  // coll_cells' source of parameters for one cloth
     __device__ const StepParams &params(int) const { return p; }
 };
 
-// Candidate filter: every grid entry carries its triangle's box in 16-bit
-// units of 1 / grid_filter_sub of a cell (grown by p.qpad units), laid out so
+// Candidate filter: every grid entry carries its triangle's box in units of
+// 1 / 64 of a cell (coarser on long grids, see grid_filter_scale; grown by one
+// unit and the rounding of the mesh's coordinates), laid out so
 // that three subtractions compare it with a path's box on all six sides: word
 // lanes of 15 bits under a guard bit, T = (hx, hy) (hz, M - lx) (M - ly,
 // M - lz) for the triangle and N = (lo x, lo y) (lo z, M - hi x) (...) for the
 // path, M = 32767; the boxes overlap iff every lane of T is >= that of N, i.e.
 // iff no guard bit is borrowed from.  A path can only hit a triangle whose
-// box it overlaps, so the test below it runs on the entries that pass.
+// box it overlaps, so the test below it runs on the entries that pass.  The
+// float32 test by itself can also accept a triangle far outside whose box the
+// path lies, in the triangle's own plane: its errors in u, v and t grow as 1 / a,
+// and a path along a large tilted triangle has a far below the triangle's size.
+// The filter turns those away; whatever looks at hits has to look through it.
 // The fourth word has bit a (0, 1, 2) where the entry's cell is the first of
 // the triangle's box along axis a: a triangle listed in several cells of a
 // path's box is tested only in the first cell the two boxes share, which is
@@ -732,8 +737,9 @@ __device__ __forceinline__ void edge_acc_add(EdgeAcc &a, float delta, float sx, 
 }
 
 // An edge with more hits than pass A stored: walks its candidates again, in
-// order, and adds every hit after the first (already added).  Out of line:
-// rare, and it keeps the gather's unrolled loop small.
+// order and behind the same filter (the hits must be pass A's, also where
+// rounding alone decides), and adds every hit after the first (already added).
+// Out of line: rare, and it keeps the gather's unrolled loop small.
 static __device__ __noinline__ EdgeAcc edge_rewalk(const StepParams &p, const float *xs, long long oa, long long ob,
                                                    float sx, float sy, float sz, EdgeAcc a)
 {
@@ -743,15 +749,18 @@ static __device__ __noinline__ EdgeAcc edge_rewalk(const StepParams &p, const fl
     CollPath path;
     if (!coll_path(p, x0, y0, z0, x1, y1, z1, path)) return a;
     const CollBox bx = coll_box(p, x0, y0, z0, x1, y1, z1);
+    const CollWords w = coll_words(p, x0, y0, z0, x1, y1, z1, path);
     bool first = true;
     for (int cz = bx.loz; cz <= bx.hiz; cz++)
         for (int cy = bx.loy; cy <= bx.hiy; cy++)
             for (int cx = bx.lox; cx <= bx.hix; cx++) {
                 const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
                 const int e0 = __ldg(p.cell_start + cell), e1 = __ldg(p.cell_start + cell + 1);
+                const unsigned need = coll_need(bx, cx, cy, cz);
                 for (int ee = e0; ee < e1; ee++) {
                     float th, over, f;
                     float4 A, B, C;
+                    if (!coll_overlap(__ldg(p.efil + ee), w, need)) continue;
                     if (!coll_candidate(p, path, ee, cx, cy, cz, bx.lox, bx.loy, bx.loz, th, over, f, A, B, C)) continue;
                     if (first) {
                         first = false;

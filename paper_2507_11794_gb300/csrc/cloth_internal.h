@@ -221,9 +221,9 @@ cudaError_t launch_soa_to_aos(const float *state0, const float *state1, long lon
 // Narrow-phase filter (see cloth_collide.cuh): boxes in units of 1 / sub of a
 // cell, 15 bits a side; sub is 64 where the grid's longest side leaves room for
 // it.  The scale is 0 where it does not fit at all (then every box is the
-// same and passes).  The triangles' boxes grow by grid_filter_pad units: one
-// for the narrow phase's own rounding, far below 1 / 64 of a cell, and what
-// float32 coordinates of the mesh's magnitude can be off.
+// same and passes).  The triangles' boxes grow by one unit and what float32
+// coordinates of the mesh's magnitude can be off (grid_build), so that a path
+// that crosses a triangle passes.
 #define GRID_FILTER_MAX 32767u
 #define GRID_FILTER_GUARD 0x80008000u
 inline float grid_filter_scale(const int dims[3], float inv)
