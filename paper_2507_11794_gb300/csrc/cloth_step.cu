@@ -21,6 +21,7 @@
 // every spring is evaluated once, with no atomics and a fixed summation order:
 // results are bitwise reproducible.  The first two rows of each walk only
 // produce the springs that reach into the strip.
+#include <cuda.h>
 #include <string.h>
 
 #include <mutex>
@@ -1008,18 +1009,43 @@ cudaError_t launch_soa_to_aos(const float *state0, const float *state1, long lon
 }
 
 namespace {
-// The device's address of a host array of n floats the GPU can reach
-// (page-locked from end to end), else null.
+// The driver's cuPointerGetAttributes, which knows the extent of a page-locked
+// range (the library does not link the driver); null if there is none.
+decltype(&cuPointerGetAttributes) pointer_attributes()
+{
+    static const decltype(&cuPointerGetAttributes) f = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &p, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return (decltype(&cuPointerGetAttributes))p;
+    }();
+    return f;
+}
+
+// The device's address of a host array of n floats the GPU can reach, which
+// takes one page-locked range around all of it (its ends can lie in two with
+// pageable memory in between), else null.
 float *mapped(const float *host, long long n)
 {
-    cudaPointerAttributes a, z;
+    cudaPointerAttributes a;
     if (!host || n < 1) return nullptr;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&z, host + n - 1) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    const bool ok = a.type == cudaMemoryTypeHost && z.type == cudaMemoryTypeHost && a.devicePointer &&
-                    (float *)z.devicePointer == (float *)a.devicePointer + (n - 1);
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer || !pointer_attributes()) return nullptr;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&start, &size};
+    const CUdeviceptr first = (CUdeviceptr)a.devicePointer;
+    // with another address on the device than on the host the range could be in either's terms: not taken
+    if (a.devicePointer != host || pointer_attributes()(2, what, to, first) != CUDA_SUCCESS) return nullptr;
+    const bool ok = start && start <= first && first + sizeof(float) * (size_t)n <= start + size;
     return ok ? (float *)a.devicePointer : nullptr;
 }
 

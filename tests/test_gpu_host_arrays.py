@@ -1,0 +1,43 @@
+"""State read into and set from arrays of unusual memory: what the kernels may
+not reach goes through buffers and the driver's copies."""
+import mmap
+
+import numpy as np
+import pytest
+
+from helpers import make_scene
+
+pytestmark = pytest.mark.gpu
+
+
+def scene(nx, ny, seed=1):
+    rng = np.random.default_rng(seed)
+    sc = make_scene(nx, ny, dt=1e-3)
+    sc.init_pos[:] = rng.normal(size=sc.init_pos.shape)
+    sc.init_vel[:] = rng.normal(size=sc.init_vel.shape)
+    return sc
+
+
+@pytest.fixture
+def two_ranges():
+    """An array of 6,400 nodes whose ends lie in two page-locked ranges, with pageable memory in between."""
+    import torch
+    n, page = 6400, max(mmap.PAGESIZE, 65536)
+    raw = np.frombuffer(mmap.mmap(-1, 4 * page), np.uint8)
+    at = -raw.ctypes.data % page
+    rt = torch.cuda.cudart()
+    ends = [raw.ctypes.data + at, raw.ctypes.data + at + 2 * page]
+    for p in ends:
+        assert int(rt.cudaHostRegister(p, page, 0)) == 0
+    yield raw[at + page - 4096:][:12 * n].view(np.float32).reshape(n, 3)
+    for p in ends:
+        assert int(rt.cudaHostUnregister(p)) == 0
+
+
+def test_array_over_two_page_locked_ranges(cloth_lib, two_ranges):
+    sc = scene(80, 80)
+    with cloth_lib.Cloth(sc) as cl:
+        for k in range(2):
+            two_ranges[:] = 0.0
+            p, _ = cl.read(vel=False, out_pos=two_ranges)
+            assert p is two_ranges and np.array_equal(p, sc.init_pos)
