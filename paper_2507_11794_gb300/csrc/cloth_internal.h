@@ -8,7 +8,7 @@
 
 #define CLOTH_STAT_SLOTS 16
 // Device-side control block of one cloth (one per handle, in device memory).
-struct DevCtrl {
+struct alignas(16) DevCtrl {
     // The substep counter k (selects time and ping-pong buffer), as two words:
     // kk[k & 1] = k and the other one lower, so k is the larger (ctrl_k).  A
     // launch that knows its parity reads kk[parity], which nothing writes while
@@ -211,11 +211,13 @@ void grid_free(DevGrid *g);
 cudaError_t grid_query(const DevGrid &g, const float *dS, const float *dE, int nseg, int *counts, int *ids, int cap,
                        cudaStream_t s);
 
-// AoS <-> SoA state transfer through the ping-pong buffer selected by ctrl->k.
+// AoS <-> SoA state transfer through the ping-pong buffer selected by ctrl->k;
+// host: an array is page-locked host memory.
 cudaError_t launch_aos_to_soa(const float *aos_pos, const float *aos_vel, float *state0, float *state1,
-                              long long stride, int n, int nx, int pitch, DevCtrl *ctrl, cudaStream_t s);
+                              long long stride, int n, int nx, int pitch, DevCtrl *ctrl, cudaStream_t s,
+                              bool host = false);
 cudaError_t launch_soa_to_aos(const float *state0, const float *state1, long long stride, int n, int nx, int pitch,
-                              const DevCtrl *ctrl, float *aos_pos, float *aos_vel, cudaStream_t s,
+                              const DevCtrl *ctrl, float *aos_pos, float *aos_vel, cudaStream_t s, bool host = false,
                               unsigned *flags = nullptr);
 
 // Narrow-phase filter (see cloth_collide.cuh): boxes in units of 1 / sub of a
@@ -241,6 +243,14 @@ __device__ __forceinline__ unsigned long long ctrl_k(const DevCtrl *ctrl)
     const volatile DevCtrl *c = ctrl;
     const unsigned long long a = c->kk[0], b = c->kk[1];
     return a > b ? a : b;
+}
+// The same in a kernel whose launch waits for every substep before it: each warp
+// may read it, through the L1.  (As ctrl_k's two loads per warp, all to one line of
+// L2, it was most of a state transfer's time: see aos_to_soa_kernel.)
+__device__ __forceinline__ unsigned long long ctrl_k_settled(const DevCtrl *ctrl)
+{
+    const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(ctrl->kk);
+    return w.x > w.y ? w.x : w.y;
 }
 // End of substep k, by one thread of its last kernel, at any point after that
 // kernel's wait: nothing reads k + 1 or the other listing counts before the next

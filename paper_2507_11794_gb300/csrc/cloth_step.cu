@@ -834,43 +834,81 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) batch_collid
     coll_stats_add(b.ctrl, s_stat, s_n, ntest, nhit);
 }
 
-// State transfer, one thread per float of the [n][3] arrays, so that their side
-// is read or written in whole lines (it can be host memory, over the link).
+// State transfer between the planes and [n][3] arrays.  HOST: an array is host
+// memory, over the link: one thread per float, so that its side is read or
+// written in whole lines.  On the device a thread takes a node: a third of the
+// warps and of the index arithmetic (640,000 nodes, ncu: into the planes 12.4 us
+// with a thread per float, 6.4 with one per node; every warp reading the
+// substep counter past the L1 made the two 15.2 and 15.1).
+template <bool HOST>
 __global__ void aos_to_soa_kernel(const float *__restrict__ pos, const float *__restrict__ vel, float *state0,
                                   float *state1, long long st, int n, int nx, int pitch, DevCtrl *ctrl)
 {
-    const unsigned long long k = ctrl_k(ctrl);
+    const unsigned long long k = ctrl_k_settled(ctrl);
     float *dst = (k & 1ull) ? state1 : state0;
-    const long long total = 3ll * n;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const unsigned node = (unsigned)(i / 3), a = (unsigned)(i - 3ll * node), r = node / (unsigned)nx;
-        const long long o = a * st + (long long)r * pitch + (node - r * (unsigned)nx);
-        if (pos) dst[o] = pos[i];
-        if (vel) dst[3 * st + o] = vel[i];
+    if (HOST) {
+        const long long total = 3ll * n;
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+            const unsigned node = (unsigned)(i / 3), a = (unsigned)(i - 3ll * node), r = node / (unsigned)nx;
+            const long long o = a * st + (long long)r * pitch + (node - r * (unsigned)nx);
+            if (pos) dst[o] = pos[i];
+            if (vel) dst[3 * st + o] = vel[i];
+        }
+    } else {
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+            const long long o = (long long)(i / nx) * pitch + (i % nx);
+            if (pos) {
+                dst[0 * st + o] = pos[3 * (long long)i];
+                dst[1 * st + o] = pos[3 * (long long)i + 1];
+                dst[2 * st + o] = pos[3 * (long long)i + 2];
+            }
+            if (vel) {
+                dst[3 * st + o] = vel[3 * (long long)i];
+                dst[4 * st + o] = vel[3 * (long long)i + 1];
+                dst[5 * st + o] = vel[3 * (long long)i + 2];
+            }
+        }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->flags = 0u;
 }
 
+template <bool HOST>
 __global__ void soa_to_aos_kernel(const float *state0, const float *state1, long long st, int n, int nx, int pitch,
                                   const DevCtrl *ctrl, float *__restrict__ pos, float *__restrict__ vel,
                                   unsigned *flags)
 {
-    const unsigned long long k = ctrl_k(ctrl);
-    const float *src = (k & 1ull) ? state1 : state0;
-    const long long total = 3ll * n;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const unsigned node = (unsigned)(i / 3), a = (unsigned)(i - 3ll * node), r = node / (unsigned)nx;
-        const long long o = a * st + (long long)r * pitch + (node - r * (unsigned)nx);
-        if (pos) pos[i] = src[o];
-        if (vel) vel[i] = src[3 * st + o];
-    }
     if (flags && blockIdx.x == 0 && threadIdx.x == 0) *flags = ctrl->flags;
+    const unsigned long long k = ctrl_k_settled(ctrl);
+    const float *src = (k & 1ull) ? state1 : state0;
+    if (HOST) {
+        const long long total = 3ll * n;
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+            const unsigned node = (unsigned)(i / 3), a = (unsigned)(i - 3ll * node), r = node / (unsigned)nx;
+            const long long o = a * st + (long long)r * pitch + (node - r * (unsigned)nx);
+            if (pos) pos[i] = src[o];
+            if (vel) vel[i] = src[3 * st + o];
+        }
+    } else {
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+            const long long o = (long long)(i / nx) * pitch + (i % nx);
+            if (pos) {
+                pos[3 * (long long)i] = src[0 * st + o];
+                pos[3 * (long long)i + 1] = src[1 * st + o];
+                pos[3 * (long long)i + 2] = src[2 * st + o];
+            }
+            if (vel) {
+                vel[3 * (long long)i] = src[3 * st + o];
+                vel[3 * (long long)i + 1] = src[4 * st + o];
+                vel[3 * (long long)i + 2] = src[5 * st + o];
+            }
+        }
+    }
 }
 
-int transfer_blocks(int n)
+int transfer_blocks(int n, bool host)
 {
-    const long long b = (3ll * n + 255) / 256;
-    return (int)(b < 1 ? 1 : (b > 152 * 8 ? 152 * 8 : b));
+    const long long b = ((host ? 3ll : 1ll) * n + 255) / 256, most = 152 * (host ? 8 : 16);
+    return (int)(b < 1 ? 1 : (b > most ? most : b));
 }
 
 }  // namespace
@@ -993,18 +1031,20 @@ int batch_min_ctas()
 }
 
 cudaError_t launch_aos_to_soa(const float *aos_pos, const float *aos_vel, float *state0, float *state1,
-                              long long stride, int n, int nx, int pitch, DevCtrl *ctrl, cudaStream_t s)
+                              long long stride, int n, int nx, int pitch, DevCtrl *ctrl, cudaStream_t s, bool host)
 {
-    aos_to_soa_kernel<<<transfer_blocks(n), 256, 0, s>>>(aos_pos, aos_vel, state0, state1, stride, n, nx, pitch,
-                                                         ctrl);
+    auto *kernel = host ? aos_to_soa_kernel<true> : aos_to_soa_kernel<false>;
+    kernel<<<transfer_blocks(n, host), 256, 0, s>>>(aos_pos, aos_vel, state0, state1, stride, n, nx, pitch, ctrl);
     return cudaGetLastError();
 }
 
 cudaError_t launch_soa_to_aos(const float *state0, const float *state1, long long stride, int n, int nx, int pitch,
-                              const DevCtrl *ctrl, float *aos_pos, float *aos_vel, cudaStream_t s, unsigned *flags)
+                              const DevCtrl *ctrl, float *aos_pos, float *aos_vel, cudaStream_t s, bool host,
+                              unsigned *flags)
 {
-    soa_to_aos_kernel<<<transfer_blocks(n), 256, 0, s>>>(state0, state1, stride, n, nx, pitch, ctrl, aos_pos,
-                                                         aos_vel, flags);
+    auto *kernel = host ? soa_to_aos_kernel<true> : soa_to_aos_kernel<false>;
+    kernel<<<transfer_blocks(n, host), 256, 0, s>>>(state0, state1, stride, n, nx, pitch, ctrl, aos_pos, aos_vel,
+                                                    flags);
     return cudaGetLastError();
 }
 
@@ -1100,8 +1140,9 @@ cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, HostBounce *b, fl
     const bool small = db && 6 * N <= HOST_BOUNCE_FLOATS;
     float *dp = mp ? mp : small ? db : h->staging;
     float *dv = mv ? mv : small ? db + 3 * N : h->staging + 3 * N;
+    const bool host = (pos && dp != h->staging) || (vel && dv != h->staging + 3 * N);
     cudaError_t e = launch_soa_to_aos(h->state, h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, ctrl,
-                                      pos ? dp : nullptr, vel ? dv : nullptr, s,
+                                      pos ? dp : nullptr, vel ? dv : nullptr, s, host,
                                       db ? (unsigned *)(db + HOST_BOUNCE_FLOATS) : nullptr);
     if (e == cudaSuccess && pos && dp == h->staging)
         e = cudaMemcpyAsync(pos, dp, sizeof(float) * 3 * N, cudaMemcpyDeviceToHost, s);
@@ -1126,5 +1167,6 @@ cudaError_t state_from_host(ClothHandle *h, DevCtrl *ctrl, const float *pos, con
         e = cudaMemcpyAsync(h->staging + 3 * N, vel, sizeof(float) * 3 * N, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     return launch_aos_to_soa(mp ? mp : pos ? h->staging : nullptr, mv ? mv : vel ? h->staging + 3 * N : nullptr,
-                             h->state, h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, ctrl, s);
+                             h->state, h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, ctrl, s,
+                             mp || mv);
 }
