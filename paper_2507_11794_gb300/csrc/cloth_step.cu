@@ -1072,7 +1072,7 @@ decltype(&cuPointerGetAttributes) pointer_attributes()
 float *mapped(const float *host, long long n)
 {
     cudaPointerAttributes a;
-    if (!host || n < 1) return nullptr;
+    if (!host || n < 1 || (uintptr_t)host % sizeof(float)) return nullptr;  // a copy takes any alignment, a kernel not
     if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;

@@ -41,3 +41,25 @@ def test_array_over_two_page_locked_ranges(cloth_lib, two_ranges):
             two_ranges[:] = 0.0
             p, _ = cl.read(vel=False, out_pos=two_ranges)
             assert p is two_ranges and np.array_equal(p, sc.init_pos)
+
+
+@pytest.mark.parametrize("nx,ny", [(7, 5), (127, 87)])
+@pytest.mark.parametrize("page_locked", [True, False])
+def test_arrays_off_the_float_boundary(cloth_lib, nx, ny, page_locked):
+    import torch
+    n = nx * ny
+
+    def array():
+        raw = torch.empty(12 * n + 4, dtype=torch.uint8)
+        raw = (raw.pin_memory() if page_locked else raw).numpy()
+        a = raw[1:1 + 12 * n].view(np.float32).reshape(n, 3)
+        assert a.ctypes.data % 4 == 1
+        return a
+
+    sc, p, v = scene(nx, ny), array(), array()
+    with cloth_lib.Cloth(sc) as cl:
+        cl.read(out_pos=p, out_vel=v)
+        assert np.array_equal(p, sc.init_pos) and np.array_equal(v, sc.init_vel)
+        cl.set_state(v, p)
+        got = cl.read()
+    assert np.array_equal(got[0], sc.init_vel) and np.array_equal(got[1], sc.init_pos)
