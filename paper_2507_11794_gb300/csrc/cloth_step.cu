@@ -1066,27 +1066,36 @@ decltype(&cuPointerGetAttributes) pointer_attributes()
     return f;
 }
 
-// The device's address of a host array of n floats the GPU can reach, which
-// takes one page-locked range around all of it (its ends can lie in two with
-// pageable memory in between), else null.
-float *mapped(const float *host, long long n)
+// What a caller's array of n floats is: gpu, the device's address if the GPU
+// can reach it, which takes one page-locked range around all of it (its ends can
+// lie in two with pageable memory in between), else null; cpu: it is host memory
+// (device and managed memory is left to the driver's copies, which take it or
+// refuse it).
+struct HostArray {
+    float *gpu;
+    bool cpu;
+};
+HostArray host_array(const float *host, long long n)
 {
     cudaPointerAttributes a;
-    if (!host || n < 1 || (uintptr_t)host % sizeof(float)) return nullptr;  // a copy takes any alignment, a kernel not
+    if (!host || n < 1) return {nullptr, false};
     if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        return {nullptr, false};
     }
-    if (a.type != cudaMemoryTypeHost || !a.devicePointer || !pointer_attributes()) return nullptr;
+    const bool cpu = a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeUnregistered;
+    const HostArray copied = {nullptr, cpu};
+    if ((uintptr_t)host % sizeof(float)) return copied;  // a copy takes any alignment, a kernel not
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer || !pointer_attributes()) return copied;
     CUdeviceptr start = 0;
     size_t size = 0;
     CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
     void *to[] = {&start, &size};
     const CUdeviceptr first = (CUdeviceptr)a.devicePointer;
     // with another address on the device than on the host the range could be in either's terms: not taken
-    if (a.devicePointer != host || pointer_attributes()(2, what, to, first) != CUDA_SUCCESS) return nullptr;
+    if (a.devicePointer != host || pointer_attributes()(2, what, to, first) != CUDA_SUCCESS) return copied;
     const bool ok = start && start <= first && first + sizeof(float) * (size_t)n <= start + size;
-    return ok ? (float *)a.devicePointer : nullptr;
+    return {ok ? (float *)a.devicePointer : nullptr, cpu};
 }
 
 // Page-locked buffers returned by destroyed handles, kept for the next ones
@@ -1135,11 +1144,11 @@ cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, HostBounce *b, fl
                           cudaStream_t s)
 {
     const long long N = h->n;
-    float *bp = bounce_get(b), *db = mapped(bp, HOST_BOUNCE_FLOATS + 1);
-    float *mp = mapped(pos, 3 * N), *mv = mapped(vel, 3 * N);
+    float *bp = bounce_get(b), *db = host_array(bp, HOST_BOUNCE_FLOATS + 1).gpu;
+    const HostArray ap = host_array(pos, 3 * N), av = host_array(vel, 3 * N);
     const bool small = db && 6 * N <= HOST_BOUNCE_FLOATS;
-    float *dp = mp ? mp : small ? db : h->staging;
-    float *dv = mv ? mv : small ? db + 3 * N : h->staging + 3 * N;
+    float *dp = ap.gpu ? ap.gpu : small && ap.cpu ? db : h->staging;
+    float *dv = av.gpu ? av.gpu : small && av.cpu ? db + 3 * N : h->staging + 3 * N;
     const bool host = (pos && dp != h->staging) || (vel && dv != h->staging + 3 * N);
     cudaError_t e = launch_soa_to_aos(h->state, h->state + 6 * h->stride, h->stride, h->n, h->desc.nx, h->pitch, ctrl,
                                       pos ? dp : nullptr, vel ? dv : nullptr, s, host,
@@ -1151,8 +1160,8 @@ cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, HostBounce *b, fl
     if (e == cudaSuccess && !db) e = cudaMemcpyAsync(flags, &ctrl->flags, sizeof(*flags), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    if (pos && !mp && small) memcpy(pos, bp, sizeof(float) * 3 * N);
-    if (vel && !mv && small) memcpy(vel, bp + 3 * N, sizeof(float) * 3 * N);
+    if (pos && dp == db) memcpy(pos, bp, sizeof(float) * 3 * N);
+    if (vel && dv == db + 3 * N) memcpy(vel, bp + 3 * N, sizeof(float) * 3 * N);
     if (db) *flags = *(const volatile unsigned *)(bp + HOST_BOUNCE_FLOATS);
     return cudaSuccess;
 }
@@ -1160,7 +1169,7 @@ cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, HostBounce *b, fl
 cudaError_t state_from_host(ClothHandle *h, DevCtrl *ctrl, const float *pos, const float *vel, cudaStream_t s)
 {
     const long long N = h->n;
-    const float *mp = mapped(pos, 3 * N), *mv = mapped(vel, 3 * N);
+    const float *mp = host_array(pos, 3 * N).gpu, *mv = host_array(vel, 3 * N).gpu;
     cudaError_t e = cudaSuccess;
     if (pos && !mp) e = cudaMemcpyAsync(h->staging, pos, sizeof(float) * 3 * N, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && vel && !mv)

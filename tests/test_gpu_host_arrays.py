@@ -1,5 +1,6 @@
 """State read into and set from arrays of unusual memory: what the kernels may
 not reach goes through buffers and the driver's copies."""
+import ctypes as C
 import mmap
 
 import numpy as np
@@ -63,3 +64,18 @@ def test_arrays_off_the_float_boundary(cloth_lib, nx, ny, page_locked):
         cl.set_state(v, p)
         got = cl.read()
     assert np.array_equal(got[0], sc.init_vel) and np.array_equal(got[1], sc.init_pos)
+
+
+@pytest.mark.parametrize("nx,ny", [(7, 5), (127, 87)])
+def test_device_array_is_left_to_the_driver(cloth_lib, nx, ny):
+    """cloth_read into device memory: an error code or the driver's copy, not a store by the host."""
+    import torch
+    sc, lib = scene(nx, ny), cloth_lib.capi.lib()
+    out = torch.zeros((nx * ny, 3), device="cuda")
+    torch.cuda.synchronize()
+    with cloth_lib.Cloth(sc) as cl:
+        rc = lib.cloth_read(cl.h, C.cast(out.data_ptr(), C.POINTER(C.c_float)), None)
+        if rc == 0:
+            assert np.array_equal(out.cpu().numpy(), sc.init_pos)
+        else:
+            assert rc == -3 and not out.any()  # CLOTH_ERR_CUDA
