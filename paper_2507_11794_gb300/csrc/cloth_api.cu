@@ -78,7 +78,6 @@ void free_all(ClothHandle *h)
     cudaFree(h->kd_slot);
     cudaFree(h->ctrl);
     cudaFree(h->staging);
-    bounce_release(&h->bounce);
     cudaFree(h->coll_list);
     h->coll_list = nullptr;
     cudaFree(h->wind_tab);
@@ -561,7 +560,7 @@ int cloth_read(ClothHandle *h, float *pos_out, float *vel_out)
     DeviceScope ds(h->device);
     unsigned flags = 0;
     if (pos_out || vel_out) {
-        CTRY(h, state_to_host(h, h->ctrl, &h->bounce, pos_out, vel_out, &flags, h->stream), "read state");
+        CTRY(h, state_to_host(h, h->ctrl, pos_out, vel_out, &flags, h->stream), "read state");
     } else {
         rc = read_flags(h, &flags);
         if (rc) return rc;

@@ -21,7 +21,6 @@ struct ClothBatch {
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
     DevCtrl *ctrl = nullptr;
-    HostBounce bounce;
     unsigned *work = nullptr;
     int *coll_list = nullptr;
     int *coll_cloth = nullptr;
@@ -191,7 +190,6 @@ void free_batch(ClothBatch *b)
     for (ClothHandle *h : b->cl) cloth_destroy(h);
     b->cl.clear();
     cudaFree(b->ctrl);
-    bounce_release(&b->bounce);
     cudaFree(b->work);
     cudaFree(b->coll_list);
     cudaFree(b->coll_cloth);
@@ -334,7 +332,7 @@ int cloth_batch_read(ClothBatch *b, int32_t index, float *pos_out, float *vel_ou
     if (index < 0 || index >= (int)b->cl.size()) return bfail(CLOTH_ERR_INVALID_ARG, "cloth index %d", index);
     unsigned flags = 0;
     if (!pos_out && !vel_out) return read_batch_flags(b);
-    BTRY(b, state_to_host(b->cl[index], b->ctrl, &b->bounce, pos_out, vel_out, &flags, b->stream), "read state");
+    BTRY(b, state_to_host(b->cl[index], b->ctrl, pos_out, vel_out, &flags, b->stream), "read state");
     return batch_flags_status(flags);
 }
 

@@ -314,13 +314,6 @@ cudaError_t grid_build_noalloc(const float *d_verts, const int *d_tris, int nt, 
 // Sets the calling thread's cloth_last_error() message.
 void cloth_set_error_message(const char *msg);
 
-// A handle's page-locked buffer for reads, taken by the first one: state
-// floats, then the flags.
-#define HOST_BOUNCE_FLOATS 65536
-struct HostBounce {
-    float *p = nullptr;
-};
-
 // One cloth (the opaque handle of the C ABI).
 struct ClothHandle {
     ClothDesc desc;  // array pointers cleared after the copy
@@ -336,7 +329,6 @@ struct ClothHandle {
     float *ks_slot = nullptr, *kd_slot = nullptr;
     DevCtrl *ctrl = nullptr;
     float *staging = nullptr;  // 6*n floats for AoS transfers
-    HostBounce bounce;
     int *coll_list = nullptr;  // n entries
     float2 *wind_tab = nullptr; // ny row entries then nx column entries
     float4 *force = nullptr;    // CLOTH_FLAG_ATOMIC_SPRINGS: pitch*ny force accumulators
@@ -354,10 +346,8 @@ struct ClothHandle {
 };
 
 void cloth_fill_params(ClothHandle *h);
-// The current state to host arrays (either may be null) with the flags, through
-// a handle's or a batch's bounce buffer; waits for s.  And the other way, as
-// cloth_set_state: a pageable array is copied before the return.
-cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, HostBounce *b, float *pos, float *vel, unsigned *flags,
-                          cudaStream_t s);
-void bounce_release(HostBounce *b);
+// The current state to host arrays (either may be null) with the flags; waits
+// for s.  And the other way, as cloth_set_state: a pageable array is copied before
+// the return.
+cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, float *pos, float *vel, unsigned *flags, cudaStream_t s);
 cudaError_t state_from_host(ClothHandle *h, DevCtrl *ctrl, const float *pos, const float *vel, cudaStream_t s);

@@ -1098,53 +1098,68 @@ HostArray host_array(const float *host, long long n)
     return {ok ? (float *)a.devicePointer : nullptr, cpu};
 }
 
-// Page-locked buffers returned by destroyed handles, kept for the next ones
-// (allocating one takes longer than a small read); at most HOST_BOUNCE_KEEP.
+// Page-locked buffers for reads (state floats, then the flags), each taken for
+// the time of one read, so there are as many as reads at the same time; at most
+// HOST_BOUNCE_KEEP stay for later ones (allocating one takes longer than a small
+// read).
+constexpr long long HOST_BOUNCE_FLOATS = 65536;
 constexpr int HOST_BOUNCE_KEEP = 8;
 std::mutex bounce_lock;
 float *bounce_free[HOST_BOUNCE_KEEP];
 int bounce_count = 0;
-}  // namespace
 
-// A handle's buffer, its own until bounce_release; null if there is no memory.
-static float *bounce_get(HostBounce *b)
-{
-    if (b->p) return b->p;
+struct Bounce {
+    float *cpu = nullptr, *gpu = nullptr;  // null if there is no memory
+
+    Bounce()
     {
-        std::lock_guard<std::mutex> g(bounce_lock);
-        if (bounce_count > 0) b->p = bounce_free[--bounce_count];
-    }
-    if (!b->p && cudaHostAlloc((void **)&b->p, sizeof(float) * HOST_BOUNCE_FLOATS + 64, cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        b->p = nullptr;
-    }
-    return b->p;
-}
-void bounce_release(HostBounce *b)
-{
-    if (!b->p) return;
-    {
-        std::lock_guard<std::mutex> g(bounce_lock);
-        if (bounce_count < HOST_BOUNCE_KEEP) {
-            bounce_free[bounce_count++] = b->p;
-            b->p = nullptr;
+        do {
+            {
+                std::lock_guard<std::mutex> g(bounce_lock);
+                cpu = bounce_count > 0 ? bounce_free[--bounce_count] : nullptr;
+            }
+            // one from before a reset of the device is gone
+            gpu = host_array(cpu, HOST_BOUNCE_FLOATS + 1).gpu;
+        } while (cpu && !gpu);
+        if (cpu) return;
+        if (cudaHostAlloc((void **)&cpu, sizeof(float) * HOST_BOUNCE_FLOATS + 64, cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            cpu = nullptr;
+        }
+        gpu = host_array(cpu, HOST_BOUNCE_FLOATS + 1).gpu;
+        if (cpu && !gpu) {
+            cudaFreeHost(cpu);
+            cpu = nullptr;
         }
     }
-    cudaFreeHost(b->p);
-    b->p = nullptr;
-}
+    ~Bounce()
+    {
+        if (!cpu) return;
+        {
+            std::lock_guard<std::mutex> g(bounce_lock);
+            if (bounce_count < HOST_BOUNCE_KEEP) {
+                bounce_free[bounce_count++] = cpu;
+                return;
+            }
+        }
+        cudaFreeHost(cpu);
+    }
+    Bounce(const Bounce &) = delete;
+    Bounce &operator=(const Bounce &) = delete;
+};
+}  // namespace
 
 // What a read costs beside the link is copies and the calls that queue them, so
 // it takes as few as it can: page-locked arrays are written by the gather
-// kernel itself, small pageable ones through one page-locked buffer of the
-// handle, together with the flags; only large pageable arrays go through the
-// device staging buffer and the driver's copies.  Reading a 16 x 16 to 64 x 64
-// cloth of a batch took 40 us with three copies.
-cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, HostBounce *b, float *pos, float *vel, unsigned *flags,
-                          cudaStream_t s)
+// kernel itself, small pageable ones through one page-locked buffer, together
+// with the flags; only large pageable arrays go through the device staging buffer
+// and the driver's copies.  Reading a 16 x 16 to 64 x 64 cloth of a batch took
+// 40 us with three copies.
+cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, float *pos, float *vel, unsigned *flags, cudaStream_t s)
 {
     const long long N = h->n;
-    float *bp = bounce_get(b), *db = host_array(bp, HOST_BOUNCE_FLOATS + 1).gpu;
+    Bounce bounce;
+    float *bp = bounce.cpu, *db = bounce.gpu;
     const HostArray ap = host_array(pos, 3 * N), av = host_array(vel, 3 * N);
     const bool small = db && 6 * N <= HOST_BOUNCE_FLOATS;
     float *dp = ap.gpu ? ap.gpu : small && ap.cpu ? db : h->staging;
@@ -1158,7 +1173,9 @@ cudaError_t state_to_host(ClothHandle *h, const DevCtrl *ctrl, HostBounce *b, fl
     if (e == cudaSuccess && vel && dv == h->staging + 3 * N)
         e = cudaMemcpyAsync(vel, dv, sizeof(float) * 3 * N, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && !db) e = cudaMemcpyAsync(flags, &ctrl->flags, sizeof(*flags), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    // also after an error: the kernel may be writing to the buffer
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) return e;
     if (pos && dp == db) memcpy(pos, bp, sizeof(float) * 3 * N);
     if (vel && dv == db + 3 * N) memcpy(vel, bp + 3 * N, sizeof(float) * 3 * N);

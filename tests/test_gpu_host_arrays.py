@@ -2,6 +2,7 @@
 not reach goes through buffers and the driver's copies."""
 import ctypes as C
 import mmap
+from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
 import pytest
@@ -79,3 +80,20 @@ def test_device_array_is_left_to_the_driver(cloth_lib, nx, ny):
             assert np.array_equal(out.cpu().numpy(), sc.init_pos)
         else:
             assert rc == -3 and not out.any()  # CLOTH_ERR_CUDA
+
+
+def test_reads_at_the_same_time(cloth_lib):
+    """Reads share page-locked buffers, each taken for one read; twelve threads, more than are kept."""
+    scs = [scene(20 + i, 30, seed=i) for i in range(24)]
+    cls = [cloth_lib.Cloth(sc) for sc in scs]
+
+    def work(t):
+        for k in range(60):
+            i = 2 * t + k % 2
+            p, v = cls[i].read()
+            assert np.array_equal(p, scs[i].init_pos) and np.array_equal(v, scs[i].init_vel)
+
+    with ThreadPoolExecutor(12) as pool:
+        list(pool.map(work, range(12)))
+    for cl in cls:
+        cl.close()
