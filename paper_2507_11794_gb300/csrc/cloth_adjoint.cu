@@ -316,7 +316,10 @@ struct ClothRollout {
     float *final_state = nullptr;          // 6 planes
     int *map = nullptr;                    // canonical spring -> slot
     bool forward_done = false;
-    bool slots_hold_last = false;          // the slot sets hold the last segments as the forward pass recorded them
+    // the slot sets hold the last segments as the forward pass recorded them, with
+    // the kernel parameters and the constants of these generations
+    bool slots_hold_last = false;
+    unsigned long long rec_params = 0, rec_consts = 0;
     // the forward chain and the reverse pass (without and with slots_hold_last)
     // as CUDA graphs (captured on first use; rebuilt when the cloth's kernel
     // parameters change)
@@ -699,6 +702,7 @@ int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd
     if (d_ks && ro->S > 0) scatter_kernel<<<nblk(ro->S, 256), 256, 0, s>>>(d_ks, ro->map, ro->S, h->ks_slot);
     if (d_kd && ro->S > 0) scatter_kernel<<<nblk(ro->S, 256), 256, 0, s>>>(d_kd, ro->map, ro->S, h->kd_slot);
     RTRY(h, cudaGetLastError(), "constants scatter");
+    if (d_ks || d_kd) h->consts_gen++;
     set_k_kernel<<<1, 1, 0, s>>>(h->ctrl, ro->k0);
     RTRY(h, cudaGetLastError(), "set substep counter");
     RTRY(h, launch_aos_to_soa(ro->x0, d_v0 ? d_v0 : ro->v0, h->state, h->state + 6 * st, st, h->n, h->desc.nx,
@@ -707,6 +711,8 @@ int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd
     ro->slots_hold_last = false;
     RTRY(h, run_pass(ro, PASS_FORWARD, s), "forward chain");
     ro->slots_hold_last = true;
+    ro->rec_params = h->params_gen;
+    ro->rec_consts = h->consts_gen;
     h->substeps_done = (long long)ro->k_final;
     if (d_pos_out || d_vel_out)
         RTRY(h, launch_soa_to_aos(h->state, h->state + 6 * st, st, h->n, h->desc.nx, h->pitch, h->ctrl, d_pos_out,
@@ -732,7 +738,9 @@ int cloth_rollout_backward(ClothRollout *ro, const float *d_gpos, const float *d
     aos_planes_kernel<<<nblk(n, 256), 256, 0, s>>>(d_gpos, n, nx, h->pitch, st, lx);
     aos_planes_kernel<<<nblk(n, 256), 256, 0, s>>>(d_gvel, n, nx, h->pitch, st, lv);
     RTRY(h, cudaGetLastError(), "load output adjoints");
-    const bool recorded = ro->slots_hold_last;
+    // with another surface model, or another rollout's constants in the cloth, every segment is recomputed
+    const bool recorded =
+        ro->slots_hold_last && ro->rec_params == h->params_gen && ro->rec_consts == h->consts_gen;
     ro->slots_hold_last = recorded && ro->nseg <= 2;  // earlier segments' recomputes overwrite the sets
     RTRY(h, run_pass(ro, recorded ? PASS_BACKWARD_RECORDED : PASS_BACKWARD, s), "reverse pass");
     if (d_gv0) planes_aos_kernel<<<nblk(n, 256), 256, 0, s>>>(lv, n, nx, h->pitch, st, d_gv0);

@@ -341,6 +341,7 @@ struct ClothHandle {
     StepParams params{};
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // one step, by the parity of its first substep
     unsigned long long params_gen = 0;  // bumped by cloth_fill_params: graphs built from older params are stale
+    unsigned long long consts_gen = 0;  // bumped when a rollout writes the per-spring constants
     long long substeps_done = 0;
     bool dead = false;
 };

@@ -1,0 +1,47 @@
+"""What happens to a cloth between a rollout's forward and reverse pass: the
+reverse pass takes the segments that the forward pass recorded only while the
+cloth's surface model and constants are the ones they were recorded with.  Over
+more than two segments a second reverse pass recomputes all of them, so it shows
+what the first should have used."""
+import numpy as np
+import pytest
+import torch
+
+import cloth_scenes as cs
+from test_gpu_node_kernel import per_spring, scene
+
+pytestmark = pytest.mark.gpu
+
+
+def tensors(sc, scale=1.0):
+    return [torch.tensor(a * np.float32(s), device="cuda", requires_grad=True)
+            for a, s in ((sc.ks_spring, scale), (sc.kd_spring, 1.0), (sc.init_vel, 1.0))]
+
+
+@pytest.mark.parametrize("graph", [True, False])
+@pytest.mark.parametrize("change", ["model", "constants"])
+def test_change_before_the_reverse_pass(cloth_lib, graph, change):
+    from paper_2507_11794_gb300.rollout import Rollout
+    sc = per_spring(scene(23, 19, mesh=True, wind=False))
+    with cloth_lib.Cloth(sc, flags=0 if graph else cloth_lib.capi.CLOTH_FLAG_NO_GRAPH) as cl:
+        ro, other = Rollout(cl, 4, 1), Rollout(cl, 2, 1)
+        args = tensors(sc)
+
+        def loss():
+            pos, vel = ro(*args)
+            return (pos ** 2).sum() + vel.sum()
+
+        plain = torch.autograd.grad(loss(), args)
+        L = loss()
+        if change == "model":
+            cl.set_mesh(*cs.sphere_mesh(3, 0.3005))
+        else:
+            with torch.no_grad():
+                other(*[a.detach() for a in tensors(sc, 1.3)])
+        first = torch.autograd.grad(L, args, retain_graph=True)
+        again = torch.autograd.grad(L, args)
+        ro.close()
+        other.close()
+    for a, b in zip(first, again):
+        assert torch.equal(a, b)
+    assert not torch.equal(first[2], plain[2])  # the change matters
