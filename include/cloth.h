@@ -307,10 +307,9 @@ void cloth_batch_destroy(ClothBatch *b);
  * velocities.  The contact set of every substep is frozen at the one the
  * forward pass finds (the response is differentiated as a smooth map of the
  * start point and the path direction).  The forward pass stores the state
- * every checkpoint_every steps and records the last two segments into the two
- * slot sets; the backward pass starts from those and recomputes the earlier
- * segments, one at a time into a set that has been reversed (a second backward
- * pass recomputes all but up to two segments in all), so device memory grows as nsteps/checkpoint_every states plus
+ * every checkpoint_every steps; the backward pass recomputes one segment at
+ * a time into one of two slot sets while the previous segment is reversed,
+ * so device memory grows as nsteps/checkpoint_every states plus
  * 2 x (checkpoint_every x substeps + 1) slots of 19 planes.  The forward and
  * backward passes run as CUDA graphs captured on first use (rebuilt after
  * cloth_set_mesh) unless the cloth has CLOTH_FLAG_NO_GRAPH; the backward
@@ -332,6 +331,14 @@ int cloth_rollout_create(ClothHandle *h, int32_t nsteps, int32_t checkpoint_ever
  * d_vel_out ([N][3], either may be NULL); the cloth then holds that state. */
 int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd, const float *d_v0, float *d_pos_out,
                           float *d_vel_out);
+/* cloth_rollout_forward for a backward pass to follow: also records the last
+ * two segments into the two slot sets as they run, which the next backward pass
+ * then need not recompute (the same gradients, bit for bit, in less time than
+ * both passes take otherwise).  Recorded segments are dropped by
+ * cloth_set_mesh, by another rollout's constants on the same cloth and, over more
+ * than two segments, by the backward pass. */
+int cloth_rollout_forward_record(ClothRollout *ro, const float *d_ks, const float *d_kd, const float *d_v0,
+                                 float *d_pos_out, float *d_vel_out);
 /* Reverse pass of the last forward: d_gpos, d_gvel = dL/d(final positions,
  * velocities) ([N][3]; d_gvel may be NULL = 0).  Writes dL/dks, dL/dkd (S
  * floats) and dL/dv0 ([N][3]); any output may be NULL.  The cloth is left in

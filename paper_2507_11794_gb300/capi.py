@@ -40,7 +40,8 @@ EXPORTS = ("cloth_create", "cloth_set_mesh", "cloth_step", "cloth_read", "cloth_
            "cloth_batch_create", "cloth_batch_set_mesh", "cloth_batch_step", "cloth_batch_read",
            "cloth_batch_set_state", "cloth_batch_tune", "cloth_batch_set_tuning", "cloth_batch_get_tuning",
            "cloth_batch_sync", "cloth_batch_get_collision_stats", "cloth_batch_destroy",
-           "cloth_rollout_create", "cloth_rollout_forward", "cloth_rollout_backward", "cloth_rollout_destroy")
+           "cloth_rollout_create", "cloth_rollout_forward", "cloth_rollout_forward_record",
+           "cloth_rollout_backward", "cloth_rollout_destroy")
 
 
 class ClothError(RuntimeError):
@@ -143,6 +144,7 @@ def lib():
         V = C.c_void_p
         L.cloth_rollout_create.argtypes = [H, C.c_int32, C.c_int32, C.POINTER(C.c_void_p)]
         L.cloth_rollout_forward.argtypes = [H, V, V, V, V, V]
+        L.cloth_rollout_forward_record.argtypes = [H, V, V, V, V, V]
         L.cloth_rollout_backward.argtypes = [H, V, V, V, V, V]
         L.cloth_rollout_destroy.argtypes = [H]
         L.cloth_rollout_destroy.restype = None
@@ -352,6 +354,12 @@ def cloth_rollout_create(h: int, nsteps: int, checkpoint_every: int) -> int:
 def cloth_rollout_forward(r: int, d_ks: int, d_kd: int, d_v0: int, d_pos: int, d_vel: int):
     """Device addresses (ints, 0 = NULL)."""
     check(lib().cloth_rollout_forward(r, d_ks or None, d_kd or None, d_v0 or None, d_pos or None, d_vel or None))
+
+
+def cloth_rollout_forward_record(r: int, d_ks: int, d_kd: int, d_v0: int, d_pos: int, d_vel: int):
+    """cloth_rollout_forward with a backward pass to follow."""
+    check(lib().cloth_rollout_forward_record(r, d_ks or None, d_kd or None, d_v0 or None, d_pos or None,
+                                             d_vel or None))
 
 
 def cloth_rollout_backward(r: int, d_gpos: int, d_gvel: int, d_gks: int, d_gkd: int, d_gv0: int):

@@ -320,11 +320,11 @@ struct ClothRollout {
     // the kernel parameters and the constants of these generations
     bool slots_hold_last = false;
     unsigned long long rec_params = 0, rec_consts = 0;
-    // the forward chain and the reverse pass (without and with slots_hold_last)
-    // as CUDA graphs (captured on first use; rebuilt when the cloth's kernel
-    // parameters change)
-    cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};
-    unsigned long long graph_gen[3] = {0, 0, 0};
+    // the forward chain and the reverse pass, without and with recorded segments
+    // (PASS_*), as CUDA graphs (captured on first use; rebuilt when the cloth's
+    // kernel parameters change)
+    cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
+    unsigned long long graph_gen[4] = {0, 0, 0, 0};
 };
 
 namespace {
@@ -431,10 +431,13 @@ cudaError_t record_segment(ClothRollout *ro, int g, bool set_k, cudaStream_t s)
 
 // The forward chain from the restored initial state: a checkpoint before
 // every segment, the segment's substeps (the cloth's own launches), and a copy
-// of the final state.  The last two segments, the first that the reverse pass
-// needs, are recorded into the two slot sets as they run, so it has nothing to
-// recompute for them.
-cudaError_t enqueue_forward(ClothRollout *ro, cudaStream_t s)
+// of the final state.  record: the last two segments, the first that the reverse
+// pass needs, are recorded into the two slot sets as they run, so it has nothing
+// to recompute for them.  Without a reverse pass that is time lost: a recorded
+// substep writes 9 planes more, and all of them to memory of its own instead of
+// two buffers that stay in L2 (12 steps of 4 substeps on 160,000 nodes 699 -> 783
+// us, 8 steps on 640,000 493 -> 557).
+cudaError_t enqueue_forward(ClothRollout *ro, bool record, cudaStream_t s)
 {
     ClothHandle *h = ro->h;
     const long long st = h->stride;
@@ -443,7 +446,7 @@ cudaError_t enqueue_forward(ClothRollout *ro, cudaStream_t s)
     for (int g = 0; g < ro->nseg && e == cudaSuccess; g++) {
         e = copy_planes(cur, ro->ckpt + (size_t)g * 6 * st, 6 * st, s);
         const int n = seg_steps(ro, g) * h->desc.substeps;
-        if (g + 2 >= ro->nseg) {
+        if (record && g + 2 >= ro->nseg) {
             if (e == cudaSuccess) e = record_segment(ro, g, false, s);
             cur = seg_slot(ro, g & 1, n);
             continue;
@@ -453,10 +456,10 @@ cudaError_t enqueue_forward(ClothRollout *ro, cudaStream_t s)
             p.parity = (int)((ro->kseg[g] + (unsigned long long)q) & 1ull);
             e = launch_substep(p, s);
         }
-        cur = cur_state(h, ro->kseg[g + 1]);
+        cur = cur_state(h, g + 1 < ro->nseg ? ro->kseg[g + 1] : ro->k_final);
     }
     if (e == cudaSuccess) e = copy_planes(cur, ro->final_state, 6 * st, s);
-    if (e == cudaSuccess) e = copy_planes(cur, cur_state(h, ro->k_final), 6 * st, s);
+    if (e == cudaSuccess && record) e = copy_planes(cur, cur_state(h, ro->k_final), 6 * st, s);
     return e;
 }
 
@@ -553,13 +556,14 @@ cudaError_t capture_graph(ClothHandle *h, cudaGraphExec_t *exec, F &&body)
 
 // Runs the forward chain or the reverse pass on s, through a cached graph
 // unless the cloth was created with CLOTH_FLAG_NO_GRAPH.
-enum { PASS_FORWARD = 0, PASS_BACKWARD = 1, PASS_BACKWARD_RECORDED = 2 };
+enum { PASS_FORWARD = 0, PASS_FORWARD_RECORD = 1, PASS_BACKWARD = 2, PASS_BACKWARD_RECORDED = 3 };
 cudaError_t run_pass(ClothRollout *ro, int pass, cudaStream_t s)
 {
     ClothHandle *h = ro->h;
     auto body = [ro, pass](cudaStream_t cs) {
-        return pass == PASS_FORWARD ? enqueue_forward(ro, cs)
-                                    : enqueue_backward(ro, pass == PASS_BACKWARD_RECORDED, cs);
+        return pass == PASS_FORWARD || pass == PASS_FORWARD_RECORD
+                   ? enqueue_forward(ro, pass == PASS_FORWARD_RECORD, cs)
+                   : enqueue_backward(ro, pass == PASS_BACKWARD_RECORDED, cs);
     };
     if (h->desc.flags & CLOTH_FLAG_NO_GRAPH) return body(s);
     cudaGraphExec_t &gx = ro->graph[pass];
@@ -690,8 +694,8 @@ int cloth_rollout_create(ClothHandle *h, int32_t nsteps, int32_t checkpoint_ever
     return CLOTH_OK;
 }
 
-int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd, const float *d_v0, float *d_pos_out,
-                          float *d_vel_out)
+static int rollout_forward(ClothRollout *ro, bool record, const float *d_ks, const float *d_kd, const float *d_v0,
+                           float *d_pos_out, float *d_vel_out)
 {
     if (!ro || !ro->h) return rfail(CLOTH_ERR_INVALID_ARG, "null rollout");
     ClothHandle *h = ro->h;
@@ -709,8 +713,8 @@ int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd
                               h->pitch, h->ctrl, s),
          "initial state");
     ro->slots_hold_last = false;
-    RTRY(h, run_pass(ro, PASS_FORWARD, s), "forward chain");
-    ro->slots_hold_last = true;
+    RTRY(h, run_pass(ro, record ? PASS_FORWARD_RECORD : PASS_FORWARD, s), "forward chain");
+    ro->slots_hold_last = record;
     ro->rec_params = h->params_gen;
     ro->rec_consts = h->consts_gen;
     h->substeps_done = (long long)ro->k_final;
@@ -720,6 +724,18 @@ int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd
              "final state");
     ro->forward_done = true;
     return CLOTH_OK;
+}
+
+int cloth_rollout_forward(ClothRollout *ro, const float *d_ks, const float *d_kd, const float *d_v0, float *d_pos_out,
+                          float *d_vel_out)
+{
+    return rollout_forward(ro, false, d_ks, d_kd, d_v0, d_pos_out, d_vel_out);
+}
+
+int cloth_rollout_forward_record(ClothRollout *ro, const float *d_ks, const float *d_kd, const float *d_v0,
+                                 float *d_pos_out, float *d_vel_out)
+{
+    return rollout_forward(ro, true, d_ks, d_kd, d_v0, d_pos_out, d_vel_out);
 }
 
 int cloth_rollout_backward(ClothRollout *ro, const float *d_gpos, const float *d_gvel, float *d_gks, float *d_gkd,

@@ -20,12 +20,12 @@ from . import capi
 
 class _RolloutFn(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, ks, kd, v0, ro):
+    def forward(ctx, ks, kd, v0, ro, record):
         n = ro.cloth.n
         pos = torch.empty((n, 3), dtype=torch.float32, device=ks.device)
         vel = torch.empty((n, 3), dtype=torch.float32, device=ks.device)
-        capi.cloth_rollout_forward(ro.r, ks.data_ptr(), kd.data_ptr(), v0.data_ptr(), pos.data_ptr(),
-                                   vel.data_ptr())
+        forward = capi.cloth_rollout_forward_record if record else capi.cloth_rollout_forward
+        forward(ro.r, ks.data_ptr(), kd.data_ptr(), v0.data_ptr(), pos.data_ptr(), vel.data_ptr())
         ctx.ro = ro
         ctx.shapes = (ks.shape, kd.shape, v0.shape)
         return pos, vel
@@ -42,7 +42,7 @@ class _RolloutFn(torch.autograd.Function):
         gv = gvel.contiguous() if gvel is not None else None
         capi.cloth_rollout_backward(ro.r, gp.data_ptr(), gv.data_ptr() if gv is not None else 0, gks.data_ptr(),
                                     gkd.data_ptr(), gv0.data_ptr())
-        return gks, gkd, gv0, None
+        return gks, gkd, gv0, None, None
 
 
 class Rollout:
@@ -57,7 +57,9 @@ class Rollout:
         for t in (ks, kd, v0):
             if not (t.is_cuda and t.dtype == torch.float32 and t.is_contiguous()):
                 raise ValueError("ks, kd, v0 must be contiguous CUDA float32 tensors")
-        return _RolloutFn.apply(ks, kd, v0, self)
+        # segments are recorded for a backward pass only where there can be one
+        record = torch.is_grad_enabled() and any(t.requires_grad for t in (ks, kd, v0))
+        return _RolloutFn.apply(ks, kd, v0, self, record)
 
     def close(self):
         if getattr(self, "r", None):
