@@ -46,17 +46,14 @@ __device__ __forceinline__ float dot_rn(float a, float b, float c, float d, floa
     return __fmaf_rn(e, f, __fmaf_rn(a, b, __fmul_rn(c, d)));
 }
 
-// One candidate: grid entry e met in cell (cx, cy, cz) of a box whose low
-// corner is (lox, loy, loz).  Returns true on a hit, with th the distance
-// along r, over = th - delta (of the rounded th, whichever lane adds it up) and
-// f = 1/a (a = e1 . (r x e2)); A, B, C receive the triangle record (v0, e1, e2).
-__device__ __forceinline__ bool coll_candidate(const StepParams &p, const CollPath &q, long long e, int cx, int cy,
-                                               int cz, int lox, int loy, int loz, float &th, float &over, float &f,
-                                               float4 &A, float4 &B, float4 &C)
+// One candidate: triangle record (A, B, C) = (v0, e1, e2) met in cell
+// (cx, cy, cz) of a box whose low corner is (lox, loy, loz).  Returns true on a
+// hit, with th the distance along r, over = th - delta (of the rounded th,
+// whichever lane adds it up) and f = 1/a (a = e1 . (r x e2)).
+__device__ __forceinline__ bool coll_test(const StepParams &p, const CollPath &q, const float4 &A, const float4 &B,
+                                          const float4 &C, int cx, int cy, int cz, int lox, int loy, int loz, float &th,
+                                          float &over, float &f)
 {
-    A = __ldg(p.etri + 3 * e);
-    B = __ldg(p.etri + 3 * e + 1);
-    C = __ldg(p.etri + 3 * e + 2);
     // the record's w lanes hold the low cell of the triangle's box
     if (max(__float_as_int(A.w), lox) != cx || max(__float_as_int(B.w), loy) != cy ||
         max(__float_as_int(C.w), loz) != cz)
@@ -79,6 +76,17 @@ __device__ __forceinline__ bool coll_candidate(const StepParams &p, const CollPa
     over = __fsub_rn(th, p.delta);
     if (v < 0.0f || u + v > 1.0f) return false;
     return th > p.tmin && th < q.L;
+}
+
+// The same for grid entry e; A, B, C receive its record.
+__device__ __forceinline__ bool coll_candidate(const StepParams &p, const CollPath &q, long long e, int cx, int cy,
+                                               int cz, int lox, int loy, int loz, float &th, float &over, float &f,
+                                               float4 &A, float4 &B, float4 &C)
+{
+    A = __ldg(p.etri + 3 * e);
+    B = __ldg(p.etri + 3 * e + 1);
+    C = __ldg(p.etri + 3 * e + 2);
+    return coll_test(p, q, A, B, C, cx, cy, cz, lox, loy, loz, th, over, f);
 }
 
 // Point S + th r of a path, each coordinate one rounded fused multiply-add,
@@ -325,16 +333,31 @@ __device__ __noinline__ unsigned coll_wide(const StepParams &p, const CollPath q
     return tested;
 }
 
+// Where the entries of a cell start and end.
+__device__ __forceinline__ int2 coll_run(const StepParams &p, int cx, int cy, int cz)
+{
+    const int *c = p.cell_start + ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
+    return make_int2(__ldg(c), __ldg(c + 1));
+}
+
 // The hits of every lane's path (ncell cells of its box; 0: none), G lanes per
 // path: the lanes of a group are neighbours in the warp, bring the same path
-// and end with the same sums.  wide: the path has more than the caller's limit
-// of cells (ncell = 0) and is walked by the whole warp; its candidates are
-// counted with COUNT_WIDE.  src.params(cloth) are the path's parameters.
-// ntest accumulates, in a group's first lane, the candidates.
-template <int G, bool COUNT_WIDE, class Src, class Hits>
+// and end with the same sums.  run: the first cell's entries (coll_run).  wide:
+// the path has more than the caller's limit of cells (ncell = 0) and is walked by
+// the whole warp; its candidates are counted with COUNT_WIDE.  src.params(cloth)
+// are the path's parameters.  ntest accumulates, in a group's first lane, the
+// candidates.
+//
+// A lane's time is a chain of loads: of 17 filter words in a cell, four at a time
+// and the last one alone, 3,100 cycles, then 1,400 per survivor (256 x 256 nodes
+// pulled over 81,920 triangles, one lane per node; twice that from DRAM).  DEEP,
+// for kernels with the registers for it, has up to eight filter words in flight,
+// past the end the last one again, and with one lane per path the next survivor's
+// record.
+template <int G, bool COUNT_WIDE, bool DEEP, class Src, class Hits>
 __device__ __forceinline__ void coll_cells(const Src &src, int cloth, const StepParams &p, const CollPath &q,
-                                           const CollBox &bx, const CollWords &w, int ncell, bool wide, Hits &s,
-                                           unsigned &ntest)
+                                           const CollBox &bx, const CollWords &w, int2 run, int ncell, bool wide,
+                                           Hits &s, unsigned &ntest)
 {
     constexpr unsigned FULLW = 0xffffffffu;
     const int lane = threadIdx.x & 31, sub = lane % G, gbase = lane - sub;
@@ -343,9 +366,9 @@ __device__ __forceinline__ void coll_cells(const Src &src, int cloth, const Step
     for (int c = 0; c < ncw; c++) {
         int e0 = 0, cnt = 0;
         if (c < ncell) {
-            const long long cell = ((long long)cz * p.gd[1] + cy) * p.gd[0] + cx;
-            e0 = __ldg(p.cell_start + cell);
-            cnt = __ldg(p.cell_start + cell + 1) - e0;
+            if (c > 0) run = coll_run(p, cx, cy, cz);
+            e0 = run.x;
+            cnt = run.y - e0;
             if (sub == 0) ntest += (unsigned)cnt;
         }
         const unsigned need = coll_need(bx, cx, cy, cz);
@@ -355,10 +378,43 @@ __device__ __forceinline__ void coll_cells(const Src &src, int cloth, const Step
             const int n = min(own - b, 32);
             unsigned m = 0u;  // the entries of this run that pass the filter
             const uint4 *fil = p.efil + e0 + b;
+            if constexpr (DEEP) {
+                constexpr int U = G > 4 ? 32 / G : 8;  // words in flight
+                for (int t = sub; t < n; t += U * G) {
+                    uint4 f[U];
+#pragma unroll
+                    for (int j = 0; j < U; j++) f[j] = __ldg(fil + min(t + j * G, n - 1));
+#pragma unroll
+                    for (int j = 0; j < U; j++) m |= (unsigned)coll_overlap(f[j], w, need) << ((t + j * G) & 31);
+                }
+                if (n > 0) m &= 0xffffffffu >> (32 - n);
+                else m = 0u;
+            } else {
 #pragma unroll 4
-            for (int t = sub; t < n; t += G) m |= (unsigned)coll_overlap(__ldg(fil + t), w, need) << t;
+                for (int t = sub; t < n; t += G) m |= (unsigned)coll_overlap(__ldg(fil + t), w, need) << t;
+            }
 #pragma unroll
             for (int d = 1; d < G; d <<= 1) m |= __shfl_xor_sync(FULLW, m, d);
+            if constexpr (DEEP && G == 1) {
+                float4 nA, nB, nC;  // the next survivor's record
+                int t = __ffs((int)m) - 1;
+                auto fetch = [&]() {
+                    const float4 *r = p.etri + 3 * ((long long)e0 + b + t);
+                    nA = __ldg(r); nB = __ldg(r + 1); nC = __ldg(r + 2);
+                };
+                if (t >= 0) fetch();
+                while (__any_sync(FULLW, t >= 0)) {
+                    if (t >= 0) {
+                        const float4 A = nA, B = nB, C = nC;
+                        m &= m - 1u;
+                        t = __ffs((int)m) - 1;
+                        if (t >= 0) fetch();
+                        float th, over, f;
+                        const bool hit = coll_test(p, q, A, B, C, cx, cy, cz, bx.lox, bx.loy, bx.loz, th, over, f);
+                        s.template add<1>(p, q, hit, th, over, f, B, C);
+                    }
+                }
+            }
             while (__any_sync(FULLW, m != 0u)) {
                 // the group's next G survivors, one per lane in entry order
                 unsigned mine = m;
@@ -417,9 +473,9 @@ __device__ __forceinline__ void coll_cells(const Src &src, int cloth, const Step
 }
 
 // The response of every group's path S -> E (valid: whether it has one; o: its
-// node's plane offset), G lanes per path.  True in the group's first lane if
+// node's plane offset), G lanes per path; DEEP: see coll_cells.  True in the group's first lane if
 // the node hits, with its position x; REC also records the response data.
-template <bool REC, int G, class Src>
+template <bool REC, int G, bool DEEP, class Src>
 __device__ __forceinline__ bool collide_path(const Src &src, int cloth, const StepParams &p, bool valid, float sx,
                                              float sy, float sz, float ex, float ey, float ez, long long o, float3 &x,
                                              unsigned &ntest)
@@ -429,15 +485,19 @@ __device__ __forceinline__ bool collide_path(const Src &src, int cloth, const St
     CollWords w = {0u, 0u, 0u};
     int ncell = 0;
     bool wide = false;
-    if (valid && coll_path(p, sx, sy, sz, ex, ey, ez, q)) {
+    int2 run = make_int2(0, 0);
+    if (valid) {
         bx = coll_box(p, sx, sy, sz, ex, ey, ez);
-        w = coll_words(p, sx, sy, sz, ex, ey, ez, q);
-        const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
-        wide = nc > COLL_MAXC;
-        ncell = wide ? 0 : (int)nc;
+        run = coll_run(p, bx.lox, bx.loy, bx.loz);  // loads while the direction is computed
+        if (coll_path(p, sx, sy, sz, ex, ey, ez, q)) {
+            w = coll_words(p, sx, sy, sz, ex, ey, ez, q);
+            const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
+            wide = nc > COLL_MAXC;
+            ncell = wide ? 0 : (int)nc;
+        }
     }
     NodeHits<REC> s = {};
-    coll_cells<G, false>(src, cloth, p, q, bx, w, ncell, wide, s, ntest);
+    coll_cells<G, false, DEEP>(src, cloth, p, q, bx, w, run, ncell, wide, s, ntest);
     if (s.K == 0 || (threadIdx.x & 31) % G != 0) return false;
     const float m = s.acc / (float)s.K;
     // product and sum rounded separately, the same bits in every kernel
@@ -473,7 +533,7 @@ __device__ __forceinline__ void collide_round(const Src &src, unsigned long long
         ex = out[o]; ey = out[st + o]; ez = out[2 * st + o];
     }
     float3 x;
-    if (collide_path<REC, G>(src, cloth, p, valid, sx, sy, sz, ex, ey, ez, o, x, ntest)) {
+    if (collide_path<REC, G, false>(src, cloth, p, valid, sx, sy, sz, ex, ey, ez, o, x, ntest)) {
         out[o] = x.x;
         out[st + o] = x.y;
         out[2 * st + o] = x.z;
@@ -680,6 +740,7 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
         CollBox bx = {0, 0, 0, 0, 0, 0};
         CollWords w = {0u, 0u, 0u};
         EdgeHits s = {make_float4(0.0f, 0.0f, 0.0f, 0.0f), 0};
+        int2 run = make_int2(0, 0);
         if (i < n) {
             const int o = __ldg(p.coll_list + i);
             const int r = o / p.pitch, cc = o - r * p.pitch;
@@ -690,8 +751,9 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
                 const long long ob = (long long)rb * p.pitch + cb;
                 const float x0 = xs[o], y0 = xs[st + o], z0 = xs[2 * st + o];
                 const float x1 = xs[ob], y1 = xs[st + ob], z1 = xs[2 * st + ob];
+                bx = coll_box(p, x0, y0, z0, x1, y1, z1);
+                run = coll_run(p, bx.lox, bx.loy, bx.loz);
                 if (coll_path(p, x0, y0, z0, x1, y1, z1, path)) {
-                    bx = coll_box(p, x0, y0, z0, x1, y1, z1);
                     w = coll_words(p, x0, y0, z0, x1, y1, z1, path);
                     const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
                     wide = nc > EDGE_MAXC;
@@ -699,7 +761,7 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
                 }
             }
         }
-        coll_cells<G, true>(OneCloth{p}, 0, p, path, bx, w, ncell, wide, s, ntest);
+        coll_cells<G, true, false>(OneCloth{p}, 0, p, path, bx, w, run, ncell, wide, s, ntest);
         if (has && lane % G == 0) {
             p.edge_hit[s.slot] = s.rec;
             nhit += s.rec.w > 0.0f ? 1u : 0u;

@@ -335,7 +335,7 @@ __device__ __forceinline__ void node_substep(const StepParams &p, const int par,
                     const int j = valid ? s_list[i] : 0;
                     const unsigned o = base + (unsigned)j;
                     float3 x;
-                    if (collide_path<REC, G>(OneCloth{p}, 0, p, valid, s_x[0][j], s_x[1][j], s_x[2][j], s_x[3][j],
+                    if (collide_path<REC, G, true>(OneCloth{p}, 0, p, valid, s_x[0][j], s_x[1][j], s_x[2][j], s_x[3][j],
                                              s_x[4][j], s_x[5][j], (long long)o, x, ntest)) {
                         out[o] = x.x;
                         out[o + st] = x.y;
