@@ -126,7 +126,7 @@ cudaError_t rebuild(ClothBatch *b)
     b->args.coll_cloth = b->coll_cloth;
     b->args.coll_count = b->ctrl->coll_count;
     b->args.walk_blocks = b->sm_count * b->ctas_per_sm;
-    b->args.coll_blocks = b->sm_count * CLOTH_COLL_CTAS_PER_SM;
+    b->args.coll_blocks = b->sm_count * CLOTH_BATCH_COLL_CTAS_PER_SM;
     // one walk variant for the whole batch when every cloth has the same one
     int var = -1;
     for (const StepParams &q : prm) {

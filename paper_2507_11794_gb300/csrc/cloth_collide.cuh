@@ -342,16 +342,16 @@ __device__ __forceinline__ int2 coll_run(const StepParams &p, int cx, int cy, in
 
 // The hits of every lane's path (ncell cells of its box; 0: none), G lanes per
 // path: the lanes of a group are neighbours in the warp, bring the same path
-// and end with the same sums.  run: the first cell's entries (coll_run).  wide:
-// the path has more than the caller's limit of cells (ncell = 0) and is walked by
-// the whole warp; its candidates are counted with COUNT_WIDE.  src.params(cloth)
-// are the path's parameters.  ntest accumulates, in a group's first lane, the
-// candidates.
+// and end with the same sums.  wide: the path has more than the caller's limit of
+// cells (ncell = 0) and is walked by the whole warp; its candidates are counted
+// with COUNT_WIDE.  src.params(cloth) are the path's parameters.  ntest
+// accumulates, in a group's first lane, the candidates.
 //
 // A lane's time is a chain of loads: of 17 filter words in a cell, four at a time
 // and the last one alone, 3,100 cycles, then 1,400 per survivor (256 x 256 nodes
 // pulled over 81,920 triangles, one lane per node; twice that from DRAM).  DEEP,
-// for kernels with the registers for it, has up to eight filter words in flight,
+// for kernels with the registers for it, takes the first cell's entries (run) from
+// the caller, who can load them ahead, and has up to eight filter words in flight,
 // past the end the last one again, and with one lane per path the next survivor's
 // record.
 template <int G, bool COUNT_WIDE, bool DEEP, class Src, class Hits>
@@ -366,7 +366,7 @@ __device__ __forceinline__ void coll_cells(const Src &src, int cloth, const Step
     for (int c = 0; c < ncw; c++) {
         int e0 = 0, cnt = 0;
         if (c < ncell) {
-            if (c > 0) run = coll_run(p, cx, cy, cz);
+            if (c > 0 || !DEEP) run = coll_run(p, cx, cy, cz);
             e0 = run.x;
             cnt = run.y - e0;
             if (sub == 0) ntest += (unsigned)cnt;
@@ -488,7 +488,7 @@ __device__ __forceinline__ bool collide_path(const Src &src, int cloth, const St
     int2 run = make_int2(0, 0);
     if (valid) {
         bx = coll_box(p, sx, sy, sz, ex, ey, ez);
-        run = coll_run(p, bx.lox, bx.loy, bx.loz);  // loads while the direction is computed
+        if (DEEP) run = coll_run(p, bx.lox, bx.loy, bx.loz);  // loads while the direction is computed
         if (coll_path(p, sx, sy, sz, ex, ey, ez, q)) {
             w = coll_words(p, sx, sy, sz, ex, ey, ez, q);
             const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
@@ -507,20 +507,37 @@ __device__ __forceinline__ bool collide_path(const Src &src, int cloth, const St
     return true;
 }
 
+// A lane's first list entry and its path, loaded ahead by the kernel (p.parity
+// is the substep's).  Any offset is taken: one outside the planes reads node 0.
+struct CollFirst {
+    int o;
+    float sx, sy, sz, ex, ey, ez;
+
+    __device__ __forceinline__ void load(const StepParams &p, int entry)
+    {
+        const long long st = p.stride;
+        const float *in = (p.parity & 1) ? p.state1 : p.state0, *out = (p.parity & 1) ? p.state0 : p.state1;
+        o = entry >= 0 && entry < st ? entry : 0;
+        sx = __ldg(in + o); sy = __ldg(in + st + o); sz = __ldg(in + 2 * st + o);
+        ex = out[o]; ey = out[st + o]; ez = out[2 * st + o];
+    }
+};
+
 // One round of the list pass, G lanes per node: every group brings one entry
 // (valid: whether it has one; i: its index for src.entry).  Src supplies
-// entry(i, cloth, offset) and params(cloth).  has_pre: the entry's offset is
-// pre_o, loaded by the caller (cloth 0).  ntest and nhit accumulate, in the
+// entry(i, cloth, offset), params(cloth) and DEEP (see coll_cells).  ahead: the
+// entry was loaded ahead (first; cloth 0).  ntest and nhit accumulate, in the
 // group's first lane, the candidate triangles and whether the node hit.  REC:
 // also records the hits' response data (coll_record).
 template <bool REC, int G, class Src>
 __device__ __forceinline__ void collide_round(const Src &src, unsigned long long k, bool valid, unsigned long long i,
-                                              float &fsum, unsigned &ntest, unsigned &nhit, bool has_pre, int pre_o)
+                                              float &fsum, unsigned &ntest, unsigned &nhit, bool ahead,
+                                              const CollFirst *first)
 {
     int cloth = 0;
     long long o = 0;
     if (valid) {
-        if (has_pre) o = pre_o;
+        if (ahead) o = first->o;
         else src.entry(i, cloth, o);
     }
     const StepParams &p = src.params(cloth);
@@ -528,12 +545,15 @@ __device__ __forceinline__ void collide_round(const Src &src, unsigned long long
     const float *in = (k & 1ull) ? p.state1 : p.state0;
     float *out = (k & 1ull) ? p.state0 : p.state1;
     float sx = 0.0f, sy = 0.0f, sz = 0.0f, ex = 0.0f, ey = 0.0f, ez = 0.0f;
-    if (valid) {
+    if (ahead) {
+        sx = first->sx; sy = first->sy; sz = first->sz;
+        ex = first->ex; ey = first->ey; ez = first->ez;
+    } else if (valid) {
         sx = __ldg(in + o); sy = __ldg(in + st + o); sz = __ldg(in + 2 * st + o);
         ex = out[o]; ey = out[st + o]; ez = out[2 * st + o];
     }
     float3 x;
-    if (collide_path<REC, G, false>(src, cloth, p, valid, sx, sy, sz, ex, ey, ez, o, x, ntest)) {
+    if (collide_path<REC, G, Src::DEEP>(src, cloth, p, valid, sx, sy, sz, ex, ey, ez, o, x, ntest)) {
         out[o] = x.x;
         out[st + o] = x.y;
         out[2 * st + o] = x.z;
@@ -549,8 +569,8 @@ __device__ __forceinline__ void collide_round(const Src &src, unsigned long long
 // warp and round.  A list of fewer chunks than warps is dealt over the CTAs
 // first (every SM gets some); a longer one in runs of COLL_WARPS chunks per
 // CTA, so that a CTA's warps share the lines of the cells they read.
-// has_pre: the lane's entry of the first round with G = COLL_GMAX and fewer
-// chunks than warps (index coll_first_index()) is pre_o.
+// ahead: the lane's entry of the first round with G = COLL_GMAX and fewer
+// chunks than warps (index coll_first_index()), or null.
 constexpr int COLL_GMAX = 8;
 __device__ __forceinline__ unsigned coll_first_index()
 {
@@ -559,7 +579,7 @@ __device__ __forceinline__ unsigned coll_first_index()
 }
 template <bool REC, int G, class Src>
 __device__ __forceinline__ void collide_chunks(const Src &src, unsigned long long k, unsigned n, float &fsum,
-                                               unsigned &ntest, unsigned &nhit, bool has_pre, int pre_o)
+                                               unsigned &ntest, unsigned &nhit, const CollFirst *ahead)
 {
     constexpr unsigned PER = 32 / G;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -568,7 +588,7 @@ __device__ __forceinline__ void collide_chunks(const Src &src, unsigned long lon
     const unsigned first = deal ? (unsigned)wib * gridDim.x + blockIdx.x : blockIdx.x * COLL_WARPS + wib;
     for (unsigned c = first; c < chunks; c += nw) {
         const unsigned long long i = (unsigned long long)PER * c + (unsigned)(lane / G);
-        collide_round<REC, G>(src, k, i < n, i, fsum, ntest, nhit, has_pre && deal && c == first, pre_o);
+        collide_round<REC, G>(src, k, i < n, i, fsum, ntest, nhit, G == COLL_GMAX && ahead && deal && c == first, ahead);
     }
 }
 // Lanes per node: a short list leaves most of the grid's lanes idle and is
@@ -578,15 +598,15 @@ __device__ __forceinline__ void collide_chunks(const Src &src, unsigned long lon
 // the first form is compiled in.
 template <bool REC, bool SHORT, class Src>
 __device__ __forceinline__ void collide_list(const Src &src, unsigned long long k, unsigned n, float &fsum,
-                                             unsigned &ntest, unsigned &nhit, bool has_pre = false, int pre_o = 0)
+                                             unsigned &ntest, unsigned &nhit, const CollFirst *ahead = nullptr)
 {
     const unsigned lanes = gridDim.x * 32u * COLL_WARPS;
     if (SHORT || n <= lanes / COLL_GMAX)
-        collide_chunks<REC, COLL_GMAX>(src, k, n, fsum, ntest, nhit, has_pre, pre_o);
+        collide_chunks<REC, COLL_GMAX>(src, k, n, fsum, ntest, nhit, ahead);
     else if (n <= lanes / 2u)
-        collide_chunks<REC, 2>(src, k, n, fsum, ntest, nhit, false, 0);
+        collide_chunks<REC, 2>(src, k, n, fsum, ntest, nhit, nullptr);
     else
-        collide_chunks<REC, 1>(src, k, n, fsum, ntest, nhit, false, 0);
+        collide_chunks<REC, 1>(src, k, n, fsum, ntest, nhit, nullptr);
 }
 
 // One thread of a CTA adds its counts to the cloth's running statistics.  The
@@ -740,7 +760,6 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
         CollBox bx = {0, 0, 0, 0, 0, 0};
         CollWords w = {0u, 0u, 0u};
         EdgeHits s = {make_float4(0.0f, 0.0f, 0.0f, 0.0f), 0};
-        int2 run = make_int2(0, 0);
         if (i < n) {
             const int o = __ldg(p.coll_list + i);
             const int r = o / p.pitch, cc = o - r * p.pitch;
@@ -751,9 +770,8 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
                 const long long ob = (long long)rb * p.pitch + cb;
                 const float x0 = xs[o], y0 = xs[st + o], z0 = xs[2 * st + o];
                 const float x1 = xs[ob], y1 = xs[st + ob], z1 = xs[2 * st + ob];
-                bx = coll_box(p, x0, y0, z0, x1, y1, z1);
-                run = coll_run(p, bx.lox, bx.loy, bx.loz);
                 if (coll_path(p, x0, y0, z0, x1, y1, z1, path)) {
+                    bx = coll_box(p, x0, y0, z0, x1, y1, z1);
                     w = coll_words(p, x0, y0, z0, x1, y1, z1, path);
                     const long long nc = (long long)(bx.hix - bx.lox + 1) * (bx.hiy - bx.loy + 1) * (bx.hiz - bx.loz + 1);
                     wide = nc > EDGE_MAXC;
@@ -761,7 +779,7 @@ __device__ __forceinline__ void edge_test_chunks(const StepParams &p, unsigned l
                 }
             }
         }
-        coll_cells<G, true, false>(OneCloth{p}, 0, p, path, bx, w, run, ncell, wide, s, ntest);
+        coll_cells<G, true, false>(OneCloth{p}, 0, p, path, bx, w, make_int2(0, 0), ncell, wide, s, ntest);
         if (has && lane % G == 0) {
             p.edge_hit[s.slot] = s.rec;
             nhit += s.rec.w > 0.0f ? 1u : 0u;

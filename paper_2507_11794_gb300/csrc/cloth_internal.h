@@ -100,22 +100,25 @@ struct StepParams {
 // with more hits is walked again by the gather pass).
 #define CLOTH_EDGE_MORE 3
 
-// The collision kernels come in two forms (see collide_list): for cloths
-// of up to COLL_SHORT_NODES per SM, whose lists leave lanes idle, and for more.
-// Grids are at most what is resident at once, and no more than give every node
-// its eight lanes.
+// The collision kernel of one cloth comes in two forms (see collide_list): for
+// cloths of up to COLL_SHORT_NODES per SM, whose lists leave lanes idle, and for
+// more.  Grids are at most what is resident at once, and no more than give every
+// node its eight lanes.  Three CTAs per SM have 80 registers a thread, which hold
+// a short list's chain of loads almost without spills; a batch's lists are long
+// and it runs four of 64 (1.45M nodes of 12 cloths: 139.8 us per substep, three
+// CTAs 142.3).
 #ifndef CLOTH_COLL_CTAS_PER_SM
-#define CLOTH_COLL_CTAS_PER_SM 4
+#define CLOTH_COLL_CTAS_PER_SM 3
 #endif
-#ifndef CLOTH_COLL_SHORT_CTAS_PER_SM
-#define CLOTH_COLL_SHORT_CTAS_PER_SM 3
+#ifndef CLOTH_BATCH_COLL_CTAS_PER_SM
+#define CLOTH_BATCH_COLL_CTAS_PER_SM 4
 #endif
 #define COLL_SHORT_NODES 128
 inline bool coll_short(long long n, int sms) { return n <= (long long)COLL_SHORT_NODES * sms; }
 inline int coll_ctas(long long n, int sms)
 {
     const long long want = (8 * n + 255) / 256;
-    const long long most = (long long)sms * (coll_short(n, sms) ? CLOTH_COLL_SHORT_CTAS_PER_SM : CLOTH_COLL_CTAS_PER_SM);
+    const long long most = (long long)sms * CLOTH_COLL_CTAS_PER_SM;
     return (int)(want < 1 ? 1 : (want > most ? most : want));
 }
 

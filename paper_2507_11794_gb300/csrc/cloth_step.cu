@@ -22,6 +22,7 @@
 // results are bitwise reproducible.  The first two rows of each walk only
 // produce the springs that reach into the strip.
 #include <cuda.h>
+#include <stddef.h>
 #include <string.h>
 
 #include <mutex>
@@ -40,9 +41,6 @@ namespace {
 #endif
 #ifndef CLOTH_WALK_UNROLL
 #define CLOTH_WALK_UNROLL 1
-#endif
-#ifndef CLOTH_COLL_MINB
-#define CLOTH_COLL_MINB 4
 #endif
 // the edge test holds its hit point beside the path: 80 registers without
 // spills beat a fourth CTA per SM (308 against 318 us on 256 x 256 nodes)
@@ -558,18 +556,18 @@ __global__ void CLOTH_WALK_BOUNDS substep_kernel(const StepParams p)
 // then the substep counter advances.
 
 // Start of a collision kernel (one thread per CTA): the substep and the number
-// of nodes its walk listed.
+// of nodes its walk listed, in one load (every CTA's goes to the same line of L2).
 __device__ __forceinline__ void coll_begin(DevCtrl *ctrl, unsigned long long &k, unsigned &n)
 {
-    const volatile DevCtrl *c = ctrl;
-    const unsigned long long kc = c->kc;
-    const unsigned n0 = c->coll_count[0], n1 = c->coll_count[1];
-    k = kc;
-    n = (kc & 1ull) ? n1 : n0;
+    static_assert(offsetof(DevCtrl, kc) % 16 == 0 && offsetof(DevCtrl, coll_count) == offsetof(DevCtrl, kc) + 8, "");
+    unsigned long long counts;
+    asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(k), "=l"(counts) : "l"(&ctrl->kc));
+    n = (unsigned)((k & 1ull) ? counts >> 32 : counts);
 }
 
 // List entries of one cloth.
 struct OneClothList {
+    static constexpr bool DEEP = true;
     const StepParams &p;
     __device__ void entry(unsigned long long i, int &cloth, long long &o) const
     {
@@ -583,27 +581,37 @@ struct OneClothList {
 // collide_list); the first CTA advances the substep counter.
 // REC: the adjoint recompute's variant, which also records each hit's
 // response data (p.cdata, p.cbits).
-// Bound by its chain of dependent loads (list entry, state, cell, filter
-// words, records, response) on short lists and by issue slots on long ones.
-// SHORT (see collide_list) holds three CTAs per SM without spilling much, the
-// long form four of 64 registers.  Measured per step of cloth_step against the
-// pass that spread every candidate's full test over the warp: 256 x 256 nodes
-// lying on 81,920 triangles (784,000 candidates a substep) 26 -> 16 us per
-// substep, 1.45M nodes in a batch (24.7M candidates) 437 -> 84 us (ncu);
-// the long form at three CTAs per SM is 8 % slower on the first, SHORT at two
-// 9 % on a rollout's 16,384 nodes.
+// Runs behind the walk (cloths of more than 12 CTAs of 64 positions per SM),
+// behind the listing form of node_kernel (8 to 12) and in cloth_profile_substeps and
+// the atomic path at any size; SHORT (see collide_list) in these two alone.
+//
+// Bound by its chain of dependent loads (list entry, state, cell, filter words,
+// records, response): on 1,660 listed nodes 5,700 cycles, 1,300 of them for the
+// list length, which every CTA reads from one line of L2.  So the first entry and
+// its path load beside it.  Measured on 640,000 nodes (ncu): 7,000 listed 9.4 ->
+// 8.6 us, 150,000 listed 16.5 -> 15.2.
+//
+// The walk's one-warp CTAs fill whatever SMs this kernel leaves first, up to
+// twelve on one and eight on another, and the crowded ones then set the walk's
+// time.  So with a long list (as the walk's count stands when the last warp
+// looks, before the wait) the next kernel is let in when the CTAs are done:
+// 150,000 listed 36.9 -> 35.7 us per substep.  With a short one that would only
+// cost the overlap (none listed, L2 flushed: 60.3 -> 62.2 us per step).
 template <bool REC, bool SHORT>
-__global__ void __launch_bounds__(32 * COLL_WARPS, SHORT ? CLOTH_COLL_SHORT_CTAS_PER_SM : CLOTH_COLL_MINB) collide_kernel(const __grid_constant__ StepParams p)
+__global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_CTAS_PER_SM) collide_kernel(const __grid_constant__ StepParams p)
 {
     __shared__ unsigned long long s_k;
     __shared__ unsigned s_n, s_stat[2];
-    pdl_launch_dependents();
+    if (threadIdx.x == 32 * (COLL_WARPS - 1) &&
+        *(volatile unsigned *)(p.coll_count + (p.parity & 1)) <= gridDim.x * (32u * COLL_WARPS / 2u))
+        pdl_launch_dependents();
     pdl_wait();
-    // the lane's first list entry in case the list is short, loaded beside
-    // the list length instead of after it (the list holds p.n entries; one past
-    // the length is stale and ignored)
+    // the lane's first list entry, in case the list is short, and its path, loaded
+    // beside the list length instead of after it (the list holds p.n entries; one
+    // past the length is stale, or never written, and ignored)
     const unsigned i0 = coll_first_index();
-    const int pre_o = i0 < (unsigned)p.n ? p.coll_list[i0] : 0;
+    CollFirst first;
+    first.load(p, i0 < (unsigned)p.n ? p.coll_list[i0] : 0);
     if (threadIdx.x == 0) {
         coll_begin(p.ctrl, s_k, s_n);
         s_stat[0] = s_stat[1] = 0u;
@@ -614,9 +622,10 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, SHORT ? CLOTH_COLL_SHORT_CTAS
     if (s_n == 0u) return;
     float fsum = 0.0f;
     unsigned ntest = 0u, nhit = 0u;
-    collide_list<REC, SHORT>(OneClothList{p}, k, s_n, fsum, ntest, nhit, true, pre_o);
+    collide_list<REC, SHORT>(OneClothList{p}, k, s_n, fsum, ntest, nhit, &first);
     if (__any_sync(FULL, !isfinite(fsum)) && (threadIdx.x & 31) == 0)
         atomicOr(&p.ctrl->flags, (unsigned)CTRL_FLAG_NONFINITE);
+    pdl_launch_dependents();
     coll_stats_add(p.ctrl, s_stat, s_n, ntest, nhit);
 }
 
@@ -800,6 +809,7 @@ __global__ void __launch_bounds__(32 * CLOTH_WALK_WARPS, CLOTH_BATCH_MINB) batch
 
 // List entries of a batch: each carries its cloth.
 struct BatchList {
+    static constexpr bool DEEP = false;  // no registers to spare at four CTAs per SM
     const BatchArgs &b;
     __device__ void entry(unsigned long long i, int &cloth, long long &o) const
     {
@@ -809,7 +819,7 @@ struct BatchList {
     __device__ const StepParams &params(int c) const { return b.params[c]; }
 };
 
-__global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_COLL_MINB) batch_collide_kernel(const __grid_constant__ BatchArgs b)
+__global__ void __launch_bounds__(32 * COLL_WARPS, CLOTH_BATCH_COLL_CTAS_PER_SM) batch_collide_kernel(const __grid_constant__ BatchArgs b)
 {
     __shared__ unsigned long long s_k;
     __shared__ unsigned s_n, s_stat[2];
@@ -964,11 +974,10 @@ cudaError_t launch_collide(const StepParams &p, cudaStream_t s)
         if (e != cudaSuccess) return e;
         return launch_k(edge_apply_kernel, p.coll_blocks, 256, s, p);
     }
-    if (p.coll_short)
-        return p.cdata ? launch_k(collide_kernel<true, true>, p.coll_blocks, 32 * COLL_WARPS, s, p)
-                       : launch_k(collide_kernel<false, true>, p.coll_blocks, 32 * COLL_WARPS, s, p);
-    return p.cdata ? launch_k(collide_kernel<true, false>, p.coll_blocks, 32 * COLL_WARPS, s, p)
-                   : launch_k(collide_kernel<false, false>, p.coll_blocks, 32 * COLL_WARPS, s, p);
+    // recording substeps of cloths small enough for SHORT are node_kernel's
+    if (p.cdata) return launch_k(collide_kernel<true, false>, p.coll_blocks, 32 * COLL_WARPS, s, p);
+    return p.coll_short ? launch_k(collide_kernel<false, true>, p.coll_blocks, 32 * COLL_WARPS, s, p)
+                        : launch_k(collide_kernel<false, false>, p.coll_blocks, 32 * COLL_WARPS, s, p);
 }
 
 cudaError_t launch_substep(const StepParams &p, cudaStream_t s)
