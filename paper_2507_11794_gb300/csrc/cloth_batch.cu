@@ -104,10 +104,28 @@ cudaError_t rebuild(ClothBatch *b)
             }
     }
     std::stable_sort(items.begin(), items.end(), [](const int4 &a, const int4 &c) { return a.w > c.w; });
+    // one walk variant for the whole batch when every cloth has the same one
+    int var = -1;
+    for (const StepParams &q : prm) {
+        const int v = (q.has_mesh ? BATCH_VAR_MESH : 0) | (q.ks_slot ? BATCH_VAR_PER_SPRING : 0);
+        var = var < 0 || var == v ? v : BATCH_VAR_MIXED;
+    }
+    if (var < 0) var = BATCH_VAR_MIXED;
+    // small cloths: a list of 64-position groups for the one-kernel substep
+    std::vector<int2> groups;
+    long long ng = 0;
+    for (const StepParams &q : prm) ng += ((long long)q.ny * q.pitch + 63) / 64;
+    if (node_batch_fits(ng, var, b->sm_count))
+        for (size_t i = 0; i < prm.size(); i++)
+            for (long long j = 0; 64 * j < (long long)prm[i].ny * prm[i].pitch; j++)
+                groups.push_back(make_int2((int)i, (int)j));
+    // no exception from here on: the arguments and the device lists change together
     cudaFree(b->d_params);
     cudaFree(b->d_items);
+    cudaFree(b->d_groups);
     b->d_params = nullptr;
     b->d_items = nullptr;
+    b->d_groups = nullptr;
     cudaError_t e = cudaMalloc(&b->d_params, sizeof(StepParams) * prm.size());
     if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(int4) * std::max<size_t>(items.size(), 1));
     if (e == cudaSuccess)
@@ -127,23 +145,7 @@ cudaError_t rebuild(ClothBatch *b)
     b->args.coll_count = b->ctrl->coll_count;
     b->args.walk_blocks = b->sm_count * b->ctas_per_sm;
     b->args.coll_blocks = b->sm_count * CLOTH_BATCH_COLL_CTAS_PER_SM;
-    // one walk variant for the whole batch when every cloth has the same one
-    int var = -1;
-    for (const StepParams &q : prm) {
-        const int v = (q.has_mesh ? BATCH_VAR_MESH : 0) | (q.ks_slot ? BATCH_VAR_PER_SPRING : 0);
-        var = var < 0 || var == v ? v : BATCH_VAR_MIXED;
-    }
-    b->args.variant = var < 0 ? BATCH_VAR_MIXED : var;
-    // small cloths: a list of 64-position groups for the one-kernel substep
-    cudaFree(b->d_groups);
-    b->d_groups = nullptr;
-    std::vector<int2> groups;
-    long long ng = 0;
-    for (const StepParams &q : prm) ng += ((long long)q.ny * q.pitch + 63) / 64;
-    if (node_batch_fits(ng, b->args.variant, b->sm_count))
-        for (size_t i = 0; i < prm.size(); i++)
-            for (long long j = 0; 64 * j < (long long)prm[i].ny * prm[i].pitch; j++)
-                groups.push_back(make_int2((int)i, (int)j));
+    b->args.variant = var;
     if (e == cudaSuccess && !groups.empty()) {
         e = cudaMalloc(&b->d_groups, sizeof(int2) * groups.size());
         if (e == cudaSuccess)
@@ -305,6 +307,7 @@ int cloth_batch_set_mesh(ClothBatch *b, int32_t index, const float *verts, int32
     try {
         BTRY(b, rebuild(b), "batch rebuild");
     } catch (...) {
+        b->dead = true;  // the cloth's parameters on the device still name its old model
         return bfail(CLOTH_ERR_OOM, "host allocation failed");
     }
     return CLOTH_OK;
