@@ -284,9 +284,12 @@ int cloth_batch_set_state(ClothBatch *b, int32_t index, const float *pos, const 
 /* Autotuner: times trial_substeps substeps of the batch for every candidate
  * (rows_per_warp in {4,6,8,12,16,24,32} x walk CTAs per SM), keeps the
  * fastest, and restores every cloth's state and the substep counter, so the
- * simulation is unchanged.  Synchronises. */
+ * simulation is unchanged.  Both settings are the persistent walk's: a batch of
+ * small cloths, stepped by one launch, keeps the ones it has and is timed once
+ * (candidates = 1).  Synchronises. */
 int cloth_batch_tune(ClothBatch *b, int32_t trial_substeps, ClothBatchTuning *out);
-/* Set the tuning explicitly (rows_per_warp 1..32, walk_ctas_per_sm 1..32). */
+/* Set the tuning explicitly (rows_per_warp 1..32, walk_ctas_per_sm 1..32); a
+ * batch stepped by one launch takes it up when its cloths need the walk. */
 int cloth_batch_set_tuning(ClothBatch *b, int32_t rows_per_warp, int32_t walk_ctas_per_sm);
 int cloth_batch_get_tuning(ClothBatch *b, ClothBatchTuning *out);
 /* Wait for the batch's stream and report device-side error flags. */

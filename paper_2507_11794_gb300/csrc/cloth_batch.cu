@@ -389,33 +389,40 @@ int cloth_batch_tune(ClothBatch *b, int32_t trial_substeps, ClothBatchTuning *ou
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     const int Rs[] = {4, 6, 8, 12, 16, 24, 32};
     long long k = b->substeps_done;
-    for (int c = 1; c <= batch_min_ctas() && e == cudaSuccess; c++)
-        for (int R : Rs) {
-            if (e != cudaSuccess) break;
-            b->rows_per_warp = R;
-            b->ctas_per_sm = c;
-            try {
-                e = rebuild(b);
-            } catch (...) {
-                e = cudaErrorMemoryAllocation;
-            }
-            if (e == cudaSuccess) e = launch_parity(b, k++, b->stream);  // warm-up
-            if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-            for (int s = 0; s < trial_substeps && e == cudaSuccess; s++) e = launch_parity(b, k++, b->stream);
-            if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
-            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-            float ms = 0.0f;
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-            if (e == cudaSuccess) {
-                tried++;
-                const float us = 1e3f * ms / (float)trial_substeps;
-                if (us < best_us) {
-                    best_us = us;
-                    best_R = R;
-                    best_c = c;
-                }
-            }
+    // one trial of the current settings
+    auto trial = [&]() {
+        e = launch_parity(b, k++, b->stream);  // warm-up
+        if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
+        for (int s = 0; s < trial_substeps && e == cudaSuccess; s++) e = launch_parity(b, k++, b->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        if (e != cudaSuccess) return;
+        tried++;
+        const float us = 1e3f * ms / (float)trial_substeps;
+        if (us < best_us) {
+            best_us = us;
+            best_R = b->rows_per_warp;
+            best_c = b->ctas_per_sm;
         }
+    };
+    // the one-kernel substep has no strips: the settings would all time the same
+    if (b->d_groups) {
+        if (e == cudaSuccess) trial();
+    } else
+        for (int c = 1; c <= batch_min_ctas() && e == cudaSuccess; c++)
+            for (int R : Rs) {
+                if (e != cudaSuccess) break;
+                b->rows_per_warp = R;
+                b->ctas_per_sm = c;
+                try {
+                    e = rebuild(b);
+                } catch (...) {
+                    e = cudaErrorMemoryAllocation;
+                }
+                if (e == cudaSuccess) trial();
+            }
     // restore the states and the counter, then apply the winner
     for (size_t i = 0; i < b->cl.size(); i++) {
         ClothHandle *h = b->cl[i];
