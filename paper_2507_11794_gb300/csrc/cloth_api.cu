@@ -465,12 +465,14 @@ int cloth_set_mesh(ClothHandle *h, const float *verts, int32_t nverts, const int
         return fail(CLOTH_ERR_BAD_MESH, "triangle index %d at %lld out of range [0, %d)", tris[i], i, nverts);
     };
     auto bad_vertex = [&](long long i) { return fail(CLOTH_ERR_BAD_MESH, "non-finite vertex coordinate at %lld", i); };
-    if (!scan) {
+    auto look_over = [&]() {
         for (long long i = 0; i < 3 * (long long)ntris; i++)
             if (tris[i] < 0 || tris[i] >= nverts) return bad_index(i);
         for (long long i = 0; i < 3 * (long long)nverts && ntris > 0; i++)
             if (!isfinite(verts[i])) return bad_vertex(i);
-    }
+        return (int)CLOTH_OK;
+    };
+    if (!scan && (rc = look_over()) != CLOTH_OK) return rc;
     DeviceScope ds(h->device);
     CTRY(h, cudaStreamSynchronize(h->stream), "synchronize");
     DevGrid g{};
@@ -516,6 +518,8 @@ int cloth_set_mesh(ClothHandle *h, const float *verts, int32_t nverts, const int
         }
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();
+            // a bad mesh is one also where there is no memory to look at it on the device
+            if (scan && (rc = look_over()) != CLOTH_OK) return rc;
             return fail(CLOTH_ERR_OOM, "device allocation failed while building the grid");
         }
         if (e != cudaSuccess) return cuda_fail(h, e, "grid build");
