@@ -185,8 +185,10 @@ int cloth_sync(ClothHandle *h);
  * (not part of the paper, which gives no counts; they describe the work of
  * the grid broad phase and narrow phase of Section 3): listed = nodes whose
  * substep path box reached the surface model's (padded) bounding box,
- * tested = candidate triangles put through the extended Moller-Trumbore
- * test, hits = nodes that received a response.  With the edge narrow phase
+ * tested = candidate triangles, i.e. entries of the grid cells that a path's
+ * box meets (paths over more than 8 cells excepted; a box filter then leaves a
+ * few per path for the extended Moller-Trumbore test), hits = nodes that received
+ * a response.  With the edge narrow phase
  * (CLOTH_FLAG_EDGE_COLLISION): listed = nodes whose 3 x 3 block box reached
  * that box, tested = candidate triangles of their owned edges, hits = edges
  * with at least one hit.  Zero without a surface model.  Synchronises.  Any

@@ -14,9 +14,9 @@
 //
 // Measured against the walk and the collision pass as two launches (graph
 // replay, us per substep; n x n nodes lying on 20,480 triangles): n = 16
-// 9.3 -> 6.2, 96 10.9 -> 7.2, 160 12.9 -> 8.6, 240 14.6 -> 12.7; without a mesh
-// n = 16 to 160 3.6 -> 3.1, 240 4.2 -> 3.6, 330 5.2 -> 4.7.  What is left is the
-// launch and one chain of loads per phase.
+// 9.3 -> 6.2, 96 10.9 -> 6.7, 160 12.9 -> 8.2, 240 14.6 -> 11.5; without a mesh
+// n = 16 3.7 -> 3.1, 64 to 160 4.1 -> 3.6, 240 4.6 -> 4.1, 330 5.7 -> 4.8.  What is
+// left is the launch and one chain of loads per phase.
 #include "cloth_collide.cuh"
 #include "cloth_force.cuh"
 #include "cloth_internal.h"
@@ -183,7 +183,9 @@ __device__ __forceinline__ Vec2 pair_force(const StepParams &p, const float *in,
 // CTAs per SM up to which a cloth gets W warps per CTA, so that all are
 // resident at once (registers); more lanes per node shorten its chain of loads.
 // Two warps of 128 registers (8 CTAs per SM) beat listing the nodes for the
-// collision pass on 256 x 256 and 272 x 272 nodes, 12.9 against 15.5 us; beyond
+// collision pass on 256 x 256 and 272 x 272 nodes lying on the model, 12.9 against
+// 15.5 us (11.8 now); in light contact, pulled over it, listing was ahead with 11.2
+// against 12.3, until the narrow phase had more loads in flight (10.3).  Beyond
 // that the nodes are listed, and from 12 CTAs per SM the walk takes over (its
 // rows then have the warps they need).
 #define CLOTH_NODE_W8 1

@@ -588,8 +588,8 @@ struct OneClothList {
 // Bound by its chain of dependent loads (list entry, state, cell, filter words,
 // records, response): on 1,660 listed nodes 5,700 cycles, 1,300 of them for the
 // list length, which every CTA reads from one line of L2.  So the first entry and
-// its path load beside it.  Measured on 640,000 nodes (ncu): 7,000 listed 9.4 ->
-// 8.6 us, 150,000 listed 16.5 -> 15.2.
+// its path load beside it.  Measured on 640,000 nodes (ncu): 1,660 listed 9.4 ->
+// 8.6 us (from a cold L2 10.8 -> 9.4), 150,000 listed 16.5 -> 15.2.
 //
 // The walk's one-warp CTAs fill whatever SMs this kernel leaves first, up to
 // twelve on one and eight on another, and the crowded ones then set the walk's
