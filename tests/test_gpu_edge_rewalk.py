@@ -1,7 +1,7 @@
 """An edge with more hits than the edge test stores points for is walked again by
 the node's gather, which has to find the same hits.  Beside five small triangles
 that the edge crosses lies a large tilted one: the edge is in its plane to within
-1e-7 m, but 4 to 16 mm outside its box and in the same grid cell.  The float32 test
+1e-7 m, but 6 to 22 mm outside its box and in the same grid cell.  The float32 test
 accepts it (its errors in u and v grow as 1 / a), the candidate filter does not,
 and in exact arithmetic it is missed.  Checked against the FP64 oracle."""
 import numpy as np
